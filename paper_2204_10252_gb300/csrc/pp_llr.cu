@@ -4,20 +4,28 @@
 // per coefficient image) is replaced by U max(S - lambda, 0) V^H, its
 // singular values soft-thresholded.
 //
-// One CTA per block.  The SVD is a one-sided Jacobi iteration in FP32:
-// columns i, j of M are rotated until every pair is orthogonal; the rotated
-// matrix is U S and the accumulated rotations are V, so the output is
-// (M V) diag(max(0, 1 - lambda / s_i)) V^H.  One-sided Jacobi works on M
-// itself, so small singular values keep their relative accuracy (no Gram
-// matrix whose rounding is relative to the largest one).  A sweep visits all
-// T(T-1)/2 pairs in T'-1 rounds of disjoint pairs (round-robin schedule,
-// T' = T rounded up to even); the column norms and inner products of one
-// round's pairs are summed over the block's voxels in one block reduction.
-// The sweeps stop when every pair's |a_i^H a_j| <= tol sqrt(|a_i|^2 |a_j|^2)
-// (the same decision in every thread: it is taken from the reduced sums),
-// tol = sqrt(R) * 2^-24 for R voxels per block: the rounding level of an
-// R-term FP32 inner product (the threshold LAPACK's one-sided Jacobi uses
-// with its own precision), below which a rotation only moves noise.
+// One CTA per block, the matrix in registers (RPT rows of T columns a thread).
+// The SVD goes through the T x T Gram matrix twice:
+//   H  = M^H M   (one block reduction), Jacobi eigenvectors V0, M1 = M V0;
+//   H1 = M1^H M1 (one block reduction), Jacobi eigenvectors V1, V = V0 V1;
+//   out = M1 Q,  Q = V1 diag(max(0, 1 - lambda / s_i)) V^H,  s_i^2 the
+//   eigenvalues of H1.
+// The rounding of H is relative to its largest eigenvalue, so V0 leaves the
+// columns of M1 orthogonal only to about 2^-24 s_1^2 / (s_i s_j).  H1 is formed
+// from those columns themselves: each of its entries is accurate relative to
+// |a_i| |a_j|, and Jacobi with a relative threshold keeps that accuracy, as
+// one-sided Jacobi on M does (its rotations leave the same 2^-24 s_1 in every
+// column).  Rows meet in two block reductions instead of one for each of the
+// T'-1 rounds of every sweep, and are rotated twice instead of in every round:
+// five images of 128 x 256 x 256 with 8^3 blocks (0.67 GB in and out) took
+// 877 us with one-sided Jacobi over the rows (issue bound: 60 % of issue slots)
+// and take 373 us (1800 GB/s).
+//
+// The T x T eigenproblems run in one warp, a lane per matrix element: the
+// rounds of disjoint pairs (round-robin schedule, T' = T rounded up to even)
+// are exact in either order, so a round updates A <- J^H A J and V <- V J out
+// of one shared buffer into another with one warp barrier.  Their serial chain
+// (about 25 rounds) is hidden by the other CTAs of the SM.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -41,61 +49,138 @@ struct LlrArgs {
     float lam;
 };
 
-// Round-robin (circle method) schedule of T' players: in round r the pairs
-// are (r, T'-1) and ((r + k) mod (T'-1), (r - k) mod (T'-1)), k = 1 .. T'/2-1.
+// Partner of index i in round r of the round-robin schedule (circle method) of
+// TP players: r and TP - 1 meet, the others pair to a sum of 2r mod (TP - 1).
 template <int TP>
-__host__ __device__ constexpr int rr_i(int r, int k) {
-    return k == 0 ? r : ((r + k) % (TP - 1) < (r - k + (TP - 1)) % (TP - 1) ? (r + k) % (TP - 1)
-                                                                              : (r - k + (TP - 1)) % (TP - 1));
-}
-template <int TP>
-__host__ __device__ constexpr int rr_j(int r, int k) {
-    return k == 0 ? TP - 1 : ((r + k) % (TP - 1) < (r - k + (TP - 1)) % (TP - 1) ? (r - k + (TP - 1)) % (TP - 1)
-                                                                                  : (r + k) % (TP - 1));
+__device__ __forceinline__ int rr_partner(int r, int i) {
+    if (i == TP - 1) return r;
+    if (i == r) return TP - 1;
+    int j = 2 * r - i;
+    j += j < 0 ? TP - 1 : 0;
+    return j >= TP - 1 ? j - (TP - 1) : j;
 }
 
-// Sum N <= 16 floats per thread over the block (NT threads, NT/32 warps):
-// the result in every thread.  Within a warp a butterfly reduce-scatter
-// halves the values each step (16 shuffles for 16 values instead of 5 per
-// value): after the step with offset o a lane keeps the half its bit o
-// selects, so lanes 2i and 2i+1 end with the warp sum of value i.  One lane
-// per value writes it to `buf` ([NT/32][16] floats), and after the barrier
-// every thread adds the warps' rows with 16-byte reads.
-template <int NT, int N>
-__device__ __forceinline__ void block_sum(float* v, float* buf) {
-    static_assert(N <= 16, "block_sum handles up to 16 values");
-    float t[16];
+// The T^2 floats of the Gram matrix of the block's rows, as a T x T array:
+// |a_i|^2 at (i, i), Re a_i^H a_j at (i, j) and Im a_i^H a_j at (j, i), i < j.
+// Within a warp a butterfly reduce-scatter halves the values each step (31
+// shuffles for 32 values instead of 5 for each), which leaves value l of a
+// chunk with lane l; one row a warp in `buf`.
+template <int T, int RPT, int NT>
+__device__ __forceinline__ void gram_partials(const float2 (&m)[RPT][T], float (*buf)[64]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) t[i] = i < N ? v[i] : 0.f;
+    for (int base = 0; base < T * T; base += 32) {
+        float t[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            const int i = (base + e) / T, j = (base + e) % T;
+            float acc = 0.f;
+            if (base + e < T * T && i <= j) {
+                float2 p = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < RPT; ++q) p = __ffma2_rn(m[q][i], m[q][j], p);
+                acc = p.x + p.y;
+            } else if (base + e < T * T) {
+#pragma unroll
+                for (int q = 0; q < RPT; ++q)
+                    acc = fmaf(m[q][j].x, m[q][i].y, fmaf(-m[q][j].y, m[q][i].x, acc));
+            }
+            t[e] = acc;
+        }
+#pragma unroll
+        for (int h = 16; h >= 1; h >>= 1) {
+            const bool up = (lane & h) != 0;
+#pragma unroll
+            for (int i = 0; i < h; ++i) {
+                const float send = up ? t[i] : t[i + h];
+                const float keep = up ? t[i + h] : t[i];
+                t[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+            }
+        }
+        buf[w][base + lane] = t[0];
+    }
+}
+
+__device__ __forceinline__ float2 shfl2(float2 v, int src) {
+    return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+// Column k's share of the rotation that makes columns k and k2 of the Hermitian
+// A orthogonal: new column k = alpha * column k + beta * column k2.  Returns
+// |a_k^H a_k2| / (|a_k| |a_k2|), 0 where it is at most tol.
+template <int T>
+__device__ __forceinline__ float jacobi_pair(const float2 (*A)[T], int k, int k2, float tol,
+                                             float2* alpha, float2* beta) {
+    *alpha = make_float2(1.f, 0.f);
+    *beta = make_float2(0.f, 0.f);
+    if (k2 >= T) return 0.f;
+    const int i = min(k, k2), j = max(k, k2);
+    const float al = A[i][i].x, be = A[j][j].x;
+    const float2 gm = A[i][j];
+    const float g2 = gm.x * gm.x + gm.y * gm.y, lim = tol * tol * al * be;
+    if (!(g2 > fmaxf(lim, 1e-38f))) return 0.f;
+    // real symmetric Schur rotation of [[al, g], [g, be]] after the phase
+    // conj(gamma)/|gamma| on column j that makes gamma real; any t serves, c and
+    // sn follow from it
+    const float rg = rsqrtf(g2), g = g2 * rg;
+    const float zeta = 0.5f * (be - al) * rg;
+    const float z1 = fminf(fmaf(zeta, zeta, 1.f), 1e30f);
+    const float t = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + z1 * rsqrtf(z1));
+    const float c = rsqrtf(fmaf(t, t, 1.f)), sn = c * t;
+    const float2 ph = make_float2(gm.x * rg, -gm.y * rg);
+    const bool up = k == i;
+    *alpha = make_float2(up ? c : c * ph.x, up ? 0.f : c * ph.y);
+    *beta = make_float2(up ? -sn * ph.x : sn, up ? -sn * ph.y : 0.f);
+    // al * be <= 0 only through rounding: count it as not yet orthogonal
+    return lim > 0.f ? g * rsqrtf(al * be) : 1.f;
+}
+
+// Eigenvectors of the Hermitian T x T matrix A[0] by Jacobi rotations in one
+// warp; sweeps until every |a_ij| <= tol sqrt(a_ii a_jj) before its rotation,
+// or `last` at the start of the sweep.  Returns the buffer (0 or 1) that holds
+// the result; V[that] holds the eigenvectors in its columns.
+template <int T>
+__device__ __forceinline__ int warp_jacobi(float2 (*A)[T][T], float2 (*V)[T][T], float tol,
+                                           float last) {
+    constexpr int TP = T + (T & 1), NE = (T * T + 31) / 32;
     const int lane = threadIdx.x & 31;
+    int cur = 0;
 #pragma unroll
-    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const float send = up ? t[i] : t[i + h];
-            const float keep = up ? t[i + h] : t[i];
-            t[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
+    for (int q = 0; q < NE; ++q) {
+        const int e = lane + 32 * q;
+        if (e < T * T) V[0][e / T][e % T] = make_float2(e / T == e % T ? 1.f : 0.f, 0.f);
     }
-    t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
-    const int w = threadIdx.x >> 5;
-    if ((lane & 1) == 0) buf[w * 16 + (lane >> 1)] = t[0];
-    __syncthreads();
-    const float4* b4 = reinterpret_cast<const float4*>(buf);
+    __syncwarp();
+    const int kc = min(lane, T - 1);
+    for (int sweep = 0; T > 1 && sweep < kLlrSweeps; ++sweep) {
+        float off = 0.f;
+#pragma unroll 1
+        for (int r = 0; r < TP - 1; ++r) {
+            const float2(*Ac)[T] = A[cur];
+            const float2(*Vc)[T] = V[cur];
+            // lane k < T works out column k's rotation, the others ask for it
+            float2 al, be;
+            off = fmaxf(off, jacobi_pair<T>(Ac, kc, rr_partner<TP>(r, kc), tol, &al, &be));
 #pragma unroll
-    for (int q = 0; q < (N + 3) / 4; ++q) {
-        float4 acc = b4[q];
-#pragma unroll
-        for (int ww = 1; ww < NT / 32; ++ww) {
-            const float4 u = b4[ww * 4 + q];
-            acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+            for (int q = 0; q < NE; ++q) {
+                const int e = lane + 32 * q, i = min(e / T, T - 1), k = e % T;
+                const float2 ai = shfl2(al, i), bi = shfl2(be, i), ak = shfl2(al, k), bk = shfl2(be, k);
+                if (e < T * T) {
+                    const int i2 = rr_partner<TP>(r, i), k2 = rr_partner<TP>(r, k);
+                    const int i3 = i2 < T ? i2 : i, k3 = k2 < T ? k2 : k;   // idle: beta = 0
+                    const float2 s0 = cadd(cmul(Ac[i][k], ak), cmul(Ac[i][k3], bk));
+                    const float2 s1 = cadd(cmul(Ac[i3][k], ak), cmul(Ac[i3][k3], bk));
+                    A[cur ^ 1][i][k] = cadd(cmulc(ai, s0), cmulc(bi, s1));
+                    V[cur ^ 1][i][k] = cadd(cmul(Vc[i][k], ak), cmul(Vc[i][k3], bk));
+                }
+            }
+            cur ^= 1;
+            __syncwarp();
         }
-        if (4 * q + 0 < N) v[4 * q + 0] = acc.x;
-        if (4 * q + 1 < N) v[4 * q + 1] = acc.y;
-        if (4 * q + 2 < N) v[4 * q + 2] = acc.z;
-        if (4 * q + 3 < N) v[4 * q + 3] = acc.w;
+        off = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(off)));
+        if (off <= last) break;
     }
+    return cur;
 }
 
 // Offset of voxel `row` of block `b` in one coefficient image.
@@ -112,125 +197,161 @@ __device__ __forceinline__ int64_t llr_voxel(const LlrArgs& a, int b, int row) {
     return ((int64_t)z * a.ny + y) * a.nx + x;
 }
 
+// At most 80 registers a thread: 6 CTAs of 128 threads an SM.  One-warp CTAs are
+// left uncapped: capped at 80, their seven- and eight-image forms spill and
+// gave wrong results (the tests hold every compiled form to the oracle).
+__host__ __device__ constexpr int llr_min_ctas(int nt) { return nt > 32 ? 65536 / (nt * 80) : 0; }
+
 template <int T, int RPT, int NT>
-__global__ void __launch_bounds__(NT) llr_prox_kernel(LlrArgs a) {
-    constexpr int TP = T + (T & 1);
-    constexpr int NPR = TP / 2;                       // pairs per round
-    __shared__ float2 Vs[T][T];                       // Vs[k][i] = V(k, i)
-    __shared__ __align__(16) float red[2][NT / 32][16];
+__global__ void __launch_bounds__(NT, llr_min_ctas(NT)) llr_prox_kernel(LlrArgs a) {
+    __shared__ float part[NT / 32][64];
+    __shared__ float2 A[2][T][T], V0[2][T][T], V1[2][T][T];
+    __shared__ float4 W[T][T];   // (x, x, -y, y) of the T x T factor applied to the rows
+    __shared__ float trace;
     const int b = blockIdx.x;
+    const int lane = threadIdx.x & 31;
     float2 m[RPT][T];
-    int64_t off[RPT];
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
         const int row = threadIdx.x + q * NT;
         const bool live = row < a.R;
-        off[q] = live ? llr_voxel(a, b, row) : -1;
+        const int64_t off = live ? llr_voxel(a, b, row) : 0;
 #pragma unroll
         for (int t = 0; t < T; ++t)
-            m[q][t] = live ? a.in[t * a.nimg + off[q]] : make_float2(0.f, 0.f);
+            m[q][t] = live ? a.in[t * a.nimg + off] : make_float2(0.f, 0.f);
     }
-    if (threadIdx.x < T)
-#pragma unroll
-        for (int i = 0; i < T; ++i) Vs[threadIdx.x][i] = make_float2(i == (int)threadIdx.x ? 1.f : 0.f, 0.f);
     const float tol = sqrtf((float)a.R) * 5.9604645e-8f;
-    int par = 0;
-    if (T > 1) {
-        for (int sweep = 0; sweep < kLlrSweeps; ++sweep) {
-            float offmax = 0.f;
+    int c0 = 0;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        gram_partials<T, RPT, NT>(m, part);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            // sum the warps' rows; scale by 1 / trace (pass 0's) against over- and underflow
+            float g[(T * T + 31) / 32];
+            float tr = 0.f;
 #pragma unroll
-            for (int r = 0; r < TP - 1; ++r) {
-                float s[4 * NPR];
+            for (int q = 0; q < (T * T + 31) / 32; ++q) {
+                const int e = lane + 32 * q;
+                float acc = 0.f;
+                if (e < T * T)
 #pragma unroll
-                for (int p = 0; p < NPR; ++p) {
-                    const int i = rr_i<TP>(r, p), j = rr_j<TP>(r, p);
-                    float al = 0.f, be = 0.f, gr = 0.f, gi = 0.f;
-                    if (j < T) {
+                    for (int w = 0; w < NT / 32; ++w) acc += part[w][e];
+                g[q] = acc;
+                if (e < T * T && e / T == e % T) tr += acc;
+            }
+            if (pass == 0) {
 #pragma unroll
-                        for (int q = 0; q < RPT; ++q) {
-                            const float2 u = m[q][i], v = m[q][j];
-                            al = fmaf(u.x, u.x, fmaf(u.y, u.y, al));
-                            be = fmaf(v.x, v.x, fmaf(v.y, v.y, be));
-                            gr = fmaf(u.x, v.x, fmaf(u.y, v.y, gr));   // Re conj(u) v
-                            gi = fmaf(u.x, v.y, fmaf(-u.y, v.x, gi));  // Im conj(u) v
-                        }
-                    }
-                    s[4 * p] = al; s[4 * p + 1] = be; s[4 * p + 2] = gr; s[4 * p + 3] = gi;
-                }
-                block_sum<NT, 4 * NPR>(s, &red[par][0][0]);
-                par ^= 1;   // the next reduction writes the other buffer: no second barrier
+                for (int o = 16; o; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+                if (lane == 0) trace = tr;
+                __syncwarp();
+            }
+            tr = trace;
+            const float sc = tr > 0.f ? 1.f / tr : (tr == 0.f ? 0.f : tr);
 #pragma unroll
-                for (int p = 0; p < NPR; ++p) {
-                    const int i = rr_i<TP>(r, p), j = rr_j<TP>(r, p);
-                    if (j >= T) continue;
-                    const float al = s[4 * p], be = s[4 * p + 1], gr = s[4 * p + 2], gi = s[4 * p + 3];
-                    const float g = sqrtf(gr * gr + gi * gi), nab = sqrtf(al * be);
-                    if (!(g > tol * nab)) continue;
-                    offmax = fmaxf(offmax, g / nab);
-                    // real symmetric Schur rotation of [[al, g], [g, be]], after the
-                    // phase e^{-i phi} = conj(gamma)/|gamma| that makes gamma real
-                    const float zeta = (be - al) / (2.f * g);
-                    const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
-                    const float c = rsqrtf(fmaf(t, t, 1.f)), sn = c * t;
-                    const float2 ph = make_float2(gr / g, -gi / g);
-#pragma unroll
-                    for (int q = 0; q < RPT; ++q) {
-                        const float2 u = m[q][i], w = cmul(ph, m[q][j]);
-                        m[q][i] = make_float2(c * u.x - sn * w.x, c * u.y - sn * w.y);
-                        m[q][j] = make_float2(sn * u.x + c * w.x, sn * u.y + c * w.y);
-                    }
-                    if (threadIdx.x < T) {
-                        const int k = threadIdx.x;
-                        const float2 u = Vs[k][i], w = cmul(ph, Vs[k][j]);
-                        Vs[k][i] = make_float2(c * u.x - sn * w.x, c * u.y - sn * w.y);
-                        Vs[k][j] = make_float2(sn * u.x + c * w.x, sn * u.y + c * w.y);
+            for (int q = 0; q < (T * T + 31) / 32; ++q) {
+                const int e = lane + 32 * q, i = e / T, k = e - i * T;
+                if (e < T * T) {
+                    const float v = g[q] * sc;
+                    if (i == k) {
+                        A[0][i][i] = make_float2(v, 0.f);
+                    } else if (i < k) {
+                        A[0][i][k].x = v;
+                        A[0][k][i].x = v;
+                    } else {
+                        A[0][k][i].y = v;
+                        A[0][i][k].y = -v;
                     }
                 }
             }
-            if (offmax <= tol) break;
+            __syncwarp();
+            if (pass == 0) {
+                // near-orthogonal columns are enough here: stop after the sweep
+                // that met nothing above 0.03 (its rotations leave the square)
+                c0 = warp_jacobi<T>(A, V0, tol, 3e-2f);
+#pragma unroll
+                for (int q = 0; q < (T * T + 31) / 32; ++q) {
+                    const int e = lane + 32 * q;
+                    if (e < T * T) {
+                        const float2 v = (&V0[c0][0][0])[e];
+                        (&W[0][0])[e] = make_float4(v.x, v.x, -v.y, v.y);
+                    }
+                }
+            } else {
+                const int c1 = warp_jacobi<T>(A, V1, tol, 1e-3f);
+                // W = V1 F V^H with V = V0 V1; V goes to the buffer of A not in use
+#pragma unroll
+                for (int q = 0; q < (T * T + 31) / 32; ++q) {
+                    const int e = lane + 32 * q, i = e / T, k = e - i * T;
+                    if (e < T * T) {
+                        float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int l = 0; l < T; ++l) s = cadd(s, cmul(V0[c0][i][l], V1[c1][l][k]));
+                        A[c1 ^ 1][i][k] = s;
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < (T * T + 31) / 32; ++q) {
+                    const int e = lane + 32 * q, i = e / T, k = e - i * T;
+                    if (e < T * T) {
+                        float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int l = 0; l < T; ++l) {
+                            // s <= lambda (also s = 0) -> 0; a NaN fails the test and stays NaN
+                            const float d = A[c1][l][l].x * tr;
+                            const float sg = d < 0.f ? 0.f : sqrtf(d);
+                            const float f = sg <= a.lam ? 0.f : 1.f - a.lam / sg;
+                            const float2 v = A[c1 ^ 1][k][l];
+                            s = cadd(s, cscale(cmulc(v, V1[c1][i][l]), f));
+                        }
+                        W[i][k] = make_float4(s.x, s.x, -s.y, s.y);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            float2 y[T];
+#pragma unroll
+            for (int k = 0; k < T; ++k) y[k] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < T; ++i) {
+                const float2 u = m[q][i], us = make_float2(u.y, u.x);
+#pragma unroll
+                for (int k = 0; k < T; ++k) {
+                    const float4 w = W[i][k];
+                    y[k] = __ffma2_rn(u, make_float2(w.x, w.y), y[k]);
+                    y[k] = __ffma2_rn(us, make_float2(w.z, w.w), y[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < T; ++k) m[q][k] = y[k];
         }
     }
-    // singular values = final column norms; shrink factors
-    float nr[T];
-#pragma unroll
-    for (int i = 0; i < T; ++i) {
-        float acc = 0.f;
-#pragma unroll
-        for (int q = 0; q < RPT; ++q) acc = fmaf(m[q][i].x, m[q][i].x, fmaf(m[q][i].y, m[q][i].y, acc));
-        nr[i] = acc;
-    }
-    block_sum<NT, T>(nr, &red[par][0][0]);
-    float f[T];
-#pragma unroll
-    for (int i = 0; i < T; ++i) {
-        const float sg = sqrtf(nr[i]);
-        // s <= lambda (also s = 0) -> 0; a NaN fails the test and stays NaN
-        f[i] = sg <= a.lam ? 0.f : 1.f - a.lam / sg;
-    }
-    // every thread's Vs updates are visible after block_sum's barrier
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        if (off[q] < 0) continue;
+        const int row = threadIdx.x + q * NT;
+        if (row >= a.R) continue;
+        const int64_t off = llr_voxel(a, b, row);
 #pragma unroll
-        for (int k = 0; k < T; ++k) {
-            float2 y = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int i = 0; i < T; ++i) y = cadd(y, cscale(cmulc(Vs[k][i], m[q][i]), f[i]));
-            a.out[k * a.nimg + off[q]] = y;
-        }
+        for (int k = 0; k < T; ++k) a.out[k * a.nimg + off] = m[q][k];
     }
 }
 
 template <int T>
 cudaError_t llr_launch_t(const LlrArgs& a, int nblocks, cudaStream_t st) {
+    // R = 512, 256, 64 or 16 rows: few warps a block, so that few wait for the
+    // one that solves the eigenproblems; up to 20 matrix elements a thread
     if (a.R > 256) {
-        llr_prox_kernel<T, 4, 128><<<nblocks, 128, 0, st>>>(a);
-    } else if (a.R > 128) {
-        llr_prox_kernel<T, 2, 128><<<nblocks, 128, 0, st>>>(a);
+        if constexpr (T <= 5) llr_prox_kernel<T, 4, 128><<<nblocks, 128, 0, st>>>(a);
+        else llr_prox_kernel<T, 2, 256><<<nblocks, 256, 0, st>>>(a);
     } else if (a.R > 64) {
-        llr_prox_kernel<T, 1, 128><<<nblocks, 128, 0, st>>>(a);
+        if constexpr (T <= 5) llr_prox_kernel<T, 4, 64><<<nblocks, 64, 0, st>>>(a);
+        else llr_prox_kernel<T, 2, 128><<<nblocks, 128, 0, st>>>(a);
     } else if (a.R > 32) {
-        llr_prox_kernel<T, 1, 64><<<nblocks, 64, 0, st>>>(a);
+        llr_prox_kernel<T, 2, 32><<<nblocks, 32, 0, st>>>(a);
     } else {
         llr_prox_kernel<T, 1, 32><<<nblocks, 32, 0, st>>>(a);
     }

@@ -114,3 +114,26 @@ def test_llr_prox_mrf_sized_volume(pp):
     got = host(out)
     ref = O.prox_llr(x.astype(np.complex128), lam, 8, (4, 4, 4))
     assert rel(got, ref) <= TOL_APPLY
+
+
+@pytest.mark.parametrize("T", range(1, 9))
+@pytest.mark.parametrize("shape,block", [((8, 8, 8), 8), ((16, 16), 16), ((4, 4, 4), 4), ((4, 4), 4)],
+                         ids=["512rows", "256rows", "64rows", "16rows"])
+def test_llr_prox_graded_spectrum(pp, shape, block, T):
+    """Every compiled (images, rows) form on one block whose singular values
+    fall from 1 to 1e-3, the threshold between them: the Gram matrix of its
+    columns loses the small ones, the second Gram matrix must not.  The bound
+    is (sqrt(512) + T^2) 2^-24 < 6e-6 for the dot products and rotations."""
+    import torch
+    R = int(np.prod(shape))
+    rng = np.random.default_rng(100 * T + R)
+    U, _ = np.linalg.qr(rng.standard_normal((R, T)) + 1j * rng.standard_normal((R, T)))
+    V, _ = np.linalg.qr(rng.standard_normal((T, T)) + 1j * rng.standard_normal((T, T)))
+    s = np.logspace(0.0, -3.0, T) if T > 1 else np.ones(1)
+    x = ((U * s) @ V.conj().T).T.reshape((T,) + shape).astype(np.complex64)
+    lam = 0.9 * float(s[T // 2])
+    ref = O.prox_llr(x.astype(np.complex128), lam, block)
+    xin = dev(x)
+    out = torch.empty_like(xin)
+    pp.pp_prox_llr(shape, T, block, lam, xin, out)
+    assert rel(host(out), ref) <= 6e-6
