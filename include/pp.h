@@ -209,8 +209,9 @@ pp_status pp_adjoint_apply(const pp_plan* plan, const pp_c64* y, pp_c64* x, pp_s
  * its own pool (an allocation behind its back can fail or upset the host's
  * accounting), or a real-time loop that forbids allocation after start-up
  * (an allocation can stall or fail on fragmented memory).  The plan is built
- * beforehand with pp_plan_create.  Runs the same kernels as
- * pp_adjoint_apply.  The paper has no counterpart.
+ * beforehand with pp_plan_create.  Runs the [coil][row][col] kernels of
+ * pp_adjoint_apply (which may choose the coil-innermost ones: the results
+ * then agree to rounding).  The paper has no counterpart.
  *  - Plans whose adjoint needs more than 16 MiB of scratch (Cartesian 2-D:
  *    8*C*ny*nx bytes; 3-D: 16*nz*ny*nx; non-Cartesian: 8*C*G*(ny+G))
  *    return PP_ERR_UNSUPPORTED.

@@ -180,6 +180,11 @@ static RowArgs row_args(int n, int G, int off_in, int off_out, int nrows, int64_
     return a;
 }
 
+// Whether a non-Cartesian plan runs on the coil-innermost arrays: as the tuner
+// found faster for its normal operator (the forward and adjoint applies share
+// its FFT stages).
+static bool use_ci(const Plan& p) { return !p.toep && p.tune_stencil_kind >= 7 && p.ci_sens && p.ci_a; }
+
 // out = scale * (A^H A x) + alpha * operand   (operand may be NULL)
 static pp_status normal_into(const Plan& p, const float2* x, float2* out, float scale,
                              const float2* operand, float alpha, cudaStream_t st) {
@@ -213,7 +218,7 @@ static pp_status normal_into(const Plan& p, const float2* x, float2* out, float 
     }
     if (p.toep) return toep_normal(p, x, out, scale, operand, alpha, st);
     // non-Cartesian: rows -> cols -> G^T G stencil -> cols^H -> rows^H
-    if (p.tune_stencil_kind >= 7 && p.ci_sens)
+    if (use_ci(p))
         return ci_normal(p, x, out, scale, operand, alpha,
                          p.tune_stencil_kind == 9 ? 0 : (p.tune_stencil_kind == 8 ? 2 : 1), st);
     const int Gx = p.G_x, Gy = p.G_y;
@@ -255,19 +260,23 @@ static pp_status forward_into(const Plan& p, const float2* x, float2* y, cudaStr
         az.mul_out = p.mask_c; az.mo_q = ny; az.mo_c = 1; az.mo_cdiv = nx;
         return launch_cols(p.fz, az, y, y, false, st);
     }
+    if (use_ci(p)) {
+        PP_TRY(ci_to_grid(p, x, st));
+        return launch_nufft_degrid(p, p.ci_b, y, true, st);
+    }
     const int Gx = p.G_x, Gy = p.G_y;
     RowArgs rf = row_args(nx, Gx, nx / 2, 0, ny, (int64_t)ny * nx, 1.f);
     PP_TRY(launch_rows_fwd(p, p.gx, rf, x, p.sens, p.deapod_y, p.deapod_x, p.wk_a, p.C, 0, st));
     ColArgs cf = col_args(ny, Gy, Gy, ny / 2, 0, Gx, (int64_t)ny * Gx, (int64_t)Gy * Gx, p.C, 1.f);
     PP_TRY(launch_cols(p.gy, cf, p.wk_a, p.wk_b, false, st));
-    return launch_nufft_degrid(p, p.wk_b, y, st);
+    return launch_nufft_degrid(p, p.wk_b, y, false, st);
 }
 
 // x = A^H y (unscaled) with the intermediates in wa and wb (plan workspace, or the
 // library's fixed scratch array for pp_adjoint_apply_static): Cartesian 2-D
 // needs C*n elements in wa; 3-D n in wa and n in wb; non-Cartesian C*ny*G_x
-// in wa and C*G_y*G_x in wb.
-pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, float2* wb,
+// in wa and C*G_y*G_x in wb, and optionally the transposed k-space in kt.
+pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, float2* wb, float2* kt,
                      cudaStream_t st) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int64_t n = p.nimg;
@@ -298,7 +307,7 @@ pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, floa
         return PP_OK;
     }
     const int Gx = p.G_x, Gy = p.G_y;
-    PP_TRY(launch_nufft_spread(p, y, wb, st));
+    PP_TRY(launch_nufft_spread(p, y, kt, wb, false, st));
     ColArgs ci = col_args(Gy, ny, Gy, 0, ny / 2, Gx, (int64_t)Gy * Gx, (int64_t)ny * Gx, p.C, 1.f);
     PP_TRY(launch_cols(p.gy, ci, wb, wa, true, st));
     RowArgs ra = row_args(nx, Gx, 0, nx / 2, ny, (int64_t)ny * nx, 1.f);
@@ -307,7 +316,11 @@ pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, floa
 }
 
 static pp_status adjoint_into(const Plan& p, const float2* y, float2* x, cudaStream_t st) {
-    return adjoint_ws(p, y, x, p.wk_a, p.wk_b, st);
+    if (use_ci(p)) {
+        PP_TRY(launch_nufft_spread(p, y, p.ksp_t, p.ci_c, true, st));
+        return ci_from_grid(p, p.ci_c, x, 1.f, nullptr, 0.f, st);
+    }
+    return adjoint_ws(p, y, x, p.wk_a, p.wk_b, p.ksp_t, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -374,8 +387,8 @@ static pp_status build_noncartesian(Plan& p, const pp_sampling* s) {
         return PP_ERR_UNSUPPORTED;
     }
     p.G_x = Gx; p.G_y = Gy; p.W = W; p.K = (int)s->K;
-    if (Gx < p.T + 2 * W || Gy < p.T + 2 * W) {
-        set_error("oversampled grid too small for gridding tiles");
+    if (Gx < 32 + 2 * W || Gy < 32 + 2 * W) {   // 40 points: see pp_sampling
+        set_error("oversampled grid too small for gridding");
         return PP_ERR_UNSUPPORTED;
     }
     PP_TRY(make_fft(p, Gx, p.gx));
@@ -431,64 +444,46 @@ static pp_status build_noncartesian(Plan& p, const pp_sampling* s) {
         size_t handed = 1;
         try {
             for (int t = 1; t < nth; ++t, ++handed)
-                pool.emplace_back(body, t, (int)((int64_t)K * t / nth), (int)((int64_t)K * (t + 1) / nth));
+                pool.emplace_back(body, (int)((int64_t)K * t / nth), (int)((int64_t)K * (t + 1) / nth));
         } catch (const std::exception&) {
             // no more threads: the calling thread takes the ranges not handed out
             for (int t = (int)handed; t < nth; ++t)
-                body(t, (int)((int64_t)K * t / nth), (int)((int64_t)K * (t + 1) / nth));
+                body((int)((int64_t)K * t / nth), (int)((int64_t)K * (t + 1) / nth));
         }
-        body(0, 0, (int)((int64_t)K / nth));
+        body(0, (int)((int64_t)K / nth));
         for (auto& th : pool) th.join();
     };
-    on_threads([&](int, int k0, int k1) { taps(k0, k1); });
+    on_threads(taps);
     if (bad.load() < K) {
         const int k = bad.load();
         set_error("trajectory sample %d (%g, %g) outside [-n/2, n/2)", k, s->traj[2 * k], s->traj[2 * k + 1]);
         return PP_ERR_INVALID_ARG;
     }
     PP_TRY(upload(p, &p.samp, st));
-    // tile lists (with halo): every tile whose rows and columns meet the footprint
-    const int T = p.T, H = W - 1;
-    p.ntx = (Gx + T - 1) / T;
-    p.nty = (Gy + T - 1) / T;
-    const int ntiles = p.ntx * p.nty;
-    // per-tile lists in ascending sample order: each thread fills the lists of
-    // its sample range, and the ranges are concatenated in order
-    std::vector<std::vector<std::vector<TileEntry>>> lists(nth, std::vector<std::vector<TileEntry>>(ntiles));
-    on_threads([&](int t, int k0, int k1) {
-        for (int k = k0; k < k1; ++k) {
-            int trow[4], tcol[4], nr = 0, nc = 0;
-            for (int b = 0; b < W; ++b) {
-                const int ty = wrap_host(st[k].iy0 + b, Gy) / T;
-                if (std::find(trow, trow + nr, ty) == trow + nr) trow[nr++] = ty;
-                const int tx = wrap_host(st[k].ix0 + b, Gx) / T;
-                if (std::find(tcol, tcol + nc, tx) == tcol + nc) tcol[nc++] = tx;
-            }
-            for (int i = 0; i < nr; ++i)
-                for (int j = 0; j < nc; ++j) {
-                    const int ty0 = trow[i] * T, tx0 = tcol[j] * T;
-                    const int ly0 = wrap_host(st[k].iy0 - ty0 + H, Gy);
-                    const int lx0 = wrap_host(st[k].ix0 - tx0 + H, Gx);
-                    TileEntry e;
-                    e.wx = st[k].wx;
-                    e.wy = st[k].wy;
-                    e.lyx = ly0 | (lx0 << 16);
-                    e.k = k;
-                    lists[t][trow[i] * p.ntx + tcol[j]].push_back(e);
-                }
+    // samples sorted by the cell of their first tap (stable: trajectory order
+    // within a cell), for the spread
+    {
+        std::vector<int> start((size_t)Gx * Gy + 1, 0), cell(K);
+        for (int k = 0; k < K; ++k) {
+            cell[k] = wrap_host(st[k].iy0, Gy) * Gx + wrap_host(st[k].ix0, Gx);
+            ++start[cell[k] + 1];
         }
-    });
-    std::vector<int> start(ntiles + 1, 0);
-    std::vector<TileEntry> flat;
-    for (int t = 0; t < ntiles; ++t) {
-        start[t] = (int)flat.size();
-        for (int r = 0; r < nth; ++r) flat.insert(flat.end(), lists[r][t].begin(), lists[r][t].end());
-        p.max_tile_len = std::max(p.max_tile_len, (int)flat.size() - start[t]);
+        for (size_t i = 0; i < (size_t)Gx * Gy; ++i) start[i + 1] += start[i];
+        std::vector<float4> wx(K), wy(K);
+        std::vector<int2> kx(K);
+        std::vector<int> next(start.begin(), start.end() - 1);
+        for (int k = 0; k < K; ++k) {
+            const int j = next[cell[k]]++;
+            wx[j] = st[k].wx;
+            wy[j] = st[k].wy;
+            kx[j] = make_int2(k, cell[k] % Gx);
+        }
+        PP_TRY(upload(p, &p.cell_start, start));
+        PP_TRY(upload(p, &p.sort_wx, wx));
+        PP_TRY(upload(p, &p.sort_wy, wy));
+        PP_TRY(upload(p, &p.sort_kx, kx));
+        PP_TRY(alloc_n(p, &p.ksp_t, nufft_transposed_elems(p)));
     }
-    start[ntiles] = (int)flat.size();
-    if (flat.empty()) flat.push_back(TileEntry());
-    PP_TRY(upload(p, &p.tiles, flat));
-    PP_TRY(upload(p, &p.tile_start, start));
     // G^T G as (2W-1)^2 weight planes (FP64 sums of the taps' pairwise
     // products, stored FP32), in both layouts, built on the device
     if (!p.toep) {   // (a Toeplitz plan's normal operator needs no stencil)

@@ -75,16 +75,6 @@ struct DevFft {
     float2* tw = nullptr;
 };
 
-// One (tile, sample) pair of the gridding tile lists.  Taps of the sample are
-// at halo rows ly0 .. ly0+W-1 and columns lx0 .. lx0+W-1, where halo row 0
-// is grid row ty0 - H (H = W-1 the halo width) of the tile starting at ty0.
-struct TileEntry {
-    float4 wx;   // x-tap weights a = 0..3 (unused taps are 0)
-    float4 wy;   // y-tap weights
-    int lyx;     // ly0 | (lx0 << 16)
-    int k;       // sample index (trajectory order)
-};
-
 // Per-sample gridding metadata in trajectory order.
 struct SampleTaps {
     float4 wx;
@@ -136,12 +126,14 @@ struct Plan {
     float* mask_fo = nullptr;   // same shape, FFT order, times 1/(ny nz)
 
     // Non-Cartesian
-    int G_x = 0, G_y = 0, W = 0, K = 0, T = 32, ntx = 0, nty = 0;
+    int G_x = 0, G_y = 0, W = 0, K = 0;
     float* deapod_x = nullptr;   // [nx] 1/(sqrt(nx) psi_x)
     float* deapod_y = nullptr;   // [ny]
-    TileEntry* tiles = nullptr;
-    int* tile_start = nullptr;   // [ntiles + 1]
-    int max_tile_len = 0;
+    // samples sorted by the grid cell (row-major) of their first tap
+    int* cell_start = nullptr;   // [G_y * G_x + 1]
+    float4 *sort_wx = nullptr, *sort_wy = nullptr;   // [K] tap weights
+    int2* sort_kx = nullptr;     // [K] (sample, first tap's column)
+    float2* ksp_t = nullptr;     // [K][C rounded up] transposed k-space
     SampleTaps* samp = nullptr;  // [K]
     float* gtg = nullptr;        // [(2W-1)^2][G_y][G_x] stencil of G^T G
     float* gtg8 = nullptr;       // the same weights as [G_y][ceil(G_x/8)][(2W-1)^2][8]
@@ -260,7 +252,10 @@ pp_status launch_expand(const float2* x, const float2* s, float2* out, int64_t n
 pp_status launch_conj_accum(const float2* s, const float2* wv, float2* out, int64_t n, int first,
                             float scale, const float2* operand, float alpha, int last,
                             cudaStream_t st);
-pp_status launch_nufft_spread(const Plan& p, const float2* ksp, float2* grid_out, cudaStream_t st);
+// pp_nufft.cu; ci: coil-innermost grid; kt: scratch of the spread (NULL: none)
+size_t nufft_transposed_elems(const Plan& p);
+pp_status launch_nufft_spread(const Plan& p, const float2* ksp, float2* kt, float2* grid_out, bool ci,
+                              cudaStream_t st);
 pp_status launch_gtg_stencil(const Plan& p, const float2* grid_in, float2* grid_out, cudaStream_t st);
 pp_status prepare_gtg_stencil(Plan& p);
 pp_status build_gtg_device(Plan& p, cudaStream_t st);
@@ -296,9 +291,15 @@ pp_status launch_prox_db4(int nx, int ny, int levels, float lambda, const float2
 pp_status launch_prox_fista_db4(const Plan& p, int levels, float lambda, float gamma, float beta,
                                 const float2* u, float2* scratch, const float2* ref, double* hist_slot,
                                 cudaStream_t st);
+// the two halves of ci_normal around the G^T G stencil: image -> grid (into
+// p.ci_b) and grid -> image (through p.ci_a)
+pp_status ci_to_grid(const Plan& p, const float2* x, cudaStream_t st);
+pp_status ci_from_grid(const Plan& p, const float2* grid, float2* out, float scale,
+                       const float2* operand, float alpha, cudaStream_t st);
 pp_status ci_normal(const Plan& p, const float2* x, float2* out, float scale, const float2* operand,
                     float alpha, int ry, cudaStream_t st);   // ry 0: coil-pair stencil
-pp_status launch_nufft_degrid(const Plan& p, const float2* grid_in, float2* ksp, cudaStream_t st);
+pp_status launch_nufft_degrid(const Plan& p, const float2* grid_in, float2* ksp, bool ci,
+                              cudaStream_t st);
 pp_status launch_prox(int ndim, int nx, int ny, int nz, int levels, float lambda,
                       const float2* in, float2* out, cudaStream_t st);
 pp_status launch_prox_fista(const Plan& p, int levels, float lambda, float gamma, float beta,
@@ -313,7 +314,7 @@ pp_status launch_axpby(const float2* x, float a, const float2* y, float b, float
                        cudaStream_t st);
 pp_status launch_start_vector(float2* v, int64_t n, uint64_t seed, cudaStream_t st);
 // x = A^H y with caller-chosen intermediate buffers (pp_capi.cu)
-pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, float2* wb,
+pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, float2* wb, float2* kt,
                      cudaStream_t st);
 
 }  // namespace pp

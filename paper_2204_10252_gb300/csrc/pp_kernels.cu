@@ -333,101 +333,6 @@ __global__ void conj_accum_kernel(const float2* __restrict__ s, const float2* __
 }
 
 // ---------------------------------------------------------------------------
-// Kaiser-Bessel spreading (the adjoint's gridding, G^T) on tiles of the
-// oversampled grid (FFT order).  A CTA owns one T x T output tile and a chunk
-// of coils; every sample whose W x W footprint meets the tile is listed for
-// it (plan time), and the CTA adds the sample's value times the tap weights
-// that fall inside the tile into a shared-memory accumulator (shared-memory
-// atomics), then writes the tile once.  No global atomics.
-// ---------------------------------------------------------------------------
-template <int W>
-__global__ void __launch_bounds__(kThreads)
-nufft_spread_tile_kernel(const TileEntry* __restrict__ entries, const int* __restrict__ tile_start,
-                         int T, int ntx, int Gx, int Gy, int C, int coils_per_cta,
-                         const float2* __restrict__ ksp, int K, float2* __restrict__ grid_out) {
-    extern __shared__ float2 sm[];
-    constexpr int H = W - 1;
-    float* acc = reinterpret_cast<float*>(sm);
-    const int tile = blockIdx.x;
-    const int tyi = tile / ntx, txi = tile - tyi * ntx;
-    const int ty0 = tyi * T, tx0 = txi * T;
-    const int th = min(T, Gy - ty0), tw_ = min(T, Gx - tx0);
-    const int e0 = tile_start[tile], e1 = tile_start[tile + 1];
-    const int64_t gsz = (int64_t)Gx * Gy;
-    const int c0 = blockIdx.y * coils_per_cta;
-    const int c1 = min(C, c0 + coils_per_cta);
-    for (int c = c0; c < c1; ++c) {
-        for (int idx = threadIdx.x; idx < 2 * T * T; idx += blockDim.x) acc[idx] = 0.f;
-        __syncthreads();
-        // lane l of a warp takes entries l*S, l*S + 1, ... of the tile's list
-        // (trajectory order), so the 32 samples spread at one time lie far
-        // apart along the trajectory and their shared-memory atomics rarely
-        // hit the same grid point
-        const int ne = e1 - e0, S = (ne + 31) / 32;
-        for (int i = threadIdx.x; i < 32 * S; i += blockDim.x) {
-            const int e = e0 + (i & 31) * S + (i >> 5);
-            if (e >= e1) continue;
-            const TileEntry te = entries[e];
-            const float wx[4] = {te.wx.x, te.wx.y, te.wx.z, te.wx.w};
-            const float wy[4] = {te.wy.x, te.wy.y, te.wy.z, te.wy.w};
-            const int ly0 = te.lyx & 0xffff, lx0 = te.lyx >> 16;
-            const float2 v = ksp[(int64_t)c * K + te.k];
-#pragma unroll
-            for (int b = 0; b < W; ++b) {
-                const int yy = ly0 + b - H;
-                if (yy < 0 || yy >= th) continue;
-                const float vyx = wy[b] * v.x, vyy = wy[b] * v.y;
-#pragma unroll
-                for (int a = 0; a < W; ++a) {
-                    const int xx = lx0 + a - H;
-                    if (xx < 0 || xx >= tw_) continue;
-                    atomicAdd(&acc[2 * (yy * T + xx)], wx[a] * vyx);
-                    atomicAdd(&acc[2 * (yy * T + xx) + 1], wx[a] * vyy);
-                }
-            }
-        }
-        __syncthreads();
-        float2* gout = grid_out + c * gsz;
-        for (int idx = threadIdx.x; idx < th * T; idx += blockDim.x) {
-            const int yy = idx / T, xx = idx - yy * T;
-            if (xx < tw_)
-                gout[(int64_t)(ty0 + yy) * Gx + tx0 + xx] = make_float2(acc[2 * idx], acc[2 * idx + 1]);
-        }
-        __syncthreads();
-    }
-}
-
-// Degridding in trajectory order: ksp[c][k] = sum_ab wy_b wx_a grid_c[iy0+b][ix0+a].
-template <int W>
-__global__ void nufft_degrid_kernel(const SampleTaps* __restrict__ st, int K, int Gx, int Gy,
-                                    const float2* __restrict__ grid, float2* __restrict__ ksp) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int c = blockIdx.y;
-    if (k >= K) return;
-    const SampleTaps s = st[k];
-    const float wx[4] = {s.wx.x, s.wx.y, s.wx.z, s.wx.w};
-    const float wy[4] = {s.wy.x, s.wy.y, s.wy.z, s.wy.w};
-    const float2* gc = grid + (int64_t)c * Gx * Gy;
-    float2 v = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int b = 0; b < W; ++b) {
-        const int gy = wrapG(s.iy0 + b, Gy);
-        float2 rs = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            const int gx = wrapG(s.ix0 + a, Gx);
-            const float2 g = gc[(int64_t)gy * Gx + gx];
-            rs.x += wx[a] * g.x;
-            rs.y += wx[a] * g.y;
-        }
-        v.x += wy[b] * rs.x;
-        v.y += wy[b] * rs.y;
-    }
-    ksp[(int64_t)c * K + k] = v;
-}
-
-
-// ---------------------------------------------------------------------------
 // Gridding pair of the normal operator as a stencil.  With interpolation
 // G (samples <- grid) and spreading G^T, the normal operator needs G^T G on
 // the oversampled grid, a real symmetric matrix that couples grid points at
@@ -1429,7 +1334,6 @@ pp_status configure_kernels() {
     PP_TRY_CUDA(cudaFuncSetAttribute(cart2d_normal_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_adj_cb_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_adj_cb_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
-    PP_TRY_CUDA(cudaFuncSetAttribute(nufft_spread_tile_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     return PP_OK;
 }
 
@@ -1533,8 +1437,6 @@ pp_status launch_conj_accum(const float2* s, const float2* wv, float2* out, int6
                                                           last);
     return check_launch("conj_accum_kernel");
 }
-
-static size_t tile_smem(const Plan& p) { return sizeof(float2) * (size_t)p.T * p.T; }
 
 template <int R, int CG, int NWY>
 static pp_status rb_prepare(const Plan& p, int* grid) {
@@ -1672,20 +1574,6 @@ pp_status launch_gtg_stencil(const Plan& p, const float2* grid_in, float2* grid_
     dim3 grid((p.G_x + 15) / 16, (p.G_y + 15) / 16, (p.C + cpc - 1) / cpc);
     gtg_stencil_kernel<4><<<grid, kThreads, 0, st>>>(p.gtg, p.G_x, p.G_y, p.C, cpc, grid_in, grid_out);
     return check_launch("gtg_stencil_kernel");
-}
-
-pp_status launch_nufft_spread(const Plan& p, const float2* ksp, float2* grid_out, cudaStream_t st) {
-    const int cpc = 4;
-    dim3 grid(p.ntx * p.nty, (p.C + cpc - 1) / cpc);
-    nufft_spread_tile_kernel<4><<<grid, kThreads, tile_smem(p), st>>>(
-        p.tiles, p.tile_start, p.T, p.ntx, p.G_x, p.G_y, p.C, cpc, ksp, p.K, grid_out);
-    return check_launch("nufft_spread_tile_kernel");
-}
-
-pp_status launch_nufft_degrid(const Plan& p, const float2* grid_in, float2* ksp, cudaStream_t st) {
-    dim3 grid((p.K + kThreads - 1) / kThreads, p.C);
-    nufft_degrid_kernel<4><<<grid, kThreads, 0, st>>>(p.samp, p.K, p.G_x, p.G_y, grid_in, ksp);
-    return check_launch("nufft_degrid_kernel");
 }
 
 pp_status launch_prox(int ndim, int nx, int ny, int nz, int levels, float lambda,

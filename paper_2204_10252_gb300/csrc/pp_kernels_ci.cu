@@ -886,56 +886,46 @@ pp_status ci_prepare(Plan& p, cudaStream_t st) {
     return PP_OK;
 }
 
-// out = scale * A^H A x + alpha * operand on the coil-innermost buffers
-pp_status ci_normal(const Plan& p, const float2* x, float2* out, float scale, const float2* operand,
-                    float alpha, int ry, cudaStream_t st) {
-    const int nx = p.nx, ny = p.ny, Gx = p.G_x, Gy = p.G_y;
-    const int n2x = fft4_n2(Gx), n2y = fft4_n2(Gy);
-    const bool pdl = p.pdl != 0;
+// Column FFTs of a coil-innermost plan along the rows of [H][Gx][32] arrays
+static pp_status ci_cols(const Plan& p, bool inv, const float2* src, float2* dst, cudaStream_t st) {
+    const int ny = p.ny, Gx = p.G_x, Gy = p.G_y, n2y = fft4_n2(Gy);
+    const int hin = inv ? Gy : ny, hout = inv ? ny : Gy, oin = inv ? 0 : ny / 2, oout = inv ? ny / 2 : 0;
+#define PP_CIC(N2_)                                                                                \
+    if (n2y == N2_)                                                                                \
+        PP_TRY_CUDA(launch_ex(inv ? ci_cols_kernel<N2_, true> : ci_cols_kernel<N2_, false>,        \
+                              dim3(Gx, NCB), dim3(CB * tpr<N2_>()), 0, st, p.pdl != 0, 0,          \
+                              (const float2*)p.gy.tw, hin, hout, oin, oout, Gx, src, dst));
+    PP_CIC(8) PP_CIC(12) PP_CIC(16) PP_CIC(20) PP_CIC(24)
+#undef PP_CIC
+    return check_ci("ci_cols_kernel");
+}
+
+static RowArgs ci_row_args(const Plan& p) {
     RowArgs rf{};
-    rf.n = nx; rf.G = Gx; rf.off_in = nx / 2; rf.off_out = 0; rf.nrows = ny; rf.scale = 1.f;
+    rf.n = p.nx; rf.G = p.G_x; rf.off_in = p.nx / 2; rf.off_out = 0; rf.nrows = p.ny; rf.scale = 1.f;
+    return rf;
+}
+
+pp_status ci_to_grid(const Plan& p, const float2* x, cudaStream_t st) {
+    const int n2x = fft4_n2(p.G_x);
+    const RowArgs rf = ci_row_args(p);
 #define PP_CIR(N2_)                                                                                \
     if (n2x == N2_)                                                                                \
-        PP_TRY_CUDA(launch_ex(ci_rows_fwd_kernel<N2_>, dim3(ny, NCB), dim3(CB * tpr<N2_>()), 0, st, \
-                              pdl, 0, (const float2*)p.gx.tw, rf, x, (const float2*)p.ci_sens,    \
+        PP_TRY_CUDA(launch_ex(ci_rows_fwd_kernel<N2_>, dim3(p.ny, NCB), dim3(CB * tpr<N2_>()), 0, st, \
+                              p.pdl != 0, 0, (const float2*)p.gx.tw, rf, x, (const float2*)p.ci_sens, \
                               (const float*)p.deapod_y, (const float*)p.deapod_x, p.ci_a));
     PP_CIR(8) PP_CIR(12) PP_CIR(16) PP_CIR(20) PP_CIR(24)
 #undef PP_CIR
     PP_TRY(check_ci("ci_rows_fwd_kernel"));
-#define PP_CIC(N2_, INV_, HIN, HOUT, OIN, OOUT, SRC, DST)                                          \
-    if (n2y == N2_)                                                                                \
-        PP_TRY_CUDA(launch_ex(ci_cols_kernel<N2_, INV_>, dim3(Gx, NCB), dim3(CB * tpr<N2_>()), 0,   \
-                              st, pdl, 0, (const float2*)p.gy.tw, (int)(HIN), (int)(HOUT),        \
-                              (int)(OIN), (int)(OOUT), Gx, (const float2*)(SRC), (float2*)(DST)));
-    PP_CIC(8, false, ny, Gy, ny / 2, 0, p.ci_a, p.ci_b)
-    PP_CIC(12, false, ny, Gy, ny / 2, 0, p.ci_a, p.ci_b)
-    PP_CIC(16, false, ny, Gy, ny / 2, 0, p.ci_a, p.ci_b)
-    PP_CIC(20, false, ny, Gy, ny / 2, 0, p.ci_a, p.ci_b)
-    PP_CIC(24, false, ny, Gy, ny / 2, 0, p.ci_a, p.ci_b)
-    PP_TRY(check_ci("ci_cols_kernel"));
-    const int ntiles = ry ? ((Gx + 15) / 16) * ((Gy + 4 * ry - 1) / (4 * ry)) : 0;
-    if (ry == 0)
-        PP_TRY_CUDA(launch_ex(ci_stencil_cp_kernel,
-                              dim3(((Gx + CPS_TX - 1) / CPS_TX) * ((Gy + CPS_TY - 1) / CPS_TY)), dim3(256),
-                              CPS_SMEM, st, pdl, 0, (const float*)p.gtg8, Gx, Gy, (Gx + 7) / 8,
-                              (const int*)p.ci_tile_nz, (const float2*)p.ci_b, p.ci_c));
-    else if (ry == 2)
-        PP_TRY_CUDA(launch_ex(ci_stencil_kernel<2>, dim3(ntiles), dim3(256), CiStencil<2>::SMEM, st,
-                              pdl, 0, (const float*)p.gtg8, Gx, Gy, (Gx + 7) / 8,
-                              (const float2*)p.ci_b, p.ci_c));
-    else
-        PP_TRY_CUDA(launch_ex(ci_stencil_kernel<1>, dim3(ntiles), dim3(256), CiStencil<1>::SMEM, st,
-                              pdl, 0, (const float*)p.gtg8, Gx, Gy, (Gx + 7) / 8,
-                              (const float2*)p.ci_b, p.ci_c));
-    PP_TRY(check_ci("ci_stencil_kernel"));
-    PP_CIC(8, true, Gy, ny, 0, ny / 2, p.ci_c, p.ci_a)
-    PP_CIC(12, true, Gy, ny, 0, ny / 2, p.ci_c, p.ci_a)
-    PP_CIC(16, true, Gy, ny, 0, ny / 2, p.ci_c, p.ci_a)
-    PP_CIC(20, true, Gy, ny, 0, ny / 2, p.ci_c, p.ci_a)
-    PP_CIC(24, true, Gy, ny, 0, ny / 2, p.ci_c, p.ci_a)
-#undef PP_CIC
-    PP_TRY(check_ci("ci_cols_kernel"));
-    RowArgs ra = rf;
+    return ci_cols(p, false, p.ci_a, p.ci_b, st);
+}
+
+pp_status ci_from_grid(const Plan& p, const float2* grid, float2* out, float scale,
+                       const float2* operand, float alpha, cudaStream_t st) {
+    const int nx = p.nx, ny = p.ny, n2x = fft4_n2(p.G_x);
+    const bool pdl = p.pdl != 0;
+    PP_TRY(ci_cols(p, true, grid, p.ci_a, st));
+    RowArgs ra = ci_row_args(p);
     ra.off_in = 0; ra.off_out = nx / 2;
     if (p.tune_rows_adj_cl == 4) {
         cudaError_t e = cudaSuccess;
@@ -964,6 +954,30 @@ pp_status ci_normal(const Plan& p, const float2* x, float2* out, float scale, co
     PP_TRY_CUDA(launch_ex(ci_sum_kernel, dim3(blocks), dim3(256), 0, st, pdl, 0,
                           (const float2*)p.ci_part, n, scale, operand, alpha, out));
     return check_ci("ci_sum_kernel");
+}
+
+// out = scale * A^H A x + alpha * operand on the coil-innermost buffers
+pp_status ci_normal(const Plan& p, const float2* x, float2* out, float scale, const float2* operand,
+                    float alpha, int ry, cudaStream_t st) {
+    const int Gx = p.G_x, Gy = p.G_y;
+    const bool pdl = p.pdl != 0;
+    PP_TRY(ci_to_grid(p, x, st));
+    const int ntiles = ry ? ((Gx + 15) / 16) * ((Gy + 4 * ry - 1) / (4 * ry)) : 0;
+    if (ry == 0)
+        PP_TRY_CUDA(launch_ex(ci_stencil_cp_kernel,
+                              dim3(((Gx + CPS_TX - 1) / CPS_TX) * ((Gy + CPS_TY - 1) / CPS_TY)), dim3(256),
+                              CPS_SMEM, st, pdl, 0, (const float*)p.gtg8, Gx, Gy, (Gx + 7) / 8,
+                              (const int*)p.ci_tile_nz, (const float2*)p.ci_b, p.ci_c));
+    else if (ry == 2)
+        PP_TRY_CUDA(launch_ex(ci_stencil_kernel<2>, dim3(ntiles), dim3(256), CiStencil<2>::SMEM, st,
+                              pdl, 0, (const float*)p.gtg8, Gx, Gy, (Gx + 7) / 8,
+                              (const float2*)p.ci_b, p.ci_c));
+    else
+        PP_TRY_CUDA(launch_ex(ci_stencil_kernel<1>, dim3(ntiles), dim3(256), CiStencil<1>::SMEM, st,
+                              pdl, 0, (const float*)p.gtg8, Gx, Gy, (Gx + 7) / 8,
+                              (const float2*)p.ci_b, p.ci_c));
+    PP_TRY(check_ci("ci_stencil_kernel"));
+    return ci_from_grid(p, p.ci_c, out, scale, operand, alpha, st);
 }
 
 bool toep_supported(int nx, int ny, int C) {

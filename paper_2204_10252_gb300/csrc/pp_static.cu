@@ -93,6 +93,12 @@ extern "C" pp_status pp_adjoint_apply_static(const pp_plan* plan, const pp_c64* 
     PP_TRY(static_scratch(&base));
     // Every scratch element read by the adjoint is written earlier in the
     // same call, so nothing needs clearing between calls.
+    // The transposed k-space of the spread takes what is left, if it fits.
+    float2* kt = nullptr;
+    if (p.kind != PP_CARTESIAN &&
+        (na + nb + (int64_t)nufft_transposed_elems(p)) * (int64_t)sizeof(float2) <=
+            (int64_t)PP_STATIC_SCRATCH_BYTES)
+        kt = base + na + nb;
     return adjoint_ws(p, reinterpret_cast<const float2*>(yk), reinterpret_cast<float2*>(xo), base,
-                      base + na, (cudaStream_t)stream);
+                      base + na, kt, (cudaStream_t)stream);
 }
