@@ -202,6 +202,8 @@ static pp_status normal_into(const Plan& p, const float2* x, float2* out, float 
         bool done = false;
         PP_TRY(cart3d4_normal(p, x, out, scale, operand, alpha, p.wk_a, st, &done));
         if (done) return PP_OK;
+        PP_TRY(gen_cart3d_normal(p, x, out, scale, operand, alpha, p.wk_a, p.c3_chunk, st, &done));
+        if (done) return PP_OK;
         // 3-D: per coil, y FFT -> (z FFT, mask, z IFFT) -> y IFFT -> conj accumulate
         for (int c = 0; c < p.C; ++c) {
             const float2* sc = p.sens + (int64_t)c * n;
@@ -247,18 +249,26 @@ static pp_status forward_into(const Plan& p, const float2* x, float2* y, cudaStr
     if (p.kind == PP_CARTESIAN) {
         // centred orthonormal FFT along x, then y (then z), mask on the last axis pass
         RowArgs rf = row_args(nx, nx, nx / 2, nx / 2, ny * nz, n, (float)(1.0 / sqrt((double)nx)));
-        PP_TRY(launch_rows_fwd(p, p.fx, rf, x, p.sens, nullptr, nullptr, y, p.C, 0, st));
         ColArgs ay = col_args(ny, ny, ny, ny / 2, ny / 2, nx, (int64_t)ny * nx, (int64_t)ny * nx,
                               p.C * nz, (float)(1.0 / sqrt((double)ny)));
         if (p.ndim == 2) {
+            PP_TRY(launch_rows_fwd(p, p.fx, rf, x, p.sens, nullptr, nullptr, y, p.C, 0, st));
             ay.mul_out = p.mask_c; ay.mo_q = 1; ay.mo_c = 0; ay.mo_cdiv = 1;
             return launch_cols(p.fy, ay, y, y, false, st);
         }
-        PP_TRY(launch_cols(p.fy, ay, y, y, false, st));
-        ColArgs az = col_args(nz, nz, nz, nz / 2, nz / 2, ny * nx, n, n, p.C,
-                              (float)(1.0 / sqrt((double)nz)));
-        az.mul_out = p.mask_c; az.mo_q = ny; az.mo_c = 1; az.mo_cdiv = nx;
-        return launch_cols(p.fz, az, y, y, false, st);
+        // a chunk of coils at a time, so that its three passes meet in L2
+        for (int c0 = 0; c0 < p.C; c0 += p.c3_chunk) {
+            const int nc = std::min(p.c3_chunk, p.C - c0);
+            float2* yc = y + (int64_t)c0 * n;
+            PP_TRY(launch_rows_fwd(p, p.fx, rf, x, p.sens + (int64_t)c0 * n, nullptr, nullptr, yc, nc, 0, st));
+            ay.nbatch = nc * nz;
+            PP_TRY(launch_cols(p.fy, ay, yc, yc, false, st));
+            ColArgs az = col_args(nz, nz, nz, nz / 2, nz / 2, ny * nx, n, n, nc,
+                                  (float)(1.0 / sqrt((double)nz)));
+            az.mul_out = p.mask_c; az.mo_q = ny; az.mo_c = 1; az.mo_cdiv = nx;
+            PP_TRY(launch_cols(p.fz, az, yc, yc, false, st));
+        }
+        return PP_OK;
     }
     if (use_ci(p)) {
         PP_TRY(ci_to_grid(p, x, st));
@@ -274,10 +284,10 @@ static pp_status forward_into(const Plan& p, const float2* x, float2* y, cudaStr
 
 // x = A^H y (unscaled) with the intermediates in wa and wb (plan workspace, or the
 // library's fixed scratch array for pp_adjoint_apply_static): Cartesian 2-D
-// needs C*n elements in wa; 3-D n in wa and n in wb; non-Cartesian C*ny*G_x
+// needs C*n elements in wa; 3-D chunk*n in wa; non-Cartesian C*ny*G_x
 // in wa and C*G_y*G_x in wb, and optionally the transposed k-space in kt.
 pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, float2* wb, float2* kt,
-                     cudaStream_t st) {
+                     int chunk, cudaStream_t st) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int64_t n = p.nimg;
     if (p.kind == PP_CARTESIAN && p.ndim == 2) {
@@ -289,20 +299,21 @@ pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, floa
         return launch_rows_adj(p, p.fx, ra, wa, p.sens, nullptr, nullptr, x, nullptr, 0.f, p.C, st);
     }
     if (p.kind == PP_CARTESIAN) {
-        // 3-D, per coil: mask and inverse centred FFT along z, then y, then
-        // the x rows with the conjugate sensitivity, accumulated into x.
-        for (int c = 0; c < p.C; ++c) {
-            const float2* yc = y + (int64_t)c * n;
-            ColArgs az = col_args(nz, nz, nz, nz / 2, nz / 2, ny * nx, 0, 0, 1,
+        // 3-D, `chunk` coils at a time (their planes meet in L2): mask and
+        // inverse centred FFT along z into wa, then y in place, then the x rows
+        // with the conjugate sensitivities, accumulated into x.
+        for (int c0 = 0; c0 < p.C; c0 += chunk) {
+            const int nc = std::min(chunk, p.C - c0);
+            ColArgs az = col_args(nz, nz, nz, nz / 2, nz / 2, ny * nx, n, n, nc,
                                   (float)(1.0 / sqrt((double)nz)));
             az.mul_in = p.mask_c; az.mi_q = ny; az.mi_c = 1; az.mi_cdiv = nx;
-            PP_TRY(launch_cols(p.fz, az, yc, wa, true, st));
+            PP_TRY(launch_cols(p.fz, az, y + (int64_t)c0 * n, wa, true, st));
             ColArgs ay = col_args(ny, ny, ny, ny / 2, ny / 2, nx, (int64_t)ny * nx, (int64_t)ny * nx,
-                                  nz, (float)(1.0 / sqrt((double)ny)));
-            PP_TRY(launch_cols(p.fy, ay, wa, wb, true, st));
-            RowArgs ra = row_args(nx, nx, nx / 2, nx / 2, ny * nz, 0, (float)(1.0 / sqrt((double)nx)));
-            PP_TRY(launch_rows_adj(p, p.fx, ra, wb, p.sens + (int64_t)c * n, nullptr, nullptr, x,
-                                   c == 0 ? nullptr : x, 1.f, 1, st));
+                                  nz * nc, (float)(1.0 / sqrt((double)ny)));
+            PP_TRY(launch_cols(p.fy, ay, wa, wa, true, st));
+            RowArgs ra = row_args(nx, nx, nx / 2, nx / 2, ny * nz, n, (float)(1.0 / sqrt((double)nx)));
+            PP_TRY(launch_rows_adj(p, p.fx, ra, wa, p.sens + (int64_t)c0 * n, nullptr, nullptr, x,
+                                   c0 == 0 ? nullptr : x, 1.f, nc, st));
         }
         return PP_OK;
     }
@@ -320,7 +331,7 @@ static pp_status adjoint_into(const Plan& p, const float2* y, float2* x, cudaStr
         PP_TRY(launch_nufft_spread(p, y, p.ksp_t, p.ci_c, true, st));
         return ci_from_grid(p, p.ci_c, x, 1.f, nullptr, 0.f, st);
     }
-    return adjoint_ws(p, y, x, p.wk_a, p.wk_b, p.ksp_t, st);
+    return adjoint_ws(p, y, x, p.wk_a, p.wk_b, p.ksp_t, p.c3_chunk, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -358,7 +369,9 @@ static pp_status build_cartesian(Plan& p, const uint8_t* mask) {
     } else if (p.ndim == 2) {
         PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.C * p.nimg));
     } else {
-        PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.nimg));
+        // coils whose planes fill about half of the L2 (129 MB) together
+        p.c3_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(p.C, (72ll << 20) / (8 * p.nimg)));
+        PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.c3_chunk * p.nimg));
         PP_TRY(alloc_n(p, &p.wk_b, (size_t)p.nimg));
     }
     p.nksp = (int64_t)p.C * p.nimg;

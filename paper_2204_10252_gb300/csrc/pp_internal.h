@@ -75,6 +75,12 @@ struct DevFft {
     float2* tw = nullptr;
 };
 
+// A transform length as the product of two register DFT lengths, n1 <= n2
+// (0: none), see pp_fftgen.cuh.
+struct GenSplit {
+    int n1 = 0, n2 = 0;
+};
+
 // Per-sample gridding metadata in trajectory order.
 struct SampleTaps {
     float4 wx;
@@ -177,6 +183,7 @@ struct Plan {
                                 // a 1- / 2-row coil-lane or a coil-pair stencil
     int tune_stencil_cpc = 0;   // coils per CTA of kinds 0 and 1
     int stencil_rb_grid[4] = {0, 0, 0, 0};   // persistent grid of kinds 2..5 (0: unavailable)
+    int c3_chunk = 1;           // 3-D: coils that the workspace wk_a holds
     int c3cl_clusters = 0;      // 3-D: resident 16-CTA clusters of the one-kernel operator, 4 columns
     int c3cl2_clusters = 0;     //      the same with 2 columns per task (0: n/a)
     // 3-D dataflow operator (one persistent kernel per apply, pp_cart3d_df.cu)
@@ -236,6 +243,23 @@ pp_status launch_cart2d4_normal(const Plan& p, const float2* x, float2* out, flo
 pp_status launch_rows4_adj(const DevFft& f, const RowArgs& a, const float2* src, const float2* sens,
                            const float* wrow, const float* wcol, float2* out, const float2* operand,
                            float alpha, int ncoils, cudaStream_t st, bool* done, int cluster = 0);
+// two-factor FFT stages for any supported length (pp_kernels_gen.cu); *done =
+// false when the length has no pair of register factors
+GenSplit gen_split_of(int n);
+pp_status configure_gen_kernels();
+pp_status launch_gen_cols(const DevFft& f, const ColArgs& a, const float2* src, float2* dst, bool inv,
+                          const float2* ximg, int nimgs, cudaStream_t st, bool* done);
+pp_status launch_gen_roundtrip(const DevFft& f, const ColArgs& a, const float* mask_fo,
+                               const float2* src, float2* dst, cudaStream_t st, bool* done);
+pp_status launch_gen_rows_fwd(const DevFft& f, const RowArgs& a, const float2* x, const float2* sens,
+                              const float* wrow, const float* wcol, float2* out, int ncoils,
+                              int64_t img_batch_stride, cudaStream_t st, bool* done);
+pp_status launch_gen_rows_adj(const DevFft& f, const RowArgs& a, const float2* src, const float2* sens,
+                              const float* wrow, const float* wcol, float2* out, const float2* operand,
+                              float alpha, int ncoils, cudaStream_t st, bool* done);
+pp_status gen_cart3d_normal(const Plan& p, const float2* x, float2* out, float scale,
+                            const float2* operand, float alpha, float2* W, int chunk, cudaStream_t st,
+                            bool* done);
 pp_status launch_rows_fwd(const Plan& p, const DevFft& f, const RowArgs& a, const float2* x,
                           const float2* sens, const float* wrow, const float* wcol, float2* out,
                           int ncoils, int64_t img_batch_stride, cudaStream_t st);
@@ -315,7 +339,7 @@ pp_status launch_axpby(const float2* x, float a, const float2* y, float b, float
 pp_status launch_start_vector(float2* v, int64_t n, uint64_t seed, cudaStream_t st);
 // x = A^H y with caller-chosen intermediate buffers (pp_capi.cu)
 pp_status adjoint_ws(const Plan& p, const float2* y, float2* x, float2* wa, float2* wb, float2* kt,
-                     cudaStream_t st);
+                     int chunk, cudaStream_t st);
 
 }  // namespace pp
 

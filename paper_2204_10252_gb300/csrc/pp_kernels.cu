@@ -1319,6 +1319,7 @@ static size_t rows_smem(int G) { return sizeof(float2) * (size_t)(G + 2 * RB * r
 static size_t cols_smem(int G) { return sizeof(float2) * (size_t)(G + 2 * G * TX); }
 
 pp_status configure_kernels() {
+    PP_TRY(configure_gen_kernels());
     const int big = 200 * 1024;
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_adj_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
@@ -1344,6 +1345,8 @@ pp_status launch_rows_fwd(const Plan& p, const DevFft& f, const RowArgs& a, cons
     bool done = false;
     PP_TRY(launch_rows4_fwd(f, a, x, sens, wrow, wcol, out, ncoils, img_batch_stride, st, &done));
     if (done) return PP_OK;
+    PP_TRY(launch_gen_rows_fwd(f, a, x, sens, wrow, wcol, out, ncoils, img_batch_stride, st, &done));
+    if (done) return PP_OK;
     dim3 grid((a.nrows + RB - 1) / RB, ncoils);
     rows_fwd_kernel<<<grid, kThreads, rows_smem(a.G), st>>>(f.d, f.tw, a, x, img_batch_stride, sens,
                                                             wrow, wcol, out);
@@ -1362,6 +1365,8 @@ pp_status launch_rows_adj(const Plan& p, const DevFft& f, const RowArgs& a, cons
         set_error("row length %d exceeds the row stage limit", a.n);
         return PP_ERR_UNSUPPORTED;
     }
+    PP_TRY(launch_gen_rows_adj(f, a, src, sens, wrow, wcol, out, operand, alpha, ncoils, st, &done));
+    if (done) return PP_OK;
     if (ncoils >= 4 && a.n <= 2 * kThreads) {
         const size_t smc = rows_smem(a.G);
         if (a.n <= kThreads)
@@ -1389,6 +1394,8 @@ pp_status launch_cols(const DevFft& f, const ColArgs& a, const float2* src, floa
     bool done = false;
     PP_TRY(launch_cols4(f, a, src, dst, inv, st, &done));
     if (done) return PP_OK;
+    PP_TRY(launch_gen_cols(f, a, src, dst, inv, nullptr, 1, st, &done));
+    if (done) return PP_OK;
     dim3 grid((a.ncols + TX - 1) / TX, a.nbatch);
     if (inv)
         cols_kernel<true><<<grid, kThreads, cols_smem(a.G), st>>>(f.d, f.tw, a, src, dst);
@@ -1399,6 +1406,9 @@ pp_status launch_cols(const DevFft& f, const ColArgs& a, const float2* src, floa
 
 pp_status launch_cols_roundtrip(const DevFft& f, const ColArgs& a, const float* mask_fo,
                                 const float2* src, float2* dst, cudaStream_t st) {
+    bool done = false;
+    PP_TRY(launch_gen_roundtrip(f, a, mask_fo, src, dst, st, &done));
+    if (done) return PP_OK;
     dim3 grid((a.ncols + TX - 1) / TX, a.nbatch);
     cols_roundtrip_kernel<<<grid, kThreads, cols_smem(a.G), st>>>(f.d, f.tw, a, mask_fo, src, dst);
     return check_launch("cols_roundtrip_kernel");

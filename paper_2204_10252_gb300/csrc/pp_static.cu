@@ -100,5 +100,5 @@ extern "C" pp_status pp_adjoint_apply_static(const pp_plan* plan, const pp_c64* 
             (int64_t)PP_STATIC_SCRATCH_BYTES)
         kt = base + na + nb;
     return adjoint_ws(p, reinterpret_cast<const float2*>(yk), reinterpret_cast<float2*>(xo), base,
-                      base + na, kt, (cudaStream_t)stream);
+                      base + na, kt, 1, (cudaStream_t)stream);
 }
