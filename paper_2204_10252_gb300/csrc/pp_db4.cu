@@ -12,24 +12,31 @@
 // v[2m+1] = h1 a[m] + h3 a[m-1] + g1 d[m] + g3 d[m-1] (indices mod n/2).
 //
 // Unlike the 2-level Haar (tile-local), every level couples neighbouring
-// tiles, so the prox runs as one pass per level and direction: a CTA owns
-// whole rows (or 8 whole columns) of the band, stages them in shared memory
-// and writes its outputs back in place.  The soft threshold is applied when
+// tiles.  Images that fit the shared memory of one thread-block cluster run in
+// one launch (db4_cluster_kernel); larger ones as one pass per level and
+// direction: a CTA owns whole rows (or 8 whole columns) of the band, stages
+// them in shared memory and writes its outputs back in place.  The soft threshold is applied when
 // a coefficient becomes final (column passes); the FISTA step w = z - gamma u
 // is fused into the first pass, the momentum update and the FP64 statistics
 // into the last.
 #include <cuda_runtime.h>
+#include <cooperative_groups.h>
 #include <math.h>
 #include <stdint.h>
 
-#include "pp_fft.cuh"
+#include <algorithm>
+
+#include "pp_fft4.cuh"
 #include "pp_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace pp {
 namespace {
 
 constexpr int MAXN = 512;   // longest row / column
 constexpr int CW = 8;       // columns per CTA in the column passes
+constexpr int kDb4Threads = 512;   // threads of a CTA of the cluster form
 
 struct Db4 {
     float h[4], g[4];
@@ -75,7 +82,7 @@ __device__ __forceinline__ void hist_add(double dd, double yy, double rr, double
         yy += __shfl_down_sync(0xffffffffu, yy, off);
         rr += __shfl_down_sync(0xffffffffu, rr, off);
     }
-    __shared__ double s[3][kThreads / 32];
+    __shared__ double s[3][kDb4Threads / 32];   // the widest block that calls this
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) {
         s[0][wid] = dd;
@@ -211,6 +218,195 @@ db4_cols_kernel(Db4 f, int h, int w, int nx, float lam, int last, float2* v) {
     }
 }
 
+// The whole prox in one launch of one cluster.  CTA q owns a slab of rows, a
+// multiple of 2^levels, in two shared buffers; the x passes are local, and a y
+// pass needs two rows of the next slab (forward) or the last approximation and
+// detail row of the previous one (inverse), which their owner pushes into this
+// CTA's halo rows through distributed shared memory before one cluster barrier a
+// level and direction.  Halo rows are used once, so nothing waits for readers.
+// B0 holds the band in Mallat order (a rows above d rows, [a | d] along x), B1 the
+// band between the two passes of a level.  Same arithmetic, in the same order, as
+// the passes above.  Bound by latency: 2 levels + 1 cluster barriers and
+// 2 * levels passes over a slab in place of 4 * levels kernels of 2 to 3 us each
+// (40 iterations at 128 x 128 and 8 coils, d = 3, 2 levels: 1000 -> 701 us).
+
+struct Db4Cluster {
+    Db4 f;
+    int nx, ny, levels, R;
+    float lam, gamma;
+    const float2* in;
+    const float2* u;     // NULL: the input is `in` alone
+    float2* out;         // NULL: the FISTA epilogue
+    Epi e;
+};
+
+__global__ void __launch_bounds__(kDb4Threads) db4_cluster_kernel(const Db4Cluster p) {
+    extern __shared__ float2 sm[];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int nx = p.nx, L = p.levels, R = p.R, q = (int)cluster.block_rank();
+    const int units = p.ny >> L;
+    const int r0 = (int)((int64_t)units * q / R) << L, rows = ((int)((int64_t)units * (q + 1) / R) << L) - r0;
+    const int slab = ((units + R - 1) / R) << L;   // rows that every CTA's buffers hold
+    float2* B0 = sm;
+    float2* B1 = B0 + slab * nx;
+    float2* HF = B1 + slab * nx;          // [level][2][nx]: the next slab's first rows
+    float2* HI = HF + 2 * L * nx;         // [level][2][nx]: the previous slab's last a and d row
+    pdl_trigger();
+    cluster_arrive_relaxed();             // every CTA of the cluster runs before the first push
+    pdl_wait();
+    const int64_t g0 = (int64_t)r0 * nx;
+    for (int e = threadIdx.x; e < rows * nx; e += blockDim.x) {
+        float2 v = p.in[g0 + e];
+        if (p.u) {
+            const float2 s = p.u[g0 + e];
+            v = make_float2(v.x - p.gamma * s.x, v.y - p.gamma * s.y);
+        }
+        B0[e] = v;
+    }
+    cluster_wait_acquire();
+    float2* const next = cluster.map_shared_rank(sm, (q + 1) % R);
+    float2* const prev = cluster.map_shared_rank(sm, (q + R - 1) % R);
+    const int oHF = (int)(HF - sm), oHI = (int)(HI - sm);
+    __syncthreads();
+    for (int l = 0; l < L; ++l) {
+        const int h = rows >> l, w = nx >> l, hw = w >> 1, hh = h >> 1;
+        for (int e = threadIdx.x; e < h * hw; e += blockDim.x) {
+            const int r = e / hw, i = e - r * hw;
+            const float2* s = B0 + r * nx;
+            float2 a = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                int j = 2 * i + k;
+                if (j >= w) j -= w;
+                a = fma2(p.f.h[k], s[j], a);
+                d = fma2(p.f.g[k], s[j], d);
+            }
+            B1[r * nx + i] = a;
+            B1[r * nx + hw + i] = d;
+            if (r < 2) {
+                prev[oHF + (2 * l + r) * nx + i] = a;
+                prev[oHF + (2 * l + r) * nx + hw + i] = d;
+            }
+        }
+        cluster_arrive_release();
+        cluster_wait_acquire();
+        const bool last = l == L - 1;
+        for (int e = threadIdx.x; e < hh * w; e += blockDim.x) {
+            const int i = e / w, c = e - i * w;
+            float2 a = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = 2 * i + k;
+                const float2 s = j < h ? B1[j * nx + c] : HF[(2 * l + j - h) * nx + c];
+                a = fma2(p.f.h[k], s, a);
+                d = fma2(p.f.g[k], s, d);
+            }
+            if (last || c >= hw) a = soft4(a, p.lam);
+            B0[i * nx + c] = a;
+            B0[(hh + i) * nx + c] = soft4(d, p.lam);
+        }
+        __syncthreads();
+    }
+    double dd = 0.0, yy = 0.0, rr = 0.0;
+    for (int l = L - 1; l >= 0; --l) {
+        const int h = rows >> l, w = nx >> l, hw = w >> 1, hh = h >> 1;
+        for (int c = threadIdx.x; c < w; c += blockDim.x) {
+            next[oHI + (2 * l) * nx + c] = B0[(hh - 1) * nx + c];
+            next[oHI + (2 * l + 1) * nx + c] = B0[(h - 1) * nx + c];
+        }
+        cluster_arrive_release();
+        cluster_wait_acquire();
+        for (int e = threadIdx.x; e < h * w; e += blockDim.x) {
+            const int j = e / w, c = e - j * w, m = j >> 1, par = j & 1;
+            const float2 a1 = m ? B0[(m - 1) * nx + c] : HI[(2 * l) * nx + c];
+            const float2 d1 = m ? B0[(hh + m - 1) * nx + c] : HI[(2 * l + 1) * nx + c];
+            float2 x = make_float2(0.f, 0.f);
+            x = fma2(par ? p.f.h[1] : p.f.h[0], B0[m * nx + c], x);
+            x = fma2(par ? p.f.h[3] : p.f.h[2], a1, x);
+            x = fma2(par ? p.f.g[1] : p.f.g[0], B0[(hh + m) * nx + c], x);
+            x = fma2(par ? p.f.g[3] : p.f.g[2], d1, x);
+            B1[j * nx + c] = x;
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < h * w; e += blockDim.x) {
+            const int r = e / w, j = e - r * w;
+            const float2* s = B1 + r * nx;
+            const int m = j >> 1, par = j & 1, m1 = m == 0 ? hw - 1 : m - 1;
+            const int64_t o = g0 + (int64_t)r * nx + j;
+            float2 yo = make_float2(0.f, 0.f);
+            if (l == 0 && !p.out) yo = p.e.y[o];
+            float2 v = make_float2(0.f, 0.f);
+            v = fma2(par ? p.f.h[1] : p.f.h[0], s[m], v);
+            v = fma2(par ? p.f.h[3] : p.f.h[2], s[m1], v);
+            v = fma2(par ? p.f.g[1] : p.f.g[0], s[hw + m], v);
+            v = fma2(par ? p.f.g[3] : p.f.g[2], s[hw + m1], v);
+            if (l > 0) {
+                B0[r * nx + j] = v;
+            } else if (p.out) {
+                p.out[o] = v;
+            } else {
+                const float2 df = csub(v, yo);
+                p.e.z[o] = make_float2(v.x + p.e.beta * df.x, v.y + p.e.beta * df.y);
+                p.e.y[o] = v;
+                if (p.e.hist) {
+                    dd += (double)df.x * df.x + (double)df.y * df.y;
+                    yy += (double)v.x * v.x + (double)v.y * v.y;
+                    if (p.e.ref) {
+                        const float2 t = p.e.ref[o];
+                        const double ex = (double)v.x - t.x, ey = (double)v.y - t.y;
+                        rr += ex * ex + ey * ey;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (!p.out && p.e.hist) hist_add(dd, yy, rr, p.e.hist);
+}
+
+// Cluster size for an image, 0 when it does not fit: 8 CTAs, or 16 (beyond the
+// portable size) for images of more than 128 x 128 where the device takes them.
+size_t db4_cluster_smem(int nx, int ny, int levels, int R) {
+    const int units = ny >> levels, slab = ((units + R - 1) / R) << levels;
+    return sizeof(float2) * ((size_t)2 * slab * nx + (size_t)4 * levels * nx);
+}
+int db4_cluster_size(int nx, int ny, int levels) {
+    constexpr int kSmem = 220 * 1024;
+    static const cudaError_t allowed = [] {
+        cudaError_t e = cudaFuncSetAttribute(db4_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(db4_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaGetLastError();
+        return e;
+    }();
+    if (allowed != cudaSuccess) return 0;
+    const int units = ny >> levels;
+    int R = (int64_t)nx * ny > 128 * 128 ? 16 : 8;
+    while (R > units) R >>= 1;
+    if (db4_cluster_smem(nx, ny, levels, R) > (size_t)kSmem) return 0;
+    static const bool sixteen = [] {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 16;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(16);
+        cfg.blockDim = dim3(kDb4Threads);
+        cfg.dynamicSmemBytes = kSmem;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, db4_cluster_kernel, &cfg);
+        cudaGetLastError();
+        return e == cudaSuccess && n > 0;
+    }();
+    if (R == 16 && !sixteen) {
+        R = 8;
+        if (db4_cluster_smem(nx, ny, levels, R) > (size_t)kSmem) return 0;
+    }
+    return R;
+}
+
 pp_status check_db4(const char* what) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e, what);
@@ -228,6 +424,12 @@ pp_status db4_prox(int nx, int ny, int levels, float lambda, const float2* in, c
                    cudaStream_t st) {
     const Db4 f = db4_filter();
     const Epi none{nullptr, nullptr, nullptr, nullptr, 0.f};
+    if (const int R = db4_cluster_size(nx, ny, levels)) {
+        const Db4Cluster p{f, nx, ny, levels, R, lambda, gamma, in, u, epi ? nullptr : out, epi ? *epi : none};
+        PP_TRY_CUDA(launch_ex(db4_cluster_kernel, dim3(R), dim3(kDb4Threads), db4_cluster_smem(nx, ny, levels, R),
+                              st, pdl, R, p));
+        return check_db4("db4_cluster_kernel");
+    }
     for (int l = 0; l < levels; ++l) {
         const int h = ny >> l, w = nx >> l;
         PP_TRY_CUDA(launch_ex(db4_rows_kernel<false, false>, dim3(h), dim3(kThreads), 0, st, pdl, 0, f,
@@ -258,6 +460,8 @@ pp_status db4_prox(int nx, int ny, int levels, float lambda, const float2* in, c
 }
 
 }  // namespace
+
+void db4_prepare() { (void)db4_cluster_size(64, 64, 1); }
 
 bool db4_supported(int ndim, int nx, int ny, int levels) {
     return ndim == 2 && levels >= 1 && levels <= 4 && nx <= MAXN && ny <= MAXN && nx > 0 && ny > 0 &&

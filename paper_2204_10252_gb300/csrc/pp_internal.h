@@ -309,6 +309,7 @@ size_t toep_rows_elems(const Plan& p);
 pp_status toep_normal(const Plan& p, const float2* x, float2* out, float scale,
                       const float2* operand, float alpha, cudaStream_t st);
 pp_status toep_build_kernel(Plan& p, const float* traj, int64_t K, cudaStream_t st);
+void db4_prepare();   // kernel attributes, before any stream capture
 bool db4_supported(int ndim, int nx, int ny, int levels);
 pp_status launch_prox_db4(int nx, int ny, int levels, float lambda, const float2* in, float2* out,
                           cudaStream_t st);

@@ -1319,6 +1319,7 @@ static size_t rows_smem(int G) { return sizeof(float2) * (size_t)(G + 2 * RB * r
 static size_t cols_smem(int G) { return sizeof(float2) * (size_t)(G + 2 * G * TX); }
 
 pp_status configure_kernels() {
+    db4_prepare();
     PP_TRY(configure_gen_kernels());
     const int big = 200 * 1024;
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
