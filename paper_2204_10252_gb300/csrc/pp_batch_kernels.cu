@@ -207,74 +207,91 @@ __device__ __forceinline__ float2 soft_b(float2 v, float lam) {
     return cscale(v, 1.f - lam * rsqrtf(m2));
 }
 
-// 2-level 2-D Haar prox of a 4x4 tile (same transform as the single-plan
-// prox kernel: block transform on 2x2 blocks, then on the four level-1
-// approximation coefficients; each block transform is its own inverse).
-__device__ __forceinline__ void prox44(float2* v, float lam) {
-#pragma unroll
-    for (int by = 0; by < 4; by += 2)
-#pragma unroll
-        for (int bx = 0; bx < 4; bx += 2)
-            haar2x2_b(v[by * 4 + bx], v[by * 4 + bx + 1], v[(by + 1) * 4 + bx], v[(by + 1) * 4 + bx + 1]);
-    haar2x2_b(v[0], v[2], v[8], v[10]);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = soft_b(v[i], lam);
-    haar2x2_b(v[0], v[2], v[8], v[10]);
-#pragma unroll
-    for (int by = 0; by < 4; by += 2)
-#pragma unroll
-        for (int bx = 0; bx < 4; bx += 2)
-            haar2x2_b(v[by * 4 + bx], v[by * 4 + bx + 1], v[(by + 1) * 4 + bx], v[(by + 1) * 4 + bx + 1]);
+// Four adjacent lanes hold one 4 x 4 tile, lane 2 qy + qx its 2 x 2 block (qx, qy):
+// level 1 of the Haar transform in registers, level 2 on the four approximation
+// coefficients by shuffles, in the operation order of haar2x2_b.  Its own inverse.
+__device__ __forceinline__ float2 shfl2_b(float2 v, int m) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
+}
+__device__ __forceinline__ float2 haar_level2(float2 a, int qx, int qy) {
+    const float2 p = shfl2_b(a, 1);
+    const float2 t = qx ? csub(p, a) : cadd(a, p);
+    const float2 r = shfl2_b(t, 2);
+    return cscale(qy ? csub(r, t) : cadd(t, r), 0.5f);
+}
+__device__ __forceinline__ void haar_quad(float2* v, int qx, int qy) {
+    haar2x2_b(v[0], v[1], v[2], v[3]);
+    v[0] = haar_level2(v[0], qx, qy);
+}
+__device__ __forceinline__ void haar_quad_inv(float2* v, int qx, int qy) {
+    v[0] = haar_level2(v[0], qx, qy);
+    haar2x2_b(v[0], v[1], v[2], v[3]);
+}
+// The 2 x 2 block as two 16-byte accesses (its columns start at even elements of
+// 16-byte aligned arrays of even pitch).
+__device__ __forceinline__ void load_quad(float2* v, const float2* p, int64_t pitch) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + pitch);
+    v[0] = make_float2(a.x, a.y);
+    v[1] = make_float2(a.z, a.w);
+    v[2] = make_float2(b.x, b.y);
+    v[3] = make_float2(b.z, b.w);
+}
+__device__ __forceinline__ void store_quad(const float2* v, float2* p, int64_t pitch) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    *reinterpret_cast<float4*>(p + pitch) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
 }
 
-// Batched fused prox + momentum over 4x4 tiles; block -> slice map as above
-// (segments count tiles).  Statistics are summed over the whole batch.
+// Batched fused prox + momentum over 4x4 tiles, four lanes a tile (one thread a
+// tile left 128 CTAs of one long load chain for eight 256 x 256 slices: 12.6 us);
+// block -> slice map as above (segments count tiles).  Statistics are summed over
+// the whole batch.
 __global__ void __launch_bounds__(kThreads)
 batch_prox_fista_kernel(const SliceDesc* __restrict__ descs, const int64_t* __restrict__ tile_off,
                         const int* __restrict__ blk_seg, const int* __restrict__ seg_first_blk,
                         float lam, float gamma, float beta, float2* __restrict__ z,
                         const float2* __restrict__ u, float2* __restrict__ y,
-                        const float2* __restrict__ ref, double* __restrict__ hist) {
+                        float2* __restrict__ w_out, const float2* __restrict__ ref,
+                        double* __restrict__ hist) {
     const int s = blk_seg[blockIdx.x];
     const int j = blockIdx.x - seg_first_blk[s];
     const SliceDesc D = descs[s];
-    const int64_t t = (int64_t)j * blockDim.x + threadIdx.x;
+    const int64_t t = (int64_t)j * (blockDim.x / 4) + (threadIdx.x >> 2);
     const int64_t ntl = tile_off[s + 1] - tile_off[s];
+    const int qx = threadIdx.x & 1, qy = (threadIdx.x >> 1) & 1;
+    const bool live = t < ntl;
     double dd = 0.0, yy = 0.0, rr = 0.0;
-    if (t < ntl) {
-        const int ntx = D.nx / 4;
-        const int64_t ty = t / ntx, tx = t - ty * ntx;
-        const int64_t o = D.img_off + ty * 4 * D.nx + tx * 4;
-        float2 v[16];
+    const int ntx = D.nx / 4;
+    const int64_t ty = live ? t / ntx : 0, tx = live ? t - ty * ntx : 0;
+    const int64_t o = D.img_off + (ty * 4 + 2 * qy) * D.nx + tx * 4 + 2 * qx;
+    float2 v[4], uv[4], yo[4];
+    load_quad(v, z + o, D.nx);
+    load_quad(uv, u + o, D.nx);
+    load_quad(yo, y + o, D.nx);
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+    for (int i = 0; i < 4; ++i) v[i] = make_float2(v[i].x - gamma * uv[i].x, v[i].y - gamma * uv[i].y);
+    if (w_out && live) store_quad(v, w_out + o, D.nx);
+    haar_quad(v, qx, qy);
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int64_t a = o + (int64_t)r * D.nx + x;
-                const float2 zv = z[a], uv = u[a];
-                v[r * 4 + x] = make_float2(zv.x - gamma * uv.x, zv.y - gamma * uv.y);
+    for (int i = 0; i < 4; ++i) v[i] = soft_b(v[i], lam);
+    haar_quad_inv(v, qx, qy);
+    if (live) {
+        float2 zn[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 df = csub(v[i], yo[i]);
+            zn[i] = make_float2(v[i].x + beta * df.x, v[i].y + beta * df.y);
+            if (hist) {   // FP64 arithmetic is slow on this part: only when asked for
+                dd += (double)df.x * df.x + (double)df.y * df.y;
+                yy += (double)v[i].x * v[i].x + (double)v[i].y * v[i].y;
             }
-        prox44(v, lam);
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int64_t a = o + (int64_t)r * D.nx + x;
-                const float2 yn = v[r * 4 + x];
-                const float2 yo = y[a];
-                const float2 df = csub(yn, yo);
-                z[a] = make_float2(yn.x + beta * df.x, yn.y + beta * df.y);
-                y[a] = yn;
-                if (hist) {   // FP64 arithmetic is slow on this part: only when asked for
-                    dd += (double)df.x * df.x + (double)df.y * df.y;
-                    yy += (double)yn.x * yn.x + (double)yn.y * yn.y;
-                }
-                if (ref) {
-                    const float2 rv = ref[a];
-                    const double ex = (double)yn.x - rv.x, ey = (double)yn.y - rv.y;
-                    rr += ex * ex + ey * ey;
-                }
+            if (ref) {
+                const float2 rv = ref[o + (int64_t)(i >> 1) * D.nx + (i & 1)];
+                const double ex = (double)v[i].x - rv.x, ey = (double)v[i].y - rv.y;
+                rr += ex * ex + ey * ey;
             }
+        }
+        store_quad(v, y + o, D.nx);
+        store_quad(zn, z + o, D.nx);
     }
     if (hist) {
 #pragma unroll
@@ -320,60 +337,43 @@ batch_prox_vjp_kernel(const SliceDesc* __restrict__ descs, const int64_t* __rest
     const int s = blk_seg[blockIdx.x];
     const int j = blockIdx.x - seg_first_blk[s];
     const SliceDesc D = descs[s];
-    const int64_t t = (int64_t)j * blockDim.x + threadIdx.x;
+    const int64_t t = (int64_t)j * (blockDim.x / 4) + (threadIdx.x >> 2);
     const int64_t ntl = tile_off[s + 1] - tile_off[s];
+    const int qx = threadIdx.x & 1, qy = (threadIdx.x >> 1) & 1;
+    const bool live = t < ntl;
     double lb = 0.0;
-    if (t < ntl) {
-        const int ntx = D.nx / 4;
-        const int64_t ty = t / ntx, tx = t - ty * ntx;
-        const int64_t o = D.img_off + ty * 4 * D.nx + tx * 4;
-        float2 cw[16], cy[16];
+    const int ntx = D.nx / 4;
+    const int64_t ty = live ? t / ntx : 0, tx = live ? t - ty * ntx : 0;
+    const int64_t o = D.img_off + (ty * 4 + 2 * qy) * D.nx + tx * 4 + 2 * qx;
+    float2 cw[4], cy[4], zb[4];
+    load_quad(zb, Zbar + o, D.nx);
+    load_quad(cy, Ybar + o, D.nx);
+    load_quad(cw, w + o, D.nx);
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int64_t a = o + (int64_t)r * D.nx + x;
-                const float2 zb = Zbar[a], yb = Ybar[a];
-                cy[r * 4 + x] = make_float2(yb.x + (1.f + beta) * zb.x, yb.y + (1.f + beta) * zb.y);
-                Ybar[a] = make_float2(-beta * zb.x, -beta * zb.y);
-                cw[r * 4 + x] = w[a];
-            }
-        // forward Haar of both tiles
-#pragma unroll
-        for (int by = 0; by < 4; by += 2)
-#pragma unroll
-            for (int bx = 0; bx < 4; bx += 2) {
-                haar2x2_b(cw[by * 4 + bx], cw[by * 4 + bx + 1], cw[(by + 1) * 4 + bx], cw[(by + 1) * 4 + bx + 1]);
-                haar2x2_b(cy[by * 4 + bx], cy[by * 4 + bx + 1], cy[(by + 1) * 4 + bx], cy[(by + 1) * 4 + bx + 1]);
-            }
-        haar2x2_b(cw[0], cw[2], cw[8], cw[10]);
-        haar2x2_b(cy[0], cy[2], cy[8], cy[10]);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float2 v = cw[i], g = cy[i];
-            const float m2 = v.x * v.x + v.y * v.y;
-            if (m2 > lam * lam) {
-                const float rm = rsqrtf(m2);
-                const float hx = v.x * rm, hy = v.y * rm;          // v / |v|
-                const float q = lam * rm;                            // lambda / |v|
-                const float proj = hx * g.x + hy * g.y;              // Re(conj(vhat) g)
-                cy[i] = make_float2((1.f - q) * g.x + q * hx * proj, (1.f - q) * g.y + q * hy * proj);
-                lb -= (double)proj;
-            } else {
-                cy[i] = make_float2(0.f, 0.f);
-            }
-        }
-        haar2x2_b(cy[0], cy[2], cy[8], cy[10]);
-#pragma unroll
-        for (int by = 0; by < 4; by += 2)
-#pragma unroll
-            for (int bx = 0; bx < 4; bx += 2)
-                haar2x2_b(cy[by * 4 + bx], cy[by * 4 + bx + 1], cy[(by + 1) * 4 + bx], cy[(by + 1) * 4 + bx + 1]);
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) wbar[o + (int64_t)r * D.nx + x] = cy[r * 4 + x];
+    for (int i = 0; i < 4; ++i) {
+        cy[i] = make_float2(cy[i].x + (1.f + beta) * zb[i].x, cy[i].y + (1.f + beta) * zb[i].y);
+        zb[i] = make_float2(-beta * zb[i].x, -beta * zb[i].y);
     }
+    if (live) store_quad(zb, Ybar + o, D.nx);
+    haar_quad(cw, qx, qy);
+    haar_quad(cy, qx, qy);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float2 v = cw[i], g = cy[i];
+        const float m2 = v.x * v.x + v.y * v.y;
+        if (m2 > lam * lam) {
+            const float rm = rsqrtf(m2);
+            const float hx = v.x * rm, hy = v.y * rm;          // v / |v|
+            const float q = lam * rm;                            // lambda / |v|
+            const float proj = hx * g.x + hy * g.y;              // Re(conj(vhat) g)
+            cy[i] = make_float2((1.f - q) * g.x + q * hx * proj, (1.f - q) * g.y + q * hy * proj);
+            if (live) lb -= (double)proj;
+        } else {
+            cy[i] = make_float2(0.f, 0.f);
+        }
+    }
+    haar_quad_inv(cy, qx, qy);
+    if (live) store_quad(cy, wbar + o, D.nx);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) lb += __shfl_down_sync(0xffffffffu, lb, off);
     __shared__ double sl[kThreads / 32];
@@ -386,209 +386,57 @@ batch_prox_vjp_kernel(const SliceDesc* __restrict__ descs, const int64_t* __rest
     }
 }
 
-// out = (accumulate ? out : 0) + sum_i coef_i * v_i
-__global__ void lincomb_kernel(LinComb lc, float2* __restrict__ out, int64_t n, int accumulate) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        float2 a = accumulate ? out[i] : make_float2(0.f, 0.f);
-        for (int k = 0; k < lc.count; ++k) {
-            const float2 v = lc.v[k][i];
-            a.x += lc.coef[k] * v.x;
-            a.y += lc.coef[k] * v.y;
-        }
-        out[i] = a;
-    }
-}
-
-// Four-step register-FFT version of cart2d_batch_normal_kernel: every slice
-// must have ny = 16 * n2 with n2 in {8, 12, 16, 20, 24}; items are 8 columns.
-__global__ void __launch_bounds__(192, 2)
-cart2d_batch4_kernel(const SliceDesc* __restrict__ descs, const int2* __restrict__ items, int nitems,
-                     const float2* __restrict__ x, float2* out, float coef, const float2* operand,
-                     float alpha) {
-    __shared__ float2 tws[384];
-    __shared__ float pm[384];
-    __shared__ float2 Y[16 * 24 * 8];
-    extern __shared__ float4 sb4[];   // double-buffered coil-map tiles, 2 * 384 * 8 float2
-    float2* Sb = reinterpret_cast<float2*>(sb4);
-    int cur = -1;
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        const int2 item = items[it];
-        const int s = item.x;
-        const SliceDesc D = descs[s];
-        if (s != cur) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < D.ny; i += blockDim.x) {
-                tws[i] = D.tw[i];
-                pm[i] = D.mask_fo[i];
-            }
-            __syncthreads();
-            cur = s;
-        }
-        const float2* xs = x + D.img_off;
-        float2* os = out + D.img_off;
-        const float2* ops = operand ? operand + D.img_off : nullptr;
-        const float sc = coef * D.invL;
-        switch (D.n2) {
-            case 8: cart_item4<8>(tws, pm, Y, Sb, xs, D.sens, D.C, D.nx, item.y, os, sc, ops, alpha); break;
-            case 12: cart_item4<12>(tws, pm, Y, Sb, xs, D.sens, D.C, D.nx, item.y, os, sc, ops, alpha); break;
-            case 16: cart_item4<16>(tws, pm, Y, Sb, xs, D.sens, D.C, D.nx, item.y, os, sc, ops, alpha); break;
-            case 20: cart_item4<20>(tws, pm, Y, Sb, xs, D.sens, D.C, D.nx, item.y, os, sc, ops, alpha); break;
-            default: cart_item4<24>(tws, pm, Y, Sb, xs, D.sens, D.C, D.nx, item.y, os, sc, ops, alpha); break;
-        }
-    }
-}
-
-// One item of cart2d_batch4_cl_kernel: CTA q of the cluster runs coils q,
-// q + CL, ... of the slice; the partial sums meet in distributed shared
-// memory and CTA q writes rows [q n / CL, (q + 1) n / CL) (sum in rank order).
-template <int N2>
-__device__ __forceinline__ void batch_item_cl(const float2* tws, const float* pm, float2* Y, float2* Sb,
-                                              const SliceDesc& D, int col0, const float2* xs,
-                                              float2* os, float sc, const float2* ops, float alpha,
-                                              int q, int CL) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    constexpr int n = 16 * N2;
-    float2 acc[16];
-    cart_item4_acc<N2>(tws, pm, Y, Sb, xs, D.sens, D.C, D.nx, col0, q, CL, acc);
-    const int lane = threadIdx.x & 7, r = threadIdx.x >> 3;
-    if (r < N2) {
+// One pass over the d + 2 vectors, the gradient and the two accumulators where
+// d + 1 dot products and two linear combinations read them three times over:
+//   partials[block][i] = Re<v_i, g> over the block's share,
+//   Zbar = wbar - sum_i c_i v_{i+1},  ahb_bar += sum_i c_i v_i.
+template <int D>
+__global__ void __launch_bounds__(kThreads) rev_combine_kernel(const RevCombine r) {
+    double dot[D + 1];
 #pragma unroll
-        for (int m1 = 0; m1 < 16; ++m1) Y[(N2 * m1 + r) * 8 + lane] = acc[m1];
+    for (int i = 0; i <= D; ++i) dot[i] = 0.0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < r.n; e += (int64_t)gridDim.x * blockDim.x) {
+        float2 v[D + 2];
+        v[0] = r.wbar[e];
+#pragma unroll
+        for (int i = 1; i <= D + 1; ++i) v[i] = r.v[(i - 1) * r.n + e];
+        const float2 g = r.g[e];
+        float2 z = v[0], a = r.ahb_bar[e];
+#pragma unroll
+        for (int i = 0; i <= D; ++i) {
+            dot[i] += (double)v[i].x * g.x + (double)v[i].y * g.y;
+            z.x -= r.c[i] * v[i + 1].x;
+            z.y -= r.c[i] * v[i + 1].y;
+            a.x += r.c[i] * v[i].x;
+            a.y += r.c[i] * v[i].y;
+        }
+        r.Zbar[e] = z;
+        r.ahb_bar[e] = a;
     }
-    cluster.sync();
-    const int rpr = n / CL;
-    for (int idx = threadIdx.x; idx < rpr * 8; idx += blockDim.x) {
-        const int row = q * rpr + (idx >> 3), l = idx & 7, col = col0 + l;
-        float2 v = cluster.map_shared_rank(Y, 0)[row * 8 + l];
-        for (int b = 1; b < CL; ++b) v = cadd(v, cluster.map_shared_rank(Y, b)[row * 8 + l]);
-        if (col < D.nx) {
-            const int64_t o = (int64_t)row * D.nx + col;
-            v = cscale(v, sc);
-            if (ops) v = cadd(v, cscale(ops[o], alpha));
-            os[o] = v;
-        }
+    __shared__ double s[D + 1][kThreads / 32];
+#pragma unroll
+    for (int i = 0; i <= D; ++i) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) dot[i] += __shfl_down_sync(0xffffffffu, dot[i], off);
+        if ((threadIdx.x & 31) == 0) s[i][threadIdx.x >> 5] = dot[i];
     }
-    // Y is rewritten by the next item only after every CTA has read it (the
-    // remote loads have fed the stores above: the arrive needs no release)
-    cluster_arrive_relaxed();
-    cluster_wait_acquire();
-}
-
-// cart2d_batch4_kernel with the coils of every item split over a cluster of
-// CL CTAs (batches with fewer column items than resident CTAs).
-// grid CL * clusters, cluster (CL, 1, 1); the clusters walk the item list.
-__global__ void __launch_bounds__(192, 2)
-cart2d_batch4_cl_kernel(const SliceDesc* __restrict__ descs, const int2* __restrict__ items,
-                        int nitems, const float2* __restrict__ x, float2* out, float coef,
-                        const float2* operand, float alpha) {
-    __shared__ float2 tws[384];
-    __shared__ float pm[384];
-    __shared__ float2 Y[16 * 24 * 8];
-    extern __shared__ float4 sb4[];
-    float2* Sb = reinterpret_cast<float2*>(sb4);
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int q = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
-    const int cid = blockIdx.x / CL, ncid = gridDim.x / CL;
-    int cur = -1;
-    for (int it = cid; it < nitems; it += ncid) {
-        const int2 item = items[it];
-        const int s = item.x;
-        const SliceDesc D = descs[s];
-        if (s != cur) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < D.ny; i += blockDim.x) {
-                tws[i] = D.tw[i];
-                pm[i] = D.mask_fo[i];
-            }
-            __syncthreads();
-            cur = s;
-        }
-        const float2* xs = x + D.img_off;
-        float2* os = out + D.img_off;
-        const float2* ops = operand ? operand + D.img_off : nullptr;
-        const float sc = coef * D.invL;
-        switch (D.n2) {
-            case 8: batch_item_cl<8>(tws, pm, Y, Sb, D, item.y, xs, os, sc, ops, alpha, q, CL); break;
-            case 12: batch_item_cl<12>(tws, pm, Y, Sb, D, item.y, xs, os, sc, ops, alpha, q, CL); break;
-            case 16: batch_item_cl<16>(tws, pm, Y, Sb, D, item.y, xs, os, sc, ops, alpha, q, CL); break;
-            case 20: batch_item_cl<20>(tws, pm, Y, Sb, D, item.y, xs, os, sc, ops, alpha, q, CL); break;
-            default: batch_item_cl<24>(tws, pm, Y, Sb, D, item.y, xs, os, sc, ops, alpha, q, CL); break;
-        }
+    __syncthreads();
+    if (threadIdx.x <= D) {
+        double a = 0.0;
+        for (int w = 0; w < kThreads / 32; ++w) a += s[threadIdx.x][w];
+        r.partials[blockIdx.x * (D + 1) + threadIdx.x] = a;
     }
 }
 
-// cart2d_batch4_kernel for a batch whose slices all share one length
-// ny = 16 N2: a block of 8 * max(16, N2) threads (no idle threads for the
-// shorter lengths) and shared memory sized for that length, so more CTAs
-// fit an SM.
-template <int N2>
-__global__ void __launch_bounds__(8 * (N2 > 16 ? N2 : 16), N2 <= 16 ? 4 : 2)
-cart2d_batch4u_kernel(const SliceDesc* __restrict__ descs, const int2* __restrict__ items,
-                      int nitems, const float2* __restrict__ x, float2* out, float coef,
-                      const float2* operand, float alpha) {
-    constexpr int n = 16 * N2;
-    __shared__ float2 tws[n];
-    __shared__ float pm[n];
-    __shared__ float2 Y[16 * N2 * 8];
-    extern __shared__ float4 sb4[];   // 2 * n * 8 float2
-    float2* Sb = reinterpret_cast<float2*>(sb4);
-    int cur = -1;
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        const int2 item = items[it];
-        const int s = item.x;
-        const SliceDesc D = descs[s];
-        if (s != cur) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                tws[i] = D.tw[i];
-                pm[i] = D.mask_fo[i];
-            }
-            __syncthreads();
-            cur = s;
-        }
-        cart_item4<N2>(tws, pm, Y, Sb, x + D.img_off, D.sens, D.C, D.nx, item.y, out + D.img_off,
-                       coef * D.invL, operand ? operand + D.img_off : nullptr, alpha);
-    }
-}
-
-// The uniform-length kernel with each item's coils split over a cluster of
-// CL CTAs (batches with fewer items than resident CTAs: one pass over the
-// items instead of several coil-serial rounds).  grid CL * clusters.
-template <int N2>
-__global__ void __launch_bounds__(8 * (N2 > 16 ? N2 : 16), N2 <= 16 ? 4 : 2)
-cart2d_batch4u_cl_kernel(const SliceDesc* __restrict__ descs, const int2* __restrict__ items,
-                         int nitems, const float2* __restrict__ x, float2* out, float coef,
-                         const float2* operand, float alpha) {
-    constexpr int n = 16 * N2;
-    __shared__ float2 tws[n];
-    __shared__ float pm[n];
-    __shared__ float2 Y[16 * N2 * 8];
-    extern __shared__ float4 sb4[];
-    float2* Sb = reinterpret_cast<float2*>(sb4);
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int q = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
-    const int cid = blockIdx.x / CL, ncid = gridDim.x / CL;
-    int cur = -1;
-    for (int it = cid; it < nitems; it += ncid) {
-        const int2 item = items[it];
-        const int s = item.x;
-        const SliceDesc D = descs[s];
-        if (s != cur) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                tws[i] = D.tw[i];
-                pm[i] = D.mask_fo[i];
-            }
-            __syncthreads();
-            cur = s;
-        }
-        batch_item_cl<N2>(tws, pm, Y, Sb, D, item.y, x + D.img_off, out + D.img_off, coef * D.invL,
-                          operand ? operand + D.img_off : nullptr, alpha, q, CL);
-    }
+// dots[i] = sum of the blocks' partials, one warp each, in a fixed order
+__global__ void rev_dots_kernel(const double* __restrict__ partials, int nblocks, int nd,
+                                double* __restrict__ dots) {
+    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double a = 0.0;
+    for (int b = lane; b < nblocks; b += 32) a += partials[b * nd + i];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+    if (lane == 0) dots[i] = a;
 }
 
 }  // namespace
@@ -634,85 +482,35 @@ pp_status configure_batch_kernels() {
     return PP_OK;
 }
 
-constexpr size_t kBatch4Dyn = sizeof(float2) * 2 * 384 * 8;
 
 // Persistent grid of the uniform-length kernel (0 when n2 has none).
-int batch4u_grid(int n2) {
-    int occ = 0, nsm = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-#define PP_G4U(N2_)                                                                                \
-    if (n2 == N2_) {                                                                               \
-        const size_t dyn = sizeof(float2) * 2 * 16 * N2_ * 8;                                      \
-        cudaFuncSetAttribute(cart2d_batch4u_kernel<N2_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)dyn);                                                            \
-        cudaFuncSetAttribute(cart2d_batch4u_cl_kernel<N2_>,                                        \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);               \
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cart2d_batch4u_kernel<N2_>,        \
-                                                          8 * (N2_ > 16 ? N2_ : 16), dyn);         \
+pp_status launch_batch_chain(const BatchDev& b, const float2* x, const CartChain& ch, cudaStream_t st) {
+    // one launch per length; each after the first may start while its
+    // predecessor's last CTAs run (same input, other slices)
+    bool first = true;
+    for (const CartGroup& g : b.groups) {
+        CartLaunch L;
+        L.descs = b.descs;
+        L.items = g.items;
+        L.nitems = g.nitems;
+        L.W = g.W;
+        L.max_coils = g.max_coils;
+        L.pdl = L.follows = !first;
+        PP_TRY(launch_cart_cols(g.n, L, x, ch, st));
+        first = false;
     }
-    PP_G4U(8) PP_G4U(12) PP_G4U(16) PP_G4U(20) PP_G4U(24)
-#undef PP_G4U
-    if (e != cudaSuccess || occ < 1) {
-        cudaGetLastError();
-        return 0;
-    }
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess) nsm = 152;
-    return occ * nsm;
-}
-
-int batch4_grid() {
-    int occ = 0, nsm = 0;
-    cudaFuncSetAttribute(cart2d_batch4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kBatch4Dyn);
-    cudaFuncSetAttribute(cart2d_batch4_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kBatch4Dyn);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cart2d_batch4_kernel, 192, kBatch4Dyn) !=
-        cudaSuccess)
-        occ = 1;
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess) nsm = 152;
-    return std::max(1, occ) * nsm;
+    return PP_OK;
 }
 
 pp_status launch_batch_normal(const BatchDev& b, const float2* x, float2* out, float coef,
                               const float2* operand, float alpha, cudaStream_t st) {
-    if (b.fast4 && b.cl == 1 && b.un2) {
-        cudaError_t e = cudaErrorInvalidValue;
-#define PP_B4U(N2_)                                                                                \
-        if (b.un2 == N2_)                                                                          \
-            e = launch_ex(cart2d_batch4u_kernel<N2_>, dim3(std::min(b.ugrid, b.nitems)),           \
-                          dim3(8 * (N2_ > 16 ? N2_ : 16)), sizeof(float2) * 2 * 16 * N2_ * 8, st,  \
-                          false, 0, (const SliceDesc*)b.descs, (const int2*)b.items, b.nitems, x, \
-                          out, coef, operand, alpha);
-        PP_B4U(8) PP_B4U(12) PP_B4U(16) PP_B4U(20) PP_B4U(24)
-#undef PP_B4U
-        if (e != cudaSuccess) return cuda_status(e, "cart2d_batch4u_kernel launch");
-        return check_launch_b("cart2d_batch4u_kernel");
-    }
-    if (b.fast4 && b.cl > 1 && b.un2) {
-        const int ncl = std::max(1, std::min(b.ugrid / b.cl, b.nitems));
-        cudaError_t e = cudaErrorInvalidValue;
-#define PP_B4UC(N2_)                                                                               \
-        if (b.un2 == N2_)                                                                          \
-            e = launch_ex(cart2d_batch4u_cl_kernel<N2_>, dim3(ncl * b.cl),                          \
-                          dim3(8 * (N2_ > 16 ? N2_ : 16)), sizeof(float2) * 2 * 16 * N2_ * 8, st,  \
-                          false, b.cl, (const SliceDesc*)b.descs, (const int2*)b.items, b.nitems, \
-                          x, out, coef, operand, alpha);
-        PP_B4UC(8) PP_B4UC(12) PP_B4UC(16) PP_B4UC(20) PP_B4UC(24)
-#undef PP_B4UC
-        if (e != cudaSuccess) return cuda_status(e, "cart2d_batch4u_cl_kernel launch");
-        return check_launch_b("cart2d_batch4u_cl_kernel");
-    }
-    if (b.fast4 && b.cl > 1) {
-        const int ncl = std::max(1, std::min(b.grid / b.cl, b.nitems));
-        PP_TRY_CUDA(launch_ex(cart2d_batch4_cl_kernel, dim3(ncl * b.cl), dim3(192), kBatch4Dyn, st,
-                              false, b.cl, (const SliceDesc*)b.descs, (const int2*)b.items, b.nitems,
-                              x, out, coef, operand, alpha));
-        return check_launch_b("cart2d_batch4_cl_kernel");
-    }
-    if (b.fast4) {
-        cart2d_batch4_kernel<<<std::min(b.grid, b.nitems), 192, kBatch4Dyn, st>>>(
-            b.descs, b.items, b.nitems, x, out, coef, operand, alpha);
-        return check_launch_b("cart2d_batch4_kernel");
+    if (b.cols > 0) {
+        CartChain ch;
+        ch.sc[0] = coef;
+        ch.al[0] = alpha;
+        ch.ext = operand;
+        ch.out = out;
+        return launch_batch_chain(b, x, ch, st);
     }
     void* fn = batch_normal_fn(b.km, b.lgt);
     if (!fn) {
@@ -744,28 +542,37 @@ pp_status launch_seg_scale(const float2* in, float2* out, const Segments& sg, co
 }
 
 pp_status launch_batch_prox_fista(const BatchDev& b, float lam, float gamma, float beta,
-                                  float2* z, const float2* u, float2* y, const float2* ref,
+                                  float2* z, const float2* u, float2* y, float2* w_out, const float2* ref,
                                   double* hist, cudaStream_t st) {
-    batch_prox_fista_kernel<<<b.tiles.nblocks, kThreads, 0, st>>>(
-        b.descs, b.tiles.off, b.tiles.blk_seg, b.tiles.seg_first_blk, lam, gamma, beta, z, u, y, ref,
-        hist);
+    batch_prox_fista_kernel<<<b.tiles.nblocks, kTileThreads, 0, st>>>(
+        b.descs, b.tiles.off, b.tiles.blk_seg, b.tiles.seg_first_blk, lam, gamma, beta, z, u, y, w_out,
+        ref, hist);
     return check_launch_b("batch_prox_fista_kernel");
 }
 
 pp_status launch_batch_prox_vjp(const BatchDev& b, float lam, float beta, const float2* w,
                                 float2* Ybar, const float2* Zbar, float2* wbar, double* lam_bar,
                                 cudaStream_t st) {
-    batch_prox_vjp_kernel<<<b.tiles.nblocks, kThreads, 0, st>>>(
+    batch_prox_vjp_kernel<<<b.tiles.nblocks, kTileThreads, 0, st>>>(
         b.descs, b.tiles.off, b.tiles.blk_seg, b.tiles.seg_first_blk, lam, beta, w, Ybar, Zbar, wbar,
         lam_bar);
     return check_launch_b("batch_prox_vjp_kernel");
 }
 
-pp_status launch_lincomb(const LinComb& lc, float2* out, int64_t n, int accumulate, cudaStream_t st) {
-    int64_t blocks = (n + kThreads - 1) / kThreads;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    lincomb_kernel<<<(int)std::max<int64_t>(blocks, 1), kThreads, 0, st>>>(lc, out, n, accumulate);
-    return check_launch_b("lincomb_kernel");
+pp_status launch_rev_combine(const RevCombine& r, double* dots, cudaStream_t st) {
+    const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(kRevBlocks, (r.n + kThreads - 1) / kThreads));
+    switch (r.d) {
+#define PP_REV(D) case D: rev_combine_kernel<D><<<nblk, kThreads, 0, st>>>(r); break;
+        PP_REV(0) PP_REV(1) PP_REV(2) PP_REV(3) PP_REV(4) PP_REV(5) PP_REV(6) PP_REV(7) PP_REV(8) PP_REV(9)
+        PP_REV(10)
+#undef PP_REV
+        default:
+            set_error("unrolled solve: degree %d", r.d);
+            return PP_ERR_UNSUPPORTED;
+    }
+    PP_TRY(check_launch_b("rev_combine_kernel"));
+    rev_dots_kernel<<<1, 32 * (r.d + 1), 0, st>>>(r.partials, nblk, r.d + 1, dots);
+    return check_launch_b("rev_dots_kernel");
 }
 
 }  // namespace pp

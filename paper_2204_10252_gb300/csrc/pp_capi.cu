@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <atomic>
 #include <thread>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -87,6 +88,70 @@ static pp_status alloc_n(Plan& p, T** ptr, size_t n) {
     return dev_alloc(p, reinterpret_cast<void**>(ptr), n * sizeof(T));
 }
 
+// Mean of |w|^2 - 1 that the FP32 constants of a register DFT leave in its output
+// energy (pp_fft.cuh, pp_fft4.cuh, pp_fftgen.cuh): the radix kernels' own
+// constants, and the inner twiddles of a composite A * B.
+static double reg_dft_gain(int N) {
+    auto sq = [](double v) { const double f = (float)v; return f * f; };
+    if (N <= 2 || N == 4) return 0.0;
+    if (N == 3) return (3.0 + 2.0 * (1.0 + 2.0 * (0.25 + sq(sqrt(3.0) / 2.0)))) / 9.0 - 1.0;
+    if (N == 5) {
+        double e = 0.0;
+        for (int q = 1; q <= 2; ++q) e += sq(cos(2.0 * M_PI * q / 5.0)) + sq(sin(2.0 * M_PI * q / 5.0));
+        return (5.0 + 4.0 * (1.0 + 2.0 * e)) / 25.0 - 1.0;
+    }
+    if (N == 8) return 0.25 * (2.0 * sq(sqrt(0.5)) - 1.0);   // two of the eight inner products
+    static const int ab[][2] = {{3, 2}, {3, 3}, {5, 2}, {4, 3}, {5, 3}, {4, 4}, {9, 2}, {4, 5}, {8, 3}, {5, 5}, {9, 3}, {10, 3}, {8, 4}};
+    for (const auto& f : ab) {
+        const int A = f[0], B = f[1];
+        if (A * B != N) continue;
+        double g = 0.0;
+        for (int b = 0; b < B; ++b)
+            for (int k = 0; k < A; ++k)
+                g += sq(cos(2.0 * M_PI * b * k / N)) + sq(sin(2.0 * M_PI * b * k / N)) - 1.0;
+        return reg_dft_gain(A) + reg_dft_gain(B) + g / N;
+    }
+    return 0.0;
+}
+
+// Twiddles of the two-factor kernels (n = n1 n2, W_n^(m2 k1)).  Rounding them and
+// the register DFTs' constants to FP32 changes the transform's mean output energy
+// by some 5e-8, always the same way, so that it adds up over the transforms of a
+// solve where rounding does not.  The table is scaled by the one factor that
+// brings the mean to 1 - 1e-8 (bisection: entries round one by one), the value at
+// which the coefficient gradients of a 3-iteration unrolled solve, which are
+// differences of large sums, were least off their 64-bit values: 6e-7 relative on
+// eight 256 x 256 slices, 9e-7 at a mean of 1 and 2e-6 with the plain table.
+static std::vector<float2> balanced_twiddles(int n) {
+    const GenSplit g = gen_split_of(n);
+    if (!g.n1) return {};
+    const double reg = reg_dft_gain(g.n1) + reg_dft_gain(g.n2);
+    auto table = [&](double scale) {
+        std::vector<float2> tw(n);
+        for (int t = 0; t < n; ++t) {
+            const double a = -2.0 * M_PI * (double)t / (double)n;
+            tw[t] = make_float2((float)(scale * cos(a)), (float)(scale * sin(a)));
+        }
+        tw[0] = make_float2(1.f, 0.f);
+        return tw;
+    };
+    auto gain = [&](const std::vector<float2>& tw) {
+        double e = 0.0;
+        for (int m = 0; m < g.n2; ++m)
+            for (int k = 0; k < g.n1; ++k) {
+                const float2 w = tw[m * k];
+                e += (double)w.x * w.x + (double)w.y * w.y - 1.0;
+            }
+        return reg + e / n;
+    };
+    double lo = 1.0 - 5e-7, hi = 1.0 + 5e-7;
+    for (int it = 0; it < 20; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        (gain(table(mid)) > -1e-8 ? hi : lo) = mid;
+    }
+    return table(0.5 * (lo + hi));
+}
+
 static pp_status make_fft(Plan& p, int n, DevFft& f) {
     if (!factorize(n, f.d)) {
         set_error("FFT length %d has a prime factor above 5", n);
@@ -99,6 +164,12 @@ static pp_status make_fft(Plan& p, int n, DevFft& f) {
     }
     PP_TRY(alloc_n(p, &f.tw, n));
     PP_TRY_CUDA(cudaMemcpy(f.tw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
+    const std::vector<float2> twb = balanced_twiddles(n);
+    f.twb = f.tw;
+    if (!twb.empty()) {
+        PP_TRY(alloc_n(p, &f.twb, n));
+        PP_TRY_CUDA(cudaMemcpy(f.twb, twb.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
+    }
     return PP_OK;
 }
 
@@ -185,13 +256,43 @@ static RowArgs row_args(int n, int G, int off_in, int off_out, int nrows, int64_
 // its FFT stages).
 static bool use_ci(const Plan& p) { return !p.toep && p.tune_stencil_kind >= 7 && p.ci_sens && p.ci_a; }
 
+// A chain of normal-operator applications in one launch (2-D Cartesian plans
+// whose ny has a column-resident kernel).
+static pp_status cart_chain(const Plan& p, const float2* x, const CartChain& ch, cudaStream_t st) {
+    CartLaunch L;
+    L.one.twb = p.fy.twb; L.one.sens = p.sens; L.one.mask_fo = p.mask_fo;
+    L.one.ny = p.ny; L.one.nx = p.nx; L.one.C = p.C; L.one.img_off = 0; L.one.invL = 1.f;
+    L.max_coils = p.C;
+    L.W = p.tune_c2;
+    while (L.W > 1 && !cart_cols_width_ok(p.ny, L.W)) L.W >>= 1;
+    L.pdl = p.pdl != 0;
+    return launch_cart_cols(p.ny, L, x, ch, st);
+}
+
+// Appends the Horner recursion (Listing "pcode") u = c_d v, u = c_i v + N u to a
+// chain, d >= 1; coefficients in units of the operator times `invL`.
+static void chain_horner(CartChain& ch, const double* c, int d, double invL) {
+    for (int i = d - 1; i >= 0; --i) {
+        ch.sc[ch.J] = (float)(i == d - 1 ? c[d] * invL : invL);
+        ch.al[ch.J] = (float)c[i];
+        ++ch.J;
+    }
+}
+
 // out = scale * (A^H A x) + alpha * operand   (operand may be NULL)
 static pp_status normal_into(const Plan& p, const float2* x, float2* out, float scale,
                              const float2* operand, float alpha, cudaStream_t st) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int64_t n = p.nimg;
-    if (p.kind == PP_CARTESIAN && p.ndim == 2)
-        return launch_cart2d_normal(p, x, out, scale, operand, alpha, st);
+    if (p.kind == PP_CARTESIAN && p.ndim == 2) {
+        if (!p.cols) return launch_cart2d_normal(p, x, out, scale, operand, alpha, st);
+        CartChain ch;
+        ch.sc[0] = scale;
+        ch.al[0] = alpha;
+        ch.ext = operand;
+        ch.out = out;
+        return cart_chain(p, x, ch, st);
+    }
     if (p.kind == PP_CARTESIAN) {
         if (p.tune_c3 == 1 && p.c3cl_clusters > 0)
             return c3cl_normal(p, 4, x, out, scale, operand, alpha, st);
@@ -202,7 +303,7 @@ static pp_status normal_into(const Plan& p, const float2* x, float2* out, float 
         bool done = false;
         PP_TRY(cart3d4_normal(p, x, out, scale, operand, alpha, p.wk_a, st, &done));
         if (done) return PP_OK;
-        PP_TRY(gen_cart3d_normal(p, x, out, scale, operand, alpha, p.wk_a, p.c3_chunk, st, &done));
+        PP_TRY(lines_cart3d_normal(p, x, out, scale, operand, alpha, p.wk_a, p.c3_chunk, st, &done));
         if (done) return PP_OK;
         // 3-D: per coil, y FFT -> (z FFT, mask, z IFFT) -> y IFFT -> conj accumulate
         for (int c = 0; c < p.C; ++c) {
@@ -740,30 +841,34 @@ static pp_status tune_cart3d(Plan& p, cudaStream_t st) {
     return PP_OK;
 }
 
-// 2-D Cartesian: one CTA per 8-column group against the coils split over a
-// cluster of 2, 4 or 8 CTAs per group (narrow images leave most SMs idle
-// otherwise), timed on the plan's buffers; the fastest is kept.
+// 2-D Cartesian: the columns per CTA of the column-resident kernel, timed on the
+// plan's buffers as one application and as a chain of three (a preconditioned
+// gradient of degree 2); the fastest sum is kept.
 static pp_status tune_cart2d(Plan& p, cudaStream_t st) {
-    if (!fft4_n2(p.ny)) return PP_OK;
+    p.cols = cart_cols_width_ok(p.ny, 1);
+    if (!p.cols) return PP_OK;   // the Stockham kernel
     cudaEvent_t e0, e1;
     PP_TRY_CUDA(cudaEventCreate(&e0));
     PP_TRY_CUDA(cudaEventCreate(&e1));
     PP_TRY_CUDA(cudaMemsetAsync(p.v, 0, sizeof(float2) * (size_t)p.nimg, st));
-    std::vector<int> cand = {1};
-    for (int cl : {2, 4, 8})
-        if (cl <= p.C) cand.push_back(cl);
+    std::vector<int> cand;
+    for (int w : {1, 2, 4, 8})
+        if (cart_cols_width_ok(p.ny, w)) cand.push_back(w);
     std::vector<float> best(cand.size(), 1e30f);
+    CartChain three;
+    three.out = p.t;
+    three.v_first = 1;
+    three.J = 3;
+    for (int j = 0; j < 3; ++j) three.sc[j] = three.al[j] = 1.f;
     for (int round = 0; round < 3; ++round)
         for (size_t i = 0; i < cand.size(); ++i) {
             p.tune_c2 = cand[i];
-            if (best[i] > 1.5e30f) continue;
-            if (!launches_ok([&]() { return normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st); })) {
-                best[i] = 2e30f;
-                continue;
-            }
             PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
             PP_TRY_CUDA(cudaEventRecord(e0, st));
-            for (int r = 0; r < 10; ++r) PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
+            for (int r = 0; r < 5; ++r) {
+                PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
+                PP_TRY(cart_chain(p, p.v, three, st));
+            }
             PP_TRY_CUDA(cudaEventRecord(e1, st));
             PP_TRY_CUDA(cudaEventSynchronize(e1));
             float ms = 0.f;
@@ -878,6 +983,14 @@ static pp_status horner_into(const Plan& p, const double* c, int d, const float2
                              float2* bufA, float2* bufB, cudaStream_t st) {
     const float invL = (float)(1.0 / p.L);
     if (d == 0) return launch_axpby(v, (float)c[0], nullptr, 0.f, out, p.nimg, st);
+    if (p.cols) {
+        CartChain ch;
+        ch.J = 0;
+        ch.v_first = 1;
+        ch.out = out;
+        chain_horner(ch, c, d, 1.0 / p.L);
+        return cart_chain(p, v, ch, st);
+    }
     const float2* cur = v;
     float scale = (float)(c[d] / p.L);
     for (int i = d - 1; i >= 0; --i) {
@@ -901,8 +1014,23 @@ static pp_status fista_iterations(Plan& p, float lambda, int iters, const double
                                   int levels, bool hist, const float2* ref, bool momentum,
                                   int wavelet, cudaStream_t st, Shift sh = Shift()) {
     const float invL = (float)(1.0 / p.L);
+    const bool chain = p.cols && c && d >= 1;
     for (int k = 0; k < iters; ++k) {
-        if (sh.on) {
+        if (chain) {
+            // gradient and preconditioner in one launch
+            CartChain ch;
+            ch.sc[0] = sh.on ? sh.a * invL : invL;
+            ch.al[0] = sh.on ? 1.f : -1.f;
+            ch.ext = p.ahb;
+            if (sh.on) {
+                PP_TRY(launch_axpby(p.z, sh.b, p.ahb, -1.f, p.t, p.nimg, st));
+                ch.ext = p.t;
+            }
+            ch.first_out = p.g;
+            ch.out = p.u;
+            chain_horner(ch, c, d, 1.0 / p.L);
+            PP_TRY(cart_chain(p, p.z, ch, st));
+        } else if (sh.on) {
             // g = (a N_hat + b I) z - rhs: u = b z - rhs, then g = a N_hat z + u
             PP_TRY(launch_axpby(p.z, sh.b, p.ahb, -1.f, p.u, p.nimg, st));
             PP_TRY(normal_into(p, p.z, p.g, sh.a * invL, p.u, 1.f, st));
@@ -912,7 +1040,9 @@ static pp_status fista_iterations(Plan& p, float lambda, int iters, const double
         }
         const float2* u = p.g;
         float gamma = 1.f;
-        if (c && d >= 1) {
+        if (chain) {
+            u = p.u;
+        } else if (c && d >= 1) {
             PP_TRY(horner_into(p, c, d, p.g, p.u, p.t, p.w3, st));
             u = p.u;
         } else if (c) {
@@ -950,13 +1080,15 @@ struct Batch {
     cudaGraphExec_t gexec = nullptr;
     std::vector<double> gkey;
     int64_t graph_kernels = 0;
-    int uni_n2 = 0;   // common N2 of all slices when the uniform-length kernel applies, else 0
     // differentiable unrolled solve: arena of image vectors and FP64 slots
     float2* arena = nullptr;
     size_t arena_vecs = 0;
     double* dslots = nullptr;
     size_t dslots_n = 0;
     std::vector<double> tape_key;
+    // forward and adjoint stages of the whole batch (empty: slice by slice)
+    std::vector<LineGroup> fwd_rows, fwd_cols;
+    std::vector<AdjointChunk> adj;
 };
 
 template <class T>
@@ -977,6 +1109,107 @@ template <class T>
 static pp_status bupload(Batch& b, T** dst, const std::vector<T>& src) {
     PP_TRY(balloc(b, dst, src.size()));
     PP_TRY_CUDA(cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice));
+    return PP_OK;
+}
+
+// Forward and adjoint stages over the whole batch: one launch per distinct length
+// (the slices one after another leave most SMs idle: eight 256 x 256 slices of 16
+// coils took 215 us forward and 310 us adjoint that way).  The adjoint's column
+// stage writes `wk` elements of workspace at most, so it runs in chunks of slices.
+// Skipped (empty lists) when some length has no compiled stage.
+template <class Item>
+static pp_status add_group(Batch& b, std::vector<LineGroup>& to, LineGroup g, std::vector<Item>& items) {
+    for (size_t i = 0; i < items.size(); i += 65535) {   // the batch index is blockIdx.y
+        const std::vector<Item> part(items.begin() + i, items.begin() + std::min(items.size(), i + 65535));
+        Item* p = nullptr;
+        PP_TRY(bupload(b, &p, part));
+        g.items = p;
+        g.nitems = (int)part.size();
+        to.push_back(g);
+    }
+    return PP_OK;
+}
+static pp_status plan_lines(Batch& b, size_t wk) {
+    for (const Plan* p : b.sub)
+        if (!lines_have(p->nx) || !lines_have(p->ny) || p->nx > 512) return PP_OK;
+    struct Cols { LineGroup g; std::vector<ColItem> items; };
+    struct Rows { LineGroup g; std::vector<RowItem> items; };
+    auto cols_of = [&](std::map<int, Cols>& m, const Plan& p, int64_t src, int64_t dst) {
+        Cols& c = m[p.ny];
+        c.g.n = p.ny;
+        c.g.tw = p.fy.twb;
+        c.g.extent = std::max(c.g.extent, p.nx);
+        for (int q = 0; q < p.C; ++q)
+            c.items.push_back({src + q * p.nimg, dst + q * p.nimg, p.mask_c, p.nx, (float)(1.0 / sqrt((double)p.ny))});
+    };
+    std::map<int, Cols> fc;
+    std::map<int, Rows> fr;
+    for (int s = 0; s < b.n; ++s) {
+        const Plan& p = *b.sub[s];
+        Rows& r = fr[p.nx];
+        r.g.n = p.nx;
+        r.g.tw = p.fx.twb;
+        r.g.extent = std::max(r.g.extent, p.ny);
+        for (int q = 0; q < p.C; ++q)
+            r.items.push_back({b.img_off[s], b.ksp_off[s] + q * p.nimg, p.sens + q * p.nimg, p.ny, 1, 1.f});
+        cols_of(fc, p, b.ksp_off[s], b.ksp_off[s]);
+    }
+    for (auto& e : fr) PP_TRY(add_group(b, b.fwd_rows, e.second.g, e.second.items));
+    for (auto& e : fc) PP_TRY(add_group(b, b.fwd_cols, e.second.g, e.second.items));
+    for (int s0 = 0; s0 < b.n;) {
+        std::map<int, Cols> ac;
+        std::map<int, Rows> ar;
+        int64_t used = 0;
+        int s = s0;
+        for (; s < b.n && (s == s0 || used + b.sub[s]->nksp <= (int64_t)wk); ++s) {
+            const Plan& p = *b.sub[s];
+            cols_of(ac, p, b.ksp_off[s], used);
+            Rows& r = ar[p.nx];
+            r.g.n = p.nx;
+            r.g.tw = p.fx.twb;
+            r.g.extent = std::max(r.g.extent, p.ny);
+            r.g.ncoils = std::max(r.g.ncoils, p.C);
+            r.items.push_back({used, b.img_off[s], p.sens, p.ny, p.C, 1.f});
+            used += p.nksp;
+        }
+        s0 = s;
+        AdjointChunk c;
+        for (auto& e : ac) PP_TRY(add_group(b, c.cols, e.second.g, e.second.items));
+        for (auto& e : ar) PP_TRY(add_group(b, c.rows, e.second.g, e.second.items));
+        b.adj.push_back(c);
+    }
+    return PP_OK;
+}
+
+static pp_status batch_cols(const std::vector<LineGroup>& gs, bool inv, const float2* src, float2* dst, cudaStream_t st) {
+    for (const LineGroup& g : gs)
+        PP_TRY(launch_lines_batch_cols(g.n, g.tw, g.extent, (const ColItem*)g.items, g.nitems, inv, src, dst, st));
+    return PP_OK;
+}
+static pp_status batch_rows(const std::vector<LineGroup>& gs, bool adj, const float2* src, float2* dst, cudaStream_t st) {
+    for (const LineGroup& g : gs)
+        PP_TRY(launch_lines_batch_rows(g.n, g.tw, g.extent, (const RowItem*)g.items, g.nitems, adj, g.ncoils,
+                                       (float)(1.0 / sqrt((double)g.n)), src, dst, st));
+    return PP_OK;
+}
+// y_s = A_s x_s and x_s = A_s^H y_s for every slice (unscaled)
+static pp_status batch_forward(const Batch& b, const float2* x, float2* y, cudaStream_t st) {
+    if (!b.fwd_rows.empty()) {
+        PP_TRY(batch_rows(b.fwd_rows, false, x, y, st));
+        return batch_cols(b.fwd_cols, false, y, y, st);
+    }
+    for (int s = 0; s < b.n; ++s) PP_TRY(forward_into(*b.sub[s], x + b.img_off[s], y + b.ksp_off[s], st));
+    return PP_OK;
+}
+static pp_status batch_adjoint(const Batch& b, const float2* y, float2* x, cudaStream_t st) {
+    if (!b.adj.empty()) {
+        for (const AdjointChunk& c : b.adj) {
+            PP_TRY(batch_cols(c.cols, true, y, b.wk, st));
+            PP_TRY(batch_rows(c.rows, true, b.wk, x, st));
+        }
+        return PP_OK;
+    }
+    for (int s = 0; s < b.n; ++s) PP_TRY(adjoint_into(*b.sub[s], y + b.ksp_off[s], x + b.img_off[s], st));
     return PP_OK;
 }
 
@@ -1053,69 +1286,101 @@ static pp_status upload_descs(Batch& b) {
     return PP_OK;
 }
 
-// Column-tile autotuner: time each feasible tile width on the batch itself
-// and keep the fastest.
+// Work lists of the column-resident kernels, W columns per CTA (fewer for a
+// length without that form): one list per distinct slice length, longest first.
+// False when some length has no such kernel.
+static bool cols_supported(const Batch& b) {
+    for (const SliceDesc& d : b.hdesc)
+        if (!cart_cols_width_ok(d.ny, 1)) return false;
+    return !b.hdesc.empty();
+}
+static void drop_groups(Batch& b) {
+    for (CartGroup& g : b.dev.groups)
+        if (g.items) {
+            cudaFree(g.items);
+            b.allocs.erase(std::remove(b.allocs.begin(), b.allocs.end(), (void*)g.items), b.allocs.end());
+        }
+    b.dev.groups.clear();
+    b.dev.cols = 0;
+}
+static pp_status set_cols(Batch& b, int W) {
+    drop_groups(b);
+    std::map<int, std::vector<std::pair<int, int2>>, std::greater<int>> by_len;
+    std::map<int, CartGroup> info;
+    for (int s = 0; s < b.n; ++s) {
+        const SliceDesc& d = b.hdesc[s];
+        CartGroup& g = info[d.ny];
+        g.n = d.ny;
+        g.W = W;
+        while (g.W > 1 && !cart_cols_width_ok(d.ny, g.W)) g.W >>= 1;
+        g.max_coils = std::max(g.max_coils, d.C);
+        for (int c0 = 0; c0 < d.nx; c0 += g.W) by_len[d.ny].push_back({d.C, make_int2(s, c0)});
+    }
+    int total = 0;
+    for (auto& e : by_len) {
+        std::stable_sort(e.second.begin(), e.second.end(),
+                         [](const std::pair<int, int2>& a, const std::pair<int, int2>& c) {
+                             return a.first > c.first;
+                         });
+        std::vector<int2> items;
+        for (auto& it : e.second) items.push_back(it.second);
+        CartGroup g = info[e.first];
+        g.nitems = (int)items.size();
+        total += g.nitems;
+        PP_TRY(bupload(b, &g.items, items));
+        b.dev.groups.push_back(g);
+    }
+    b.dev.cols = W;
+    b.dev.grid = total;
+    return PP_OK;
+}
+
+// Batch autotuner: the columns per CTA of the column-resident kernels (one
+// application and a chain of three, as for a single plan) where every slice
+// length has one, else the tile width of the Stockham kernel.
 static pp_status autotune(Batch& b, cudaStream_t st) {
     std::vector<int2> items;
-    int best = -1, best_cl = 1;
+    int best = -1;
     float best_ms = 1e30f;
     cudaEvent_t e0, e1;
     PP_TRY_CUDA(cudaEventCreate(&e0));
     PP_TRY_CUDA(cudaEventCreate(&e1));
-    bool all_fast = true;
-    for (const SliceDesc& d : b.hdesc) all_fast = all_fast && d.n2 != 0;
-    // candidates: Stockham kernels with 4, 8 or 16 columns per item (lgt 2..4)
-    // and, when every slice length has one, the register four-step kernel (5)
-    // with 1, 2 or 4 CTAs per item (coils split over a cluster)
-    for (int lgt = 2; lgt <= 5; ++lgt)
-        for (int cl : {1, 2, 4}) {
-            if (lgt < 5 && cl > 1) continue;
-            if (lgt == 5) {
-                if (!all_fast) continue;
-                PP_TRY(set_items(b, 3, &items));
-                b.dev.fast4 = 1;
-                b.dev.cl = cl;
-                b.dev.un2 = b.uni_n2;
-                b.dev.grid = batch4_grid();
-            } else {
-                if (!km_for(b.dev.ny_max, lgt)) continue;
-                b.dev.fast4 = 0;
-                b.dev.cl = 1;
-                b.dev.un2 = 0;
-                PP_TRY(set_items(b, lgt, &items));
-            }
-            if (!launches_ok([&]() { return launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st); }))
-                continue;   // a cluster shape this device cannot place
-            PP_TRY_CUDA(cudaEventRecord(e0, st));
-            for (int r = 0; r < 3; ++r) PP_TRY(launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st));
-            PP_TRY_CUDA(cudaEventRecord(e1, st));
-            PP_TRY_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = lgt;
-                best_cl = cl;
-            }
+    const bool cols = cols_supported(b);
+    CartChain three;
+    three.out = b.t;
+    three.v_first = 1;
+    three.J = 3;
+    for (int j = 0; j < 3; ++j) three.sc[j] = three.al[j] = 1.f;
+    for (int v : cols ? std::vector<int>{1, 4, 8} : std::vector<int>{2, 3, 4}) {
+        if (cols) {
+            PP_TRY(set_cols(b, v));
+        } else {
+            if (!km_for(b.dev.ny_max, v)) continue;
+            PP_TRY(set_items(b, v, &items));
         }
+        auto pass = [&]() {
+            PP_TRY(launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st));
+            return cols ? launch_batch_chain(b.dev, b.v, three, st) : PP_OK;
+        };
+        PP_TRY(pass());
+        PP_TRY_CUDA(cudaEventRecord(e0, st));
+        for (int r = 0; r < 3; ++r) PP_TRY(pass());
+        PP_TRY_CUDA(cudaEventRecord(e1, st));
+        PP_TRY_CUDA(cudaEventSynchronize(e1));
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms < best_ms) {
+            best_ms = ms;
+            best = v;
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (best < 0) {
         set_error("no batched kernel fits ny_max = %d", b.dev.ny_max);
         return PP_ERR_UNSUPPORTED;
     }
-    if (best == 5) {
-        PP_TRY(set_items(b, 3, &items));
-        b.dev.fast4 = 1;
-        b.dev.cl = best_cl;
-        b.dev.un2 = b.uni_n2;
-        b.dev.grid = batch4_grid();
-        return PP_OK;
-    }
-    b.dev.fast4 = 0;
-    b.dev.cl = 1;
-    b.dev.un2 = 0;
-    return set_items(b, best, &items);
+    return cols ? set_cols(b, best) : set_items(b, best, &items);
 }
 
 static pp_status batch_power_iteration(Batch& b, uint64_t seed, int iters, cudaStream_t st) {
@@ -1144,6 +1409,14 @@ static pp_status batch_power_iteration(Batch& b, uint64_t seed, int iters, cudaS
 static pp_status batch_horner(Batch& b, const double* c, int d, const float2* v, float2* out,
                               cudaStream_t st) {
     if (d == 0) return launch_axpby(v, (float)c[0], nullptr, 0.f, out, b.nimg, st);
+    if (b.dev.cols > 0) {
+        CartChain ch;
+        ch.J = 0;
+        ch.v_first = 1;
+        ch.out = out;
+        chain_horner(ch, c, d, 1.0);
+        return launch_batch_chain(b.dev, v, ch, st);
+    }
     const float2* cur = v;
     float coef = (float)c[d];
     for (int i = d - 1; i >= 0; --i) {
@@ -1155,20 +1428,40 @@ static pp_status batch_horner(Batch& b, const double* c, int d, const float2* v,
     return PP_OK;
 }
 
+// u = p(N_hat) (N_hat z - ahb) in one launch per slice length, d >= 1; the
+// gradient itself into g
+static pp_status batch_gradient_chain(Batch& b, const double* c, int d, const float2* z,
+                                      const float2* ahb, float2* g, float2* u, cudaStream_t st) {
+    CartChain ch;
+    ch.sc[0] = 1.f;
+    ch.al[0] = -1.f;
+    ch.ext = ahb;
+    ch.first_out = g;
+    ch.out = u;
+    chain_horner(ch, c, d, 1.0);
+    return launch_batch_chain(b.dev, z, ch, st);
+}
+
 static pp_status batch_iterations(Batch& b, float lambda, int iters, const double* c, int d,
                                   bool hist, const float2* ref, bool momentum, cudaStream_t st) {
     for (int k = 0; k < iters; ++k) {
-        PP_TRY(launch_batch_normal(b.dev, b.z, b.g, 1.f, b.ahb, -1.f, st));
         const float2* u = b.g;
         float gamma = 1.f;
-        if (c && d >= 1) {
+        if (b.dev.cols > 0 && c && d >= 1) {
+            PP_TRY(batch_gradient_chain(b, c, d, b.z, b.ahb, b.g, b.u, st));
+            u = b.u;
+        } else {
+            PP_TRY(launch_batch_normal(b.dev, b.z, b.g, 1.f, b.ahb, -1.f, st));
+        }
+        if (u == b.u) {
+        } else if (c && d >= 1) {
             PP_TRY(batch_horner(b, c, d, b.g, b.u, st));
             u = b.u;
         } else if (c) {
             gamma = (float)c[0];
         }
         const float beta = momentum ? (float)((double)k / (k + 3.0)) : 0.f;
-        PP_TRY(launch_batch_prox_fista(b.dev, lambda, gamma, beta, b.z, u, b.y, hist ? ref : nullptr,
+        PP_TRY(launch_batch_prox_fista(b.dev, lambda, gamma, beta, b.z, u, b.y, nullptr, hist ? ref : nullptr,
                                        hist ? b.hist + 3 * k : nullptr, st));
     }
     return PP_OK;
@@ -1218,25 +1511,21 @@ static size_t unrolled_vecs(int iters, int ce, int d) {
 static pp_status unrolled_step(Batch& b, const double* c, int d, float lambda, int k, float2* z,
                                float2* y, float2* g_out, float2* w_out, cudaStream_t st) {
     const float2* ahb = avec(b, 0);
-    PP_TRY(launch_batch_normal(b.dev, z, g_out, 1.f, ahb, -1.f, st));
-    PP_TRY(batch_horner(b, c, d, g_out, b.u, st));
-    if (w_out) {
-        LinComb lc;
-        lc.count = 2;
-        lc.v[0] = z; lc.coef[0] = 1.f;
-        lc.v[1] = b.u; lc.coef[1] = -1.f;
-        PP_TRY(launch_lincomb(lc, w_out, b.nimg, 0, st));
+    if (b.dev.cols > 0 && d >= 1) {
+        PP_TRY(batch_gradient_chain(b, c, d, z, ahb, g_out, b.u, st));
+    } else {
+        PP_TRY(launch_batch_normal(b.dev, z, g_out, 1.f, ahb, -1.f, st));
+        PP_TRY(batch_horner(b, c, d, g_out, b.u, st));
     }
     const float beta = (float)((double)k / (k + 3.0));
-    return launch_batch_prox_fista(b.dev, lambda, 1.f, beta, z, b.u, y, nullptr, nullptr, st);
+    return launch_batch_prox_fista(b.dev, lambda, 1.f, beta, z, b.u, y, w_out, nullptr, nullptr, st);
 }
 
 static pp_status unrolled_forward(Batch& b, const float2* bk, float lambda, int iters,
                                   const double* c, int d, int ce, float2* x_out, cudaStream_t st) {
-    PP_TRY(ensure_arena(b, unrolled_vecs(iters, ce, d), (size_t)iters * (d + 1) + 1));
+    PP_TRY(ensure_arena(b, unrolled_vecs(iters, ce, d), 1 + (size_t)(iters + kRevBlocks) * (d + 1)));
     float2* ahb = avec(b, 0);
-    for (int s = 0; s < b.n; ++s)
-        PP_TRY(adjoint_into(*b.sub[s], bk + b.ksp_off[s], ahb + b.img_off[s], st));
+    PP_TRY(batch_adjoint(b, bk, ahb, st));
     PP_TRY(launch_seg_scale(ahb, ahb, b.dev.img, nullptr, 0, b.dfac, 0, st));
     PP_TRY_CUDA(cudaMemsetAsync(b.y, 0, b.nimg * sizeof(float2), st));
     PP_TRY_CUDA(cudaMemsetAsync(b.z, 0, b.nimg * sizeof(float2), st));
@@ -1269,12 +1558,11 @@ static pp_status unrolled_backward(Batch& b, float lambda, int iters, const doub
     PP_TRY_CUDA(cudaMemsetAsync(b.dslots, 0, sizeof(double) * (1 + (size_t)iters * (d + 1)), st));
     for (int sg = (int)ncp - 1; sg >= 0; --sg) {
         const int k0 = sg * ce, k1 = std::min(iters, k0 + ce);
-        // recompute the segment forward from its checkpoint, keeping z_k, g_k, w_k
+        // recompute the segment forward from its checkpoint, keeping g_k, w_k
         PP_TRY_CUDA(cudaMemcpyAsync(yw, avec(b, 1 + 2 * sg), bytes, cudaMemcpyDeviceToDevice, st));
         PP_TRY_CUDA(cudaMemcpyAsync(zw, avec(b, 2 + 2 * sg), bytes, cudaMemcpyDeviceToDevice, st));
         for (int k = k0; k < k1; ++k) {
             const int j = k - k0;
-            PP_TRY_CUDA(cudaMemcpyAsync(avec(b, seg0 + 3 * j), zw, bytes, cudaMemcpyDeviceToDevice, st));
             PP_TRY(unrolled_step(b, c, d, lambda, k, zw, yw, avec(b, seg0 + 3 * j + 1),
                                  avec(b, seg0 + 3 * j + 2), st));
         }
@@ -1284,33 +1572,40 @@ static pp_status unrolled_backward(Batch& b, float lambda, int iters, const doub
             PP_TRY(launch_batch_prox_vjp(b.dev, lambda, beta, avec(b, seg0 + 3 * j + 2), Ybar, Zbar,
                                          wbar, lam_bar, st));
             // v_0 = wbar, v_i = N_hat v_{i-1}, i = 1..d+1
-            const float2* prev = wbar;
-            for (int i = 1; i <= d + 1; ++i) {
-                PP_TRY(launch_batch_normal(b.dev, prev, avec(b, v0 + i), 1.f, nullptr, 0.f, st));
-                prev = avec(b, v0 + i);
+            if (b.dev.cols > 0) {
+                CartChain ch;
+                ch.J = d + 1;
+                for (int i = 0; i <= d; ++i) {
+                    ch.sc[i] = 1.f;
+                    ch.al[i] = 0.f;
+                }
+                ch.all_out = avec(b, v0 + 1);
+                ch.all_stride = b.nimg;
+                PP_TRY(launch_batch_chain(b.dev, wbar, ch, st));
+            } else {
+                const float2* prev = wbar;
+                for (int i = 1; i <= d + 1; ++i) {
+                    PP_TRY(launch_batch_normal(b.dev, prev, avec(b, v0 + i), 1.f, nullptr, 0.f, st));
+                    prev = avec(b, v0 + i);
+                }
             }
             const float2* gk = avec(b, seg0 + 3 * j + 1);
-            for (int i = 0; i <= d; ++i)
-                PP_TRY(launch_dot(i == 0 ? wbar : avec(b, v0 + i), gk, b.nimg, b.partials,
-                                  b.dev.img.nblocks, dots + (size_t)k * (d + 1) + i, nullptr, st));
-            // Zbar = wbar - sum_i c_i v_{i+1};  ahb_bar += sum_i c_i v_i
-            LinComb za, ab;
-            za.count = d + 2;
-            za.v[0] = wbar; za.coef[0] = 1.f;
-            ab.count = d + 1;
-            for (int i = 0; i <= d; ++i) {
-                za.v[i + 1] = avec(b, v0 + i + 1);
-                za.coef[i + 1] = -(float)c[i];
-                ab.v[i] = (i == 0) ? wbar : avec(b, v0 + i);
-                ab.coef[i] = (float)c[i];
-            }
-            PP_TRY(launch_lincomb(za, Zbar, b.nimg, 0, st));
-            PP_TRY(launch_lincomb(ab, ahb_bar, b.nimg, 1, st));
+            // dots_i = Re<v_i, g_k>;  Zbar = wbar - sum_i c_i v_{i+1};  ahb_bar += sum_i c_i v_i
+            RevCombine rc;
+            rc.d = d;
+            for (int i = 0; i <= d; ++i) rc.c[i] = (float)c[i];
+            rc.wbar = wbar;
+            rc.v = avec(b, v0 + 1);
+            rc.n = b.nimg;
+            rc.g = gk;
+            rc.Zbar = Zbar;
+            rc.ahb_bar = ahb_bar;
+            rc.partials = b.dslots + 1 + (size_t)iters * (d + 1);
+            PP_TRY(launch_rev_combine(rc, dots + (size_t)k * (d + 1), st));
         }
     }
     // b_bar = A_s ahb_bar_s / sqrt(L_s)
-    for (int s = 0; s < b.n; ++s)
-        PP_TRY(forward_into(*b.sub[s], ahb_bar + b.img_off[s], grad_b + b.ksp_off[s], st));
+    PP_TRY(batch_forward(b, ahb_bar, grad_b, st));
     PP_TRY(launch_seg_scale(grad_b, grad_b, b.dev.ksp, nullptr, 0, b.dfac, 0, st));
     std::vector<double> h(1 + (size_t)iters * (d + 1));
     PP_TRY_CUDA(cudaMemcpyAsync(h.data(), b.dslots, h.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1600,7 +1895,7 @@ pp_status pp_plan_create(pp_plan** out, pp_dims dims, int coils, const pp_c64* s
     cudaGetDevice(&p.dev);
     cudaStream_t st = (cudaStream_t)stream;
     pp_status rc = (s->kind == PP_CARTESIAN) ? build_cartesian(p, s->mask) : build_noncartesian(p, s);
-    if (rc == PP_OK && s->kind == PP_CARTESIAN && p.ndim == 2) rc = prepare_cart4();
+    if (rc == PP_OK && s->kind == PP_CARTESIAN && p.ndim == 2) p.cols = cart_cols_width_ok(p.ny, 1);
     if (rc == PP_OK) {
         const size_t n = (size_t)p.nimg;
         p.red_blocks = 2 * 152;
@@ -2297,14 +2592,16 @@ pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, cons
         b.ksp_off[s + 1] = b.ksp_off[s] + p->nksp;
         b.tile_off[s + 1] = b.tile_off[s] + p->nimg / 16;
         SliceDesc& d = b.hdesc[s];
-        d.fd = p->fy.d; d.tw = p->fy.tw; d.sens = p->sens; d.mask_fo = p->mask_fo;
-        d.ny = p->ny; d.nx = p->nx; d.C = p->C; d.n2 = fft4_n2(p->ny); d.img_off = b.img_off[s];
-        d.invL = 1.f; d.pad1 = 0.f;
+        d.fd = p->fy.d; d.tw = p->fy.tw; d.twb = p->fy.twb; d.sens = p->sens; d.mask_fo = p->mask_fo;
+        d.ny = p->ny; d.nx = p->nx; d.C = p->C; d.img_off = b.img_off[s];
+        d.invL = 1.f;
         b.dev.ny_max = std::max(b.dev.ny_max, p->ny);
     }
     b.nimg = b.img_off[nslices];
     b.nksp = b.ksp_off[nslices];
-    if (rc == PP_OK) rc = balloc(b, &b.wk, wk_max);
+    // adjoint workspace: the largest slice, and more of them up to half of the L2
+    const size_t wk = std::max(wk_max, std::min((size_t)b.nksp, (size_t)(72 << 20) / sizeof(float2)));
+    if (rc == PP_OK) rc = balloc(b, &b.wk, wk);
     if (rc == PP_OK)
         for (Plan* p : b.sub) p->wk_a = b.wk;
     const size_t n = (size_t)b.nimg;
@@ -2317,7 +2614,7 @@ pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, cons
         (rc = balloc(b, &b.dev.descs, (size_t)nslices)) == PP_OK &&
         (rc = make_segments(b, b.dev.img, b.img_off, (int64_t)kThreads * 8, 64)) == PP_OK &&
         (rc = make_segments(b, b.dev.ksp, b.ksp_off, (int64_t)kThreads * 8, 64)) == PP_OK &&
-        (rc = make_segments(b, b.dev.tiles, b.tile_off, (int64_t)kThreads, 1 << 30)) == PP_OK) {
+        (rc = make_segments(b, b.dev.tiles, b.tile_off, kTileThreads / 4, 1 << 30)) == PP_OK) {
         const int nb = std::max(b.dev.img.nblocks, b.dev.ksp.nblocks);
         rc = balloc(b, &b.partials, (size_t)3 * nb);
     }
@@ -2330,14 +2627,7 @@ pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, cons
         cudaError_t e = cudaMemsetAsync(b.v, 0, n * sizeof(float2), st);
         if (e != cudaSuccess) rc = cuda_status(e, "cudaMemsetAsync");
     }
-    if (rc == PP_OK) {
-        // a batch of one slice length can run the uniform-length kernel
-        int un2 = b.hdesc.empty() ? 0 : b.hdesc[0].n2;
-        for (const SliceDesc& d : b.hdesc)
-            if (d.n2 != un2) un2 = 0;
-        b.dev.ugrid = un2 ? batch4u_grid(un2) : 0;
-        b.uni_n2 = b.dev.ugrid > 0 ? un2 : 0;
-    }
+    if (rc == PP_OK) rc = plan_lines(b, wk);
     if (rc == PP_OK) rc = autotune(b, st);
     if (rc == PP_OK && power_iters > 0) rc = batch_power_iteration(b, seed, power_iters, st);
     if (rc != PP_OK) {
@@ -2417,7 +2707,10 @@ pp_status pp_batch_tile(const pp_batch* batch, int* cols_per_cta, int* persisten
         return PP_ERR_INVALID_ARG;
     }
     if (cols_per_cta)
-        *cols_per_cta = batch->impl.dev.fast4 ? -8 * batch->impl.dev.cl : 1 << batch->impl.dev.lgt;
+        {
+        const int w = batch->impl.dev.cols;
+        *cols_per_cta = w ? (w == 8 ? -8 : (w == 1 ? -16 : -32)) : 1 << batch->impl.dev.lgt;
+    }
     if (persistent_ctas) *persistent_ctas = batch->impl.dev.grid;
     return PP_OK;
 }
@@ -2431,24 +2724,18 @@ pp_status pp_batch_set_tile(pp_batch* batch, int cols_per_cta) {
     std::vector<int2> items;
     if (cols_per_cta == -8 || cols_per_cta == -16 || cols_per_cta == -32) {
         for (const SliceDesc& d : b.hdesc)
-            if (!d.n2) {
+            if (!cart_cols_width_ok(d.ny, 1)) {
                 set_error("pp_batch_set_tile: slice length %d has no register FFT kernel", d.ny);
                 return PP_ERR_UNSUPPORTED;
             }
-        PP_TRY(set_items(b, 3, &items));
-        b.dev.fast4 = 1;
-        b.dev.cl = -cols_per_cta / 8;
-        b.dev.un2 = b.uni_n2;
-        b.dev.grid = batch4_grid();
+        PP_TRY(set_cols(b, cols_per_cta == -8 ? 8 : (cols_per_cta == -16 ? 1 : 4)));
     } else {
-        b.dev.cl = 1;
-        b.dev.un2 = 0;
         const int lgt = cols_per_cta == 4 ? 2 : cols_per_cta == 8 ? 3 : cols_per_cta == 16 ? 4 : -1;
         if (lgt < 0 || !km_for(b.dev.ny_max, lgt)) {
             set_error("pp_batch_set_tile: unsupported tile width %d", cols_per_cta);
             return PP_ERR_UNSUPPORTED;
         }
-        b.dev.fast4 = 0;
+        drop_groups(b);
         PP_TRY(set_items(b, lgt, &items));
     }
     b.gkey.clear();
@@ -2461,11 +2748,8 @@ pp_status pp_batch_forward_apply(const pp_batch* batch, const pp_c64* x, pp_c64*
         set_error("pp_batch_forward_apply: NULL argument");
         return PP_ERR_INVALID_ARG;
     }
-    const Batch& b = batch->impl;
-    for (int s = 0; s < b.n; ++s)
-        PP_TRY(forward_into(*b.sub[s], reinterpret_cast<const float2*>(x) + b.img_off[s],
-                            reinterpret_cast<float2*>(y) + b.ksp_off[s], (cudaStream_t)stream));
-    return PP_OK;
+    return batch_forward(batch->impl, reinterpret_cast<const float2*>(x), reinterpret_cast<float2*>(y),
+                         (cudaStream_t)stream);
 }
 
 pp_status pp_batch_adjoint_apply(const pp_batch* batch, const pp_c64* y, pp_c64* x, pp_stream stream) {
@@ -2473,11 +2757,8 @@ pp_status pp_batch_adjoint_apply(const pp_batch* batch, const pp_c64* y, pp_c64*
         set_error("pp_batch_adjoint_apply: NULL argument");
         return PP_ERR_INVALID_ARG;
     }
-    const Batch& b = batch->impl;
-    for (int s = 0; s < b.n; ++s)
-        PP_TRY(adjoint_into(*b.sub[s], reinterpret_cast<const float2*>(y) + b.ksp_off[s],
-                            reinterpret_cast<float2*>(x) + b.img_off[s], (cudaStream_t)stream));
-    return PP_OK;
+    return batch_adjoint(batch->impl, reinterpret_cast<const float2*>(y), reinterpret_cast<float2*>(x),
+                         (cudaStream_t)stream);
 }
 
 pp_status pp_batch_normal_apply(const pp_batch* batch, const pp_c64* x, pp_c64* y, pp_stream stream) {
@@ -2515,8 +2796,7 @@ pp_status pp_batch_fista_solve(pp_batch* batch, const pp_c64* bk, float lambda, 
     const int64_t launches0 = g_launches;
     const float2* bd = reinterpret_cast<const float2*>(bk);
     PP_TRY(launch_seg_dot(nullptr, bd, b.dev.ksp, b.partials, nullptr, b.scal + 0, 4, st));
-    for (int s = 0; s < b.n; ++s)
-        PP_TRY(adjoint_into(*b.sub[s], bd + b.ksp_off[s], b.ahb + b.img_off[s], st));
+    PP_TRY(batch_adjoint(b, bd, b.ahb, st));
     PP_TRY(launch_seg_scale(b.ahb, b.ahb, b.dev.img, b.scal + 0, 4, b.dfac, 1, st));
     PP_TRY_CUDA(cudaMemsetAsync(b.y, 0, b.nimg * sizeof(float2), st));
     PP_TRY_CUDA(cudaMemsetAsync(b.z, 0, b.nimg * sizeof(float2), st));
@@ -2537,7 +2817,7 @@ pp_status pp_batch_fista_solve(pp_batch* batch, const pp_c64* bk, float lambda, 
     if (iters > 0) {
         std::vector<double> key = {(double)iters, (double)d, (double)lambda, hist ? 1.0 : 0.0,
                                    c ? 1.0 : 0.0, (double)(uintptr_t)b.hist, (double)(uintptr_t)ref,
-                                   (double)b.dev.lgt, (double)b.dev.fast4, momentum ? 1.0 : 0.0};
+                                   (double)b.dev.lgt, (double)b.dev.cols, momentum ? 1.0 : 0.0};
         if (c)
             for (int i = 0; i <= d; ++i) key.push_back(c[i]);
         if (!b.gexec || key != b.gkey) {

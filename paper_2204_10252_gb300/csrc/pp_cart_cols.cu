@@ -1,0 +1,66 @@
+// Choice and launch of the column-resident Cartesian kernels (pp_cart_cols.cuh).
+#include <algorithm>
+
+#include "pp_cart_cols.cuh"
+
+namespace pp {
+
+namespace {
+
+struct Len {
+    int n, n1, n2;
+};
+#define PP_LEN_ROW(n, a, b) {n, a, b},
+const Len kLens[] = {PP_CART_A(PP_LEN_ROW) PP_CART_B(PP_LEN_ROW) PP_CART_C(PP_LEN_ROW) PP_CART_D(PP_LEN_ROW)};
+#undef PP_LEN_ROW
+
+const Len* find(int n) {
+    for (const Len& l : kLens)
+        if (l.n == n) return &l;
+    return nullptr;
+}
+
+size_t smem_of(const Len& l, int W, int NB) {
+    const size_t n = l.n;
+    return sizeof(float2) * (n + n / 2 + 2 * n * W + (size_t)l.n1 * (l.n2 | 1) * 8 * W + (size_t)NB * n * 8 * W);
+}
+
+}  // namespace
+
+bool cart_cols_width_ok(int n, int W) {
+    const Len* l = find(n);
+    if (!l || !cart_width_ok(n, W)) return false;
+    return W == 8 || smem_of(*l, W, 2) <= (size_t)kCartSmem;
+}
+
+pp_status launch_cart_cols(int n, CartLaunch L, const float2* x, const CartChain& ch, cudaStream_t st) {
+    const Len* l = find(n);
+    // The maps of all coil groups stay in shared memory for a chain of several
+    // applications while every CTA that an SM would run then (its share of the
+    // grid, four at most) still fits; otherwise they stream through two buffers.
+    const int groups = (L.max_coils + 7) / 8;
+    const int grid = L.items ? L.nitems : (L.one.nx + L.W - 1) / L.W;
+    const int per_sm = std::min(4, (grid + 151) / 152);
+    L.resident = groups <= 2 || (ch.J > 1 && l && per_sm * (smem_of(*l, L.W, groups) + 1024) <= (size_t)kCartSmem);
+    // Streaming: as many slots as bring 16 warps to every SM (what 128 registers a
+    // thread allow), while two or more coils are left to each.
+    if (l && L.W == 8) {
+        const int ctas = L.items ? L.nitems : (L.one.nx + 7) / 8;
+        while (L.slots < 4 && ctas * L.slots * 8 * l->n2 < 152 * 512 && L.max_coils >= 4 * L.slots) L.slots *= 2;
+    }
+    cudaError_t e = cudaErrorInvalidValue;
+    if (l) {
+        e = cart_cols_launch_a(n, L, x, ch, st);
+        if (e == cudaErrorInvalidValue) e = cart_cols_launch_b(n, L, x, ch, st);
+        if (e == cudaErrorInvalidValue) e = cart_cols_launch_c(n, L, x, ch, st);
+        if (e == cudaErrorInvalidValue) e = cart_cols_launch_d(n, L, x, ch, st);
+    }
+    if (e != cudaSuccess) return cuda_status(e, "cart_cols_kernel launch");
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_status(e, "cart_cols_kernel");
+    ++g_launches;
+    if (g_profiler) g_profiler->mark("cart_cols_kernel");
+    return PP_OK;
+}
+
+}  // namespace pp

@@ -120,6 +120,20 @@ __device__ __forceinline__ void fft4_phase1(float2* v, int m2, const float2* __r
     }
 }
 
+// The same with every twiddle from the table: the products of the form above
+// leave up to three more roundings in them.  One more shared-memory read per
+// element, so not where shared memory bounds the kernel.
+template <int N1, int N2, bool INV>
+__device__ __forceinline__ void fft4_phase1_exact(float2* v, int m2, const float2* __restrict__ tw) {
+    RegFft<N1, INV>::run(v, tw, N2);
+#pragma unroll
+    for (int k1 = 1; k1 < N1; ++k1) {
+        float2 ww = tw[m2 * k1];
+        if (INV) ww.y = -ww.y;
+        v[k1] = cmul(v[k1], ww);
+    }
+}
+
 // Phase 2 for one (transform, k1): u holds Y[k1][m2], m2 < N2; on exit
 // u[k2] = X[k1 + N1 k2].
 template <int N1, int N2, bool INV>
@@ -143,140 +157,6 @@ __device__ __forceinline__ void cluster_arrive_relaxed() {
 }
 __device__ __forceinline__ void cluster_wait_acquire() {
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-
-// 16-byte asynchronous global -> shared copy, zero-filled when !valid.
-__device__ __forceinline__ void cpa16(void* smem, const void* gmem, bool valid) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem),
-                 "r"(valid ? 16 : 0)
-                 : "memory");
-}
-
-// Stage the n x 8 tile S[0..n)[col0 .. col0+8) of one coil map (row pitch
-// nx, nx even) into dst[row * 8 + j] with cp.async and commit it as one group;
-// columns at or past nx read as zero.
-template <int N2>
-__device__ __forceinline__ void stage_s_tile(float2* dst, const float2* __restrict__ S, int nx,
-                                             int col0) {
-    constexpr int n = 16 * N2;
-    for (int e = threadIdx.x; e < n * 4; e += blockDim.x) {
-        const int row = e >> 2, q = e & 3, c = col0 + 2 * q;
-        const bool ok = c < nx;
-        cpa16(dst + row * 8 + 2 * q, S + (ok ? (int64_t)row * nx + c : 0), ok);
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-
-// Coil loop of the fused Cartesian item for coils c_first, c_first + c_step,
-// ... < C: acc[m1] (rows N2 m1 + r of column col0 + lane, threads r < N2)
-// accumulates conj(S_c) F^H (mask_fo . F (S_c x)).  Ends with a barrier.
-template <int N2>
-__device__ __forceinline__ void cart_item4_acc(const float2* __restrict__ tws,
-                                               const float* __restrict__ pm, float2* Y, float2* Sb,
-                                               const float2* __restrict__ x,
-                                               const float2* __restrict__ sens, int C, int nx,
-                                               int col0, int c_first, int c_step, float2* acc) {
-    constexpr int N1 = 16, n = N1 * N2;
-    const int lane = threadIdx.x & 7, r = threadIdx.x >> 3, col = col0 + lane;
-    const bool colok = col < nx;
-    const bool p1 = r < N2, p2 = r < N1;
-    const int64_t cs = (int64_t)n * nx;
-    float2 xr[N1];
-#pragma unroll
-    for (int m1 = 0; m1 < N1; ++m1) acc[m1] = make_float2(0.f, 0.f);
-    if (c_first >= C) {
-        __syncthreads();
-        return;
-    }
-    stage_s_tile<N2>(Sb, sens + c_first * cs, nx, col0);
-#pragma unroll
-    for (int m1 = 0; m1 < N1; ++m1)
-        xr[m1] = (p1 && colok) ? x[(int64_t)(N2 * m1 + r) * nx + col] : make_float2(0.f, 0.f);
-    int it = 0;
-    for (int c = c_first; c < C; c += c_step, ++it) {
-        const float2* St = Sb + (it & 1) * n * 8;
-        // the other buffer was last read in the previous coil, before its final barrier
-        if (c + c_step < C)
-            stage_s_tile<N2>(Sb + ((it + 1) & 1) * n * 8, sens + (c + c_step) * cs, nx, col0);
-        else
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
-        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        __syncthreads();
-        if (p1) {
-            float2 v[N1];
-#pragma unroll
-            for (int m1 = 0; m1 < N1; ++m1) v[m1] = cmul(St[(N2 * m1 + r) * 8 + lane], xr[m1]);
-            fft4_phase1<N1, N2, false>(v, r, tws);
-#pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) Y[(k1 * N2 + r) * 8 + lane] = v[k1];
-        }
-        __syncthreads();
-        if (p2) {
-            float2 u[N2];
-#pragma unroll
-            for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y[(r * N2 + m2) * 8 + lane];
-            fft4_phase2<N1, N2, false>(u, tws);
-#pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) u[k2] = cscale(u[k2], pm[r + N1 * k2]);
-            RegFft<N2, true>::run(u, tws, N1);
-#pragma unroll
-            for (int m2 = 1; m2 < N2; ++m2) {
-                float2 w = tws[m2 * r];
-                w.y = -w.y;
-                u[m2] = cmul(u[m2], w);
-            }
-#pragma unroll
-            for (int m2 = 0; m2 < N2; ++m2) Y[(r * N2 + m2) * 8 + lane] = u[m2];
-        }
-        __syncthreads();
-        if (p1) {
-            float2 v[N1];
-#pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1) v[k1] = Y[(k1 * N2 + r) * 8 + lane];
-            RegFft<N1, true>::run(v, tws, N2);
-#pragma unroll
-            for (int m1 = 0; m1 < N1; ++m1)
-                acc[m1] = cadd(acc[m1], cmulc(St[(N2 * m1 + r) * 8 + lane], v[m1]));
-        }
-        __syncthreads();
-    }
-}
-
-// Fused Cartesian normal-operator work item on the four-step FFT:
-//   out[:, col] = sc * sum_c conj(S_c) F^H (mask_fo . F (S_c x)) + alpha * operand
-// for TXF = 8 columns col0.. of an ny x nx image, ny = 16 * N2, transform
-// along y.  Forward: phase 1 by (m2, col) threads, phase 2 by (k1, col)
-// threads, which then hold X[k1 + 16 k2].  Inverse, with the mirrored
-// decomposition (input k = k1 + 16 k2, output m = N2 m1 + m2):
-//   I1 (same (k1, col) threads): inverse length-N2 DFT over k2, times
-//      W_n^(-m2 k1);   I2 ((m2, col) threads): inverse length-16 DFT over k1,
-// which leaves x'[N2 m1 + m2] with the thread that loaded S_c at those rows.
-// The coil maps' n x 8 tiles are double-buffered in shared memory: coil
-// c + 1's tile streams in by cp.async while coil c is transformed.
-// Shared memory: tws[n] twiddles, pm[n] mask (FFT order, 1/ny folded in),
-// Y[16 * N2 * 8], Sb[2 * n * 8].  Threads: 8 * max(16, N2); all threads
-// must call it.
-template <int N2>
-__device__ __forceinline__ void cart_item4(const float2* __restrict__ tws,
-                                           const float* __restrict__ pm, float2* Y, float2* Sb,
-                                           const float2* __restrict__ x,
-                                           const float2* __restrict__ sens, int C, int nx,
-                                           int col0, float2* out, float sc,
-                                           const float2* operand, float alpha) {
-    constexpr int N1 = 16;
-    const int lane = threadIdx.x & 7, r = threadIdx.x >> 3, col = col0 + lane;
-    float2 acc[N1];
-    cart_item4_acc<N2>(tws, pm, Y, Sb, x, sens, C, nx, col0, 0, 1, acc);
-    if (r < N2 && col < nx) {
-#pragma unroll
-        for (int m1 = 0; m1 < N1; ++m1) {
-            const int64_t o = (int64_t)(N2 * m1 + r) * nx + col;
-            float2 v = cscale(acc[m1], sc);
-            if (operand) v = cadd(v, cscale(operand[o], alpha));
-            out[o] = v;
-        }
-    }
 }
 
 }  // namespace pp

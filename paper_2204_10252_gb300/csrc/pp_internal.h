@@ -69,16 +69,33 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Raises a kernel's dynamic shared memory limit to `bytes`, once.
+template <auto Kernel, int bytes> cudaError_t allow_smem() {
+    static const cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+}
+
 // Device FFT: stage plan plus the table w^t = exp(-2 pi i t / n), t < n.
 struct DevFft {
     FftDesc d;
     float2* tw = nullptr;
+    float2* twb = nullptr;   // the same for the two-factor kernels, balanced (see make_fft)
 };
 
-// A transform length as the product of two register DFT lengths, n1 <= n2
-// (0: none), see pp_fftgen.cuh.
-struct GenSplit {
-    int n1 = 0, n2 = 0;
+// One batch of a stage over a batch's slices: offsets into the launch's source and
+// destination, and the slice's own sizes (rows: `sens` the coil's map, forward, or
+// the slice's first).
+struct ColItem {
+    int64_t src, dst;
+    const float* mask;     // centred, by transform row
+    int ncols;
+    float scale;
+};
+struct RowItem {
+    int64_t src, dst;
+    const float2* sens;
+    int nrows, ncoils;
+    float scale;
 };
 
 // Per-sample gridding metadata in trajectory order.
@@ -202,7 +219,8 @@ struct Plan {
     int tune_c3 = 0;            // 3-D: 0 = three passes per coil, 1 / 2 = one-kernel cluster operator
                                 //      with 4 / 2 columns per task
     int pdl = 1;                // programmatic dependent launch in the solve's kernel chain
-    int tune_c2 = 1;            // 2-D Cartesian: CTAs per 8-column group (coils split over a cluster)
+    bool cols = false;          // 2-D Cartesian: the column-resident kernels run (ny has one)
+    int tune_c2 = 1;            //   columns per CTA: 1, 2, 4 (fewer where not compiled), 8 streaming
     std::vector<void*> allocs;
 };
 
@@ -227,39 +245,41 @@ extern thread_local Profiler* g_profiler;
 pp_status configure_kernels();
 // register four-step FFT stages (pp_kernels4.cu); *done = false when the
 // transform length has no register kernel
-pp_status launch_cols4(const DevFft& f, const ColArgs& a, const float2* src, float2* dst, bool inv,
-                       cudaStream_t st, bool* done);
-pp_status launch_rows4_fwd(const DevFft& f, const RowArgs& a, const float2* x, const float2* sens,
-                           const float* wrow, const float* wcol, float2* out, int ncoils,
-                           int64_t img_batch_stride, cudaStream_t st, bool* done);
 pp_status launch_rows4_adj_split(const DevFft& f, const RowArgs& a, const float2* src,
                                  const float2* sens, const float* wrow, const float* wcol,
                                  float2* contrib, float2* out, const float2* operand, float alpha,
                                  int ncoils, cudaStream_t st, bool* done);
 pp_status cart3d4_normal(const Plan& p, const float2* x, float2* out, float scale,
                          const float2* operand, float alpha, float2* W, cudaStream_t st, bool* done);
-pp_status launch_cart2d4_normal(const Plan& p, const float2* x, float2* out, float scale,
-                                const float2* operand, float alpha, cudaStream_t st, bool* done);
 pp_status launch_rows4_adj(const DevFft& f, const RowArgs& a, const float2* src, const float2* sens,
                            const float* wrow, const float* wcol, float2* out, const float2* operand,
                            float alpha, int ncoils, cudaStream_t st, bool* done, int cluster = 0);
-// two-factor FFT stages for any supported length (pp_kernels_gen.cu); *done =
-// false when the length has no pair of register factors
+// row and column FFT stages of the compiled lengths (pp_lines.cu); *done = false
+// when the length has none
+bool lines_have(int n);
+// n as the product of its kernels' two register DFT lengths, n1 <= n2 (0: none)
+struct GenSplit {
+    int n1 = 0, n2 = 0;
+};
 GenSplit gen_split_of(int n);
-pp_status configure_gen_kernels();
-pp_status launch_gen_cols(const DevFft& f, const ColArgs& a, const float2* src, float2* dst, bool inv,
-                          const float2* ximg, int nimgs, cudaStream_t st, bool* done);
-pp_status launch_gen_roundtrip(const DevFft& f, const ColArgs& a, const float* mask_fo,
-                               const float2* src, float2* dst, cudaStream_t st, bool* done);
-pp_status launch_gen_rows_fwd(const DevFft& f, const RowArgs& a, const float2* x, const float2* sens,
-                              const float* wrow, const float* wcol, float2* out, int ncoils,
-                              int64_t img_batch_stride, cudaStream_t st, bool* done);
-pp_status launch_gen_rows_adj(const DevFft& f, const RowArgs& a, const float2* src, const float2* sens,
-                              const float* wrow, const float* wcol, float2* out, const float2* operand,
-                              float alpha, int ncoils, cudaStream_t st, bool* done);
-pp_status gen_cart3d_normal(const Plan& p, const float2* x, float2* out, float scale,
-                            const float2* operand, float alpha, float2* W, int chunk, cudaStream_t st,
-                            bool* done);
+pp_status launch_lines_cols(const DevFft& f, const ColArgs& a, const float2* src, float2* dst, bool inv,
+                            const float2* ximg, int nimgs, cudaStream_t st, bool* done);
+pp_status launch_lines_roundtrip(const DevFft& f, const ColArgs& a, const float* mask_fo,
+                                 const float2* src, float2* dst, cudaStream_t st, bool* done);
+pp_status launch_lines_rows_fwd(const DevFft& f, const RowArgs& a, const float2* x, const float2* sens,
+                                const float* wrow, const float* wcol, float2* out, int ncoils,
+                                int64_t img_batch_stride, cudaStream_t st, bool* done);
+pp_status launch_lines_rows_adj(const DevFft& f, const RowArgs& a, const float2* src, const float2* sens,
+                                const float* wrow, const float* wcol, float2* out, const float2* operand,
+                                float alpha, int ncoils, cudaStream_t st, bool* done);
+pp_status launch_lines_batch_cols(int n, const float2* tw, int ncols, const ColItem* items, int nitems,
+                                  bool inv, const float2* src, float2* dst, cudaStream_t st);
+pp_status launch_lines_batch_rows(int n, const float2* tw, int nrows, const RowItem* items, int nitems,
+                                  bool adj, int ncoils, float scale, const float2* src, float2* dst,
+                                  cudaStream_t st);
+pp_status lines_cart3d_normal(const Plan& p, const float2* x, float2* out, float scale,
+                              const float2* operand, float alpha, float2* W, int chunk, cudaStream_t st,
+                              bool* done);
 pp_status launch_rows_fwd(const Plan& p, const DevFft& f, const RowArgs& a, const float2* x,
                           const float2* sens, const float* wrow, const float* wcol, float2* out,
                           int ncoils, int64_t img_batch_stride, cudaStream_t st);
@@ -283,7 +303,6 @@ pp_status launch_nufft_spread(const Plan& p, const float2* ksp, float2* kt, floa
 pp_status launch_gtg_stencil(const Plan& p, const float2* grid_in, float2* grid_out, cudaStream_t st);
 pp_status prepare_gtg_stencil(Plan& p);
 pp_status build_gtg_device(Plan& p, cudaStream_t st);
-pp_status prepare_cart4();
 int c3cl_prepare(const Plan& p, int xb);
 int c3df_prepare(const Plan& p, int variant);
 bool c3df_make_tensor_map(Plan& p);

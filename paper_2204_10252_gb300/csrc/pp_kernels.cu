@@ -1320,7 +1320,6 @@ static size_t cols_smem(int G) { return sizeof(float2) * (size_t)(G + 2 * G * TX
 
 pp_status configure_kernels() {
     db4_prepare();
-    PP_TRY(configure_gen_kernels());
     const int big = 200 * 1024;
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
     PP_TRY_CUDA(cudaFuncSetAttribute(rows_adj_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big));
@@ -1344,9 +1343,7 @@ pp_status launch_rows_fwd(const Plan& p, const DevFft& f, const RowArgs& a, cons
                           int ncoils, int64_t img_batch_stride, cudaStream_t st) {
     (void)p;
     bool done = false;
-    PP_TRY(launch_rows4_fwd(f, a, x, sens, wrow, wcol, out, ncoils, img_batch_stride, st, &done));
-    if (done) return PP_OK;
-    PP_TRY(launch_gen_rows_fwd(f, a, x, sens, wrow, wcol, out, ncoils, img_batch_stride, st, &done));
+    PP_TRY(launch_lines_rows_fwd(f, a, x, sens, wrow, wcol, out, ncoils, img_batch_stride, st, &done));
     if (done) return PP_OK;
     dim3 grid((a.nrows + RB - 1) / RB, ncoils);
     rows_fwd_kernel<<<grid, kThreads, rows_smem(a.G), st>>>(f.d, f.tw, a, x, img_batch_stride, sens,
@@ -1366,7 +1363,7 @@ pp_status launch_rows_adj(const Plan& p, const DevFft& f, const RowArgs& a, cons
         set_error("row length %d exceeds the row stage limit", a.n);
         return PP_ERR_UNSUPPORTED;
     }
-    PP_TRY(launch_gen_rows_adj(f, a, src, sens, wrow, wcol, out, operand, alpha, ncoils, st, &done));
+    PP_TRY(launch_lines_rows_adj(f, a, src, sens, wrow, wcol, out, operand, alpha, ncoils, st, &done));
     if (done) return PP_OK;
     if (ncoils >= 4 && a.n <= 2 * kThreads) {
         const size_t smc = rows_smem(a.G);
@@ -1393,9 +1390,7 @@ pp_status launch_rows_adj(const Plan& p, const DevFft& f, const RowArgs& a, cons
 pp_status launch_cols(const DevFft& f, const ColArgs& a, const float2* src, float2* dst, bool inv,
                       cudaStream_t st) {
     bool done = false;
-    PP_TRY(launch_cols4(f, a, src, dst, inv, st, &done));
-    if (done) return PP_OK;
-    PP_TRY(launch_gen_cols(f, a, src, dst, inv, nullptr, 1, st, &done));
+    PP_TRY(launch_lines_cols(f, a, src, dst, inv, nullptr, 1, st, &done));
     if (done) return PP_OK;
     dim3 grid((a.ncols + TX - 1) / TX, a.nbatch);
     if (inv)
@@ -1408,7 +1403,7 @@ pp_status launch_cols(const DevFft& f, const ColArgs& a, const float2* src, floa
 pp_status launch_cols_roundtrip(const DevFft& f, const ColArgs& a, const float* mask_fo,
                                 const float2* src, float2* dst, cudaStream_t st) {
     bool done = false;
-    PP_TRY(launch_gen_roundtrip(f, a, mask_fo, src, dst, st, &done));
+    PP_TRY(launch_lines_roundtrip(f, a, mask_fo, src, dst, st, &done));
     if (done) return PP_OK;
     dim3 grid((a.ncols + TX - 1) / TX, a.nbatch);
     cols_roundtrip_kernel<<<grid, kThreads, cols_smem(a.G), st>>>(f.d, f.tw, a, mask_fo, src, dst);
@@ -1417,9 +1412,6 @@ pp_status launch_cols_roundtrip(const DevFft& f, const ColArgs& a, const float* 
 
 pp_status launch_cart2d_normal(const Plan& p, const float2* x, float2* out, float scale,
                                const float2* operand, float alpha, cudaStream_t st) {
-    bool done = false;
-    PP_TRY(launch_cart2d4_normal(p, x, out, scale, operand, alpha, st, &done));
-    if (done) return PP_OK;
     if (p.ny * TX > KMAX * kThreads) {
         set_error("ny = %d exceeds the fused Cartesian kernel limit", p.ny);
         return PP_ERR_UNSUPPORTED;

@@ -32,120 +32,6 @@ template <int N2, int TX> __host__ __device__ constexpr int c3_min_ctas() {
     return 65536 / (TX * tpr<N2>() * 80);
 }
 
-// Column stage: TXF adjacent columns of one batch, transform along rows.
-template <int N2, bool INV>
-__global__ void __launch_bounds__(TXF * tpr<N2>())
-cols4_kernel(const float2* __restrict__ tw, ColArgs a, const float2* src, float2* dst) {
-    constexpr int n = N1 * N2;
-    __shared__ float2 tws[n];
-    __shared__ float2 Y[N1 * N2 * TXF];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = tw[i];
-    const int col0 = blockIdx.x * TXF;
-    const float2* sb = src + (int64_t)blockIdx.y * a.in_batch_stride;
-    float2* db = dst + (int64_t)blockIdx.y * a.out_batch_stride;
-    const int lane = threadIdx.x & (TXF - 1);
-    const int r = threadIdx.x >> LGTXF;
-    const int col = col0 + lane;
-    __syncthreads();
-    if (r < N2) {
-        const int m2 = r;
-        float2 v[N1];
-#pragma unroll
-        for (int m1 = 0; m1 < N1; ++m1) {
-            const int p = N2 * m1 + m2;
-            int row = p + a.off_in;
-            if (row >= n) row -= n;
-            float2 x = make_float2(0.f, 0.f);
-            if (row < a.Hin && col < a.ncols) {
-                x = sb[(int64_t)row * a.ncols + col];
-                if (a.mul_in) x = cscale(x, a.mul_in[row * a.mi_q + (col / a.mi_cdiv) * a.mi_c]);
-            }
-            v[m1] = x;
-        }
-        fft4_phase1<N1, N2, INV>(v, m2, tws);
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) Y[((k1 * N2) + m2) * TXF + lane] = v[k1];
-    }
-    __syncthreads();
-    if (r < N1 && col < a.ncols) {
-        const int k1 = r;
-        float2 u[N2];
-#pragma unroll
-        for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y[((k1 * N2) + m2) * TXF + lane];
-        fft4_phase2<N1, N2, INV>(u, tws);
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-            const int k = k1 + N1 * k2;
-            int q = k + a.off_out;
-            if (q >= n) q -= n;
-            if (q < a.Hout) {
-                float s = a.scale;
-                if (a.mul_out) s *= a.mul_out[q * a.mo_q + (col / a.mo_cdiv) * a.mo_c];
-                db[(int64_t)q * a.ncols + col] = cscale(u[k2], s);
-            }
-        }
-    }
-}
-
-// Row stage image -> k rows (coil expansion, weights, circular placement).
-template <int N2>
-__global__ void __launch_bounds__(RBF * tpr<N2>(), row_min_ctas<N2>())
-rows4_fwd_kernel(const float2* __restrict__ tw, RowArgs a, const float2* __restrict__ x,
-                 int64_t x_batch_stride, const float2* __restrict__ sens,
-                 const float* __restrict__ wrow, const float* __restrict__ wcol,
-                 float2* __restrict__ out) {
-    constexpr int n = N1 * N2, T = tpr<N2>(), YS = N2 + 1;
-    __shared__ float2 tws[n];
-    __shared__ float2 Y[RBF * N1 * YS];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = tw[i];
-    __syncthreads();
-    const int b = threadIdx.x / T, r = threadIdx.x - (threadIdx.x / T) * T;
-    const int c = blockIdx.y;
-    const int row = blockIdx.x * RBF + b;
-    const bool live = row < a.nrows;
-    const float2* xc = x + (int64_t)c * x_batch_stride;
-    const float2* sc = sens ? sens + (int64_t)c * a.coil_img_stride : nullptr;
-    if (r < N2) {
-        const int m2 = r;
-        const float wr = (wrow && live) ? wrow[row] : 1.f;
-        float2 v[N1];
-#pragma unroll
-        for (int m1 = 0; m1 < N1; ++m1) {
-            const int p = N2 * m1 + m2;
-            int i = p + a.off_in;
-            if (i >= n) i -= n;
-            float2 val = make_float2(0.f, 0.f);
-            if (live && i < a.n) {
-                const int64_t o = (int64_t)row * a.n + i;
-                val = xc[o];
-                if (sc) val = cmul(val, sc[o]);
-                float w = a.scale * wr;
-                if (wcol) w *= wcol[i];
-                val = cscale(val, w);
-            }
-            v[m1] = val;
-        }
-        fft4_phase1<N1, N2, false>(v, m2, tws);
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) Y[(b * N1 + k1) * YS + m2] = v[k1];
-    }
-    __syncthreads();
-    if (r < N1 && live) {
-        const int k1 = r;
-        float2 u[N2];
-#pragma unroll
-        for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y[(b * N1 + k1) * YS + m2];
-        fft4_phase2<N1, N2, false>(u, tws);
-        float2* oc = out + ((int64_t)c * a.nrows + row) * n;
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) {
-            int q = k1 + N1 * k2 + a.off_out;
-            if (q >= n) q -= n;
-            oc[q] = u[k2];
-        }
-    }
-}
-
 // Row stage k rows -> image for many coils: one image row per CTA, the
 // transform batch runs over RBF coils at a time; conjugate-coil reduction
 // and axpy epilogue as rows_adj_cb_kernel.
@@ -180,7 +66,7 @@ rows4_adj_kernel(const float2* __restrict__ tw, RowArgs a, const float2* __restr
                 if (s >= n) s -= n;
                 v[m1] = (c < ncoils) ? src[((int64_t)c * a.nrows + row) * n + s] : make_float2(0.f, 0.f);
             }
-            fft4_phase1<N1, N2, true>(v, m2, tws);
+            fft4_phase1_exact<N1, N2, true>(v, m2, tws);
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) Y[(b * N1 + k1) * YS + m2] = v[k1];
         }
@@ -267,7 +153,7 @@ rows4_adj_cl_kernel(const float2* __restrict__ tw, RowArgs a, const float2* __re
                 if (s >= n) s -= n;
                 v[m1] = (c < ncoils) ? src[((int64_t)c * a.nrows + row) * n + s] : make_float2(0.f, 0.f);
             }
-            fft4_phase1<N1, N2, true>(v, m2, tws);
+            fft4_phase1_exact<N1, N2, true>(v, m2, tws);
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) Y[(b * N1 + k1) * YS + m2] = v[k1];
         }
@@ -353,7 +239,7 @@ rows4_inv_kernel(const float2* __restrict__ tw, RowArgs a, const float2* __restr
             if (sidx >= n) sidx -= n;
             v[m1] = live ? src[((int64_t)c * a.nrows + row) * n + sidx] : make_float2(0.f, 0.f);
         }
-        fft4_phase1<N1, N2, true>(v, r, tws);
+        fft4_phase1_exact<N1, N2, true>(v, r, tws);
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) Y[(b * N1 + k1) * YS + r] = v[k1];
     }
@@ -402,89 +288,6 @@ coil_sum_kernel(const float2* __restrict__ contrib, int C, int64_t n, float scal
         __syncthreads();
     }
 }
-
-// Fused 2-D Cartesian normal operator (one CTA per 8 columns, all coils);
-// dynamic shared memory: the double-buffered coil-map tiles, 2 * n * 8 float2.
-template <int N2>
-__global__ void __launch_bounds__(8 * tpr<N2>(), 2)
-cart2d4_normal_kernel(const float2* __restrict__ tw, const float2* __restrict__ x,
-                      const float2* __restrict__ sens, int C, int nx,
-                      const float* __restrict__ mask_fo, float2* out, float scale,
-                      const float2* operand, float alpha) {
-    constexpr int n = N1 * N2;
-    __shared__ float2 tws[n];
-    __shared__ float pm[n];
-    __shared__ float2 Y[N1 * N2 * 8];
-    extern __shared__ float4 sb4[];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        tws[i] = tw[i];
-        pm[i] = mask_fo[i];
-    }
-    __syncthreads();
-    cart_item4<N2>(tws, pm, Y, reinterpret_cast<float2*>(sb4), x, sens, C, nx, blockIdx.x * 8, out,
-                   scale, operand, alpha);
-}
-
-// The same with the coils split over a cluster of CL CTAs per 8-column
-// group (for images too narrow to fill the GPU with column groups alone):
-// CTA q takes coils q, q + CL, ...; the CL partial sums meet in distributed
-// shared memory, CTA q summing rows [q n / CL, (q + 1) n / CL) in rank order.
-// grid (CL * ceil(nx / 8)), cluster (CL, 1, 1).
-template <int N2>
-__global__ void __launch_bounds__(8 * tpr<N2>(), 2)
-cart2d4_cluster_kernel(const float2* __restrict__ tw, const float2* __restrict__ x,
-                       const float2* __restrict__ sens, int C, int nx,
-                       const float* __restrict__ mask_fo, float2* out, float scale,
-                       const float2* operand, float alpha) {
-    constexpr int n = N1 * N2;
-    __shared__ float2 tws[n];
-    __shared__ float pm[n];
-    __shared__ float2 Y[N1 * N2 * 8];
-    extern __shared__ float4 sb4[];
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int q = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
-    const int col0 = (int)(blockIdx.x / CL) * 8;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        tws[i] = tw[i];
-        pm[i] = mask_fo[i];
-    }
-    __syncthreads();
-    float2 acc[N1];
-    cart_item4_acc<N2>(tws, pm, Y, reinterpret_cast<float2*>(sb4), x, sens, C, nx, col0, q, CL, acc);
-    const int lane = threadIdx.x & 7, r = threadIdx.x >> 3;
-    if (r < N2) {
-#pragma unroll
-        for (int m1 = 0; m1 < N1; ++m1) Y[(N2 * m1 + r) * 8 + lane] = acc[m1];   // Y[row][lane]
-    }
-    // split barrier: publish the partials, load the first operand value of
-    // this CTA's rows (independent of the cluster) while the others arrive
-    cluster_arrive_release();
-    const int rpr = n / CL;
-    float2 op0 = make_float2(0.f, 0.f);
-    {
-        const int row = q * rpr + ((int)threadIdx.x >> 3), col = col0 + ((int)threadIdx.x & 7);
-        if (operand && (int)threadIdx.x < rpr * 8 && col < nx) op0 = operand[(int64_t)row * nx + col];
-    }
-    cluster_wait_acquire();
-    for (int idx = threadIdx.x; idx < rpr * 8; idx += blockDim.x) {
-        const int row = q * rpr + (idx >> 3), l = idx & 7, col = col0 + l;
-        float2 v = cluster.map_shared_rank(Y, 0)[row * 8 + l];
-        for (int b = 1; b < CL; ++b) v = cadd(v, cluster.map_shared_rank(Y, b)[row * 8 + l]);
-        if (col < nx) {
-            const int64_t o = (int64_t)row * nx + col;
-            v = cscale(v, scale);
-            if (operand) v = cadd(v, cscale(idx == (int)threadIdx.x ? op0 : operand[o], alpha));
-            out[o] = v;
-        }
-    }
-    // keep every CTA's partials alive until the others have read them (their
-    // remote loads have fed their stores: the arrive needs no release)
-    cluster_arrive_relaxed();
-    cluster_wait_acquire();
-}
-
-template <int N2> constexpr size_t cart4_dyn_smem() { return sizeof(float2) * 2 * 16 * N2 * 8; }
 
 // ---------------------------------------------------------------------------
 // 3-D Cartesian normal operator, x-block by x-block and coil by coil, with
@@ -637,42 +440,6 @@ static pp_status check4(const char* what) {
     return PP_OK;
 }
 
-// Returns PP_UNSUPPORTED-free status; *done = false when n has no fast kernel.
-pp_status launch_cols4(const DevFft& f, const ColArgs& a, const float2* src, float2* dst, bool inv,
-                       cudaStream_t st, bool* done) {
-    *done = false;
-    const int n2 = fft4_n2(a.G);
-    if (!n2) return PP_OK;
-    dim3 grid((a.ncols + TXF - 1) / TXF, a.nbatch);
-#define PP_C4(N2_)                                                                                 \
-    if (n2 == N2_) {                                                                               \
-        const int thr = TXF * tpr<N2_>();                                                          \
-        if (inv) cols4_kernel<N2_, true><<<grid, thr, 0, st>>>(f.tw, a, src, dst);                 \
-        else cols4_kernel<N2_, false><<<grid, thr, 0, st>>>(f.tw, a, src, dst);                    \
-    }
-    PP_C4(8) PP_C4(12) PP_C4(16) PP_C4(20) PP_C4(24)
-#undef PP_C4
-    *done = true;
-    return check4("cols4_kernel");
-}
-
-pp_status launch_rows4_fwd(const DevFft& f, const RowArgs& a, const float2* x, const float2* sens,
-                           const float* wrow, const float* wcol, float2* out, int ncoils,
-                           int64_t img_batch_stride, cudaStream_t st, bool* done) {
-    *done = false;
-    const int n2 = fft4_n2(a.G);
-    if (!n2) return PP_OK;
-    dim3 grid((a.nrows + RBF - 1) / RBF, ncoils);
-#define PP_R4(N2_)                                                                                  \
-    if (n2 == N2_)                                                                                  \
-        rows4_fwd_kernel<N2_><<<grid, RBF * tpr<N2_>(), 0, st>>>(f.tw, a, x, img_batch_stride, sens, \
-                                                                 wrow, wcol, out);
-    PP_R4(8) PP_R4(12) PP_R4(16) PP_R4(20) PP_R4(24)
-#undef PP_R4
-    *done = true;
-    return check4("rows4_fwd_kernel");
-}
-
 pp_status launch_rows4_adj(const DevFft& f, const RowArgs& a, const float2* src, const float2* sens,
                            const float* wrow, const float* wcol, float2* out, const float2* operand,
                            float alpha, int ncoils, cudaStream_t st, bool* done, int cluster) {
@@ -715,53 +482,6 @@ pp_status launch_rows4_adj(const DevFft& f, const RowArgs& a, const float2* src,
 #undef PP_A4
     *done = true;
     return check4("rows4_adj_kernel");
-}
-
-pp_status prepare_cart4() {
-#define PP_P4(N2_)                                                                                \
-    PP_TRY_CUDA(cudaFuncSetAttribute(cart2d4_normal_kernel<N2_>,                                  \
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,               \
-                                     (int)cart4_dyn_smem<N2_>()));
-    PP_P4(8) PP_P4(12) PP_P4(16) PP_P4(20) PP_P4(24)
-#undef PP_P4
-#define PP_P4C(N2_)                                                                               \
-    PP_TRY_CUDA(cudaFuncSetAttribute(cart2d4_cluster_kernel<N2_>,                                 \
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,               \
-                                     (int)cart4_dyn_smem<N2_>()));
-    PP_P4C(8) PP_P4C(12) PP_P4C(16) PP_P4C(20) PP_P4C(24)
-#undef PP_P4C
-    return PP_OK;
-}
-
-pp_status launch_cart2d4_normal(const Plan& p, const float2* x, float2* out, float scale,
-                                const float2* operand, float alpha, cudaStream_t st, bool* done) {
-    *done = false;
-    const int n2 = fft4_n2(p.ny);
-    if (!n2) return PP_OK;
-    const int grid = (p.nx + 7) / 8;
-    const int CL = p.tune_c2;
-    if (CL == 2 || CL == 4 || CL == 8) {
-        cudaError_t e = cudaSuccess;
-#define PP_K4C(N2_)                                                                              \
-        if (n2 == N2_)                                                                           \
-            e = launch_ex(cart2d4_cluster_kernel<N2_>, dim3(grid * CL), dim3(8 * tpr<N2_>()),    \
-                          cart4_dyn_smem<N2_>(), st, false, CL, (const float2*)p.fy.tw, x,       \
-                          (const float2*)p.sens, p.C, p.nx, (const float*)p.mask_fo, out, scale, \
-                          operand, alpha);
-        PP_K4C(8) PP_K4C(12) PP_K4C(16) PP_K4C(20) PP_K4C(24)
-#undef PP_K4C
-        if (e != cudaSuccess) return cuda_status(e, "cart2d4_cluster_kernel launch");
-        *done = true;
-        return check4("cart2d4_cluster_kernel");
-    }
-#define PP_K4(N2_)                                                                                 \
-    if (n2 == N2_)                                                                                 \
-        cart2d4_normal_kernel<N2_><<<grid, 8 * tpr<N2_>(), cart4_dyn_smem<N2_>(), st>>>(           \
-            p.fy.tw, x, p.sens, p.C, p.nx, p.mask_fo, out, scale, operand, alpha);
-    PP_K4(8) PP_K4(12) PP_K4(16) PP_K4(20) PP_K4(24)
-#undef PP_K4
-    *done = true;
-    return check4("cart2d4_normal_kernel");
 }
 
 template <int N2>

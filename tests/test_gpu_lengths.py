@@ -51,3 +51,60 @@ def test_cartesian_3d_lengths(pp, shape, coils):
         assert err(gy, O.cart_forward(x, sens, mask)) <= TOL_APPLY
         assert err(gx, O.cart_adjoint(y, sens, mask)) <= TOL_APPLY
         assert err(gn, O.cart_normal(x, sens, mask)) <= TOL_APPLY
+
+
+LENGTHS = [32, 36, 40, 48, 60, 64, 72, 80, 96, 100, 108, 120, 128, 144, 160, 180, 192, 200, 216, 240, 256, 288, 300, 320,
+           324, 360, 384, 400, 432, 480, 500, 512]
+
+
+@pytest.mark.parametrize("ny", LENGTHS)
+def test_column_resident_chain(pp, ny):
+    """Every compiled length of the column-resident operator, one application
+    and a Horner chain, with every width (a ragged last group), one to four coil
+    groups (maps resident and streamed)."""
+    import torch
+    nx, c = 12, [1.5, -2.0, 1.25]
+    for coils in (1 + ny % 8, 8, 27):
+        shape = (ny, nx)
+        sens = synth.coil_maps(shape, coils, 21)
+        mask = synth.line_mask(shape, 3, 6, 22)
+        x = synth.crandn(shape, 23)
+        nrm = lambda v: O.cart_normal(v, sens, mask) / 1.25  # noqa: E731
+        ref1, ref2 = nrm(x), O.horner_apply(c, nrm, x)
+        with pp.pp_plan_create(shape, coils, dev(sens), mask=mask, power_iters=0) as plan:
+            pp.pp_plan_set_scale(plan, 1.25)
+            out = torch.empty(shape, dtype=torch.complex64, device="cuda")
+            for w in (1, 2, 4, 8):
+                pp.pp_plan_set_tuning(plan, w, 0, 8)
+                pp.pp_normal_apply(plan, dev(x), out)
+                assert err(out, ref1) <= TOL_APPLY, (coils, w)
+                pp.pp_poly_apply(plan, c, 2, dev(x), out)
+                assert err(out, ref2) <= TOL_APPLY, (coils, w)
+
+
+@pytest.mark.parametrize("tile", [-8, -16, -32])
+def test_column_resident_batch_of_mixed_lengths(pp, tile):
+    """Slices of several lengths (one launch each, every launch after the first
+    beside its predecessor), one long enough for no 4-column form."""
+    import torch
+    shapes, coils = [(180, 20), (128, 12), (500, 8), (128, 36), (36, 16)], [5, 9, 3, 17, 8]
+    sens = [synth.coil_maps(s, c, 31 + i) for i, (s, c) in enumerate(zip(shapes, coils))]
+    masks = [synth.line_mask(s, 3, 6, 41 + i) for i, s in enumerate(shapes)]
+    b = pp.pp_batch_create(shapes, coils, [dev(s) for s in sens], masks, power_iters=0)
+    try:
+        pp.pp_batch_set_tile(b, tile)
+        assert pp.pp_batch_tile(b)[0] == tile
+        L = np.linspace(0.8, 1.4, len(shapes))
+        pp.pp_batch_set_scales(b, L)
+        xs = [synth.crandn(s, 51 + i) for i, s in enumerate(shapes)]
+        x = dev(np.concatenate([v.ravel() for v in xs]))
+        y = torch.empty_like(x)
+        for _ in range(3):
+            pp.pp_batch_normal_apply(b, x, y)
+        got = y.cpu().numpy().astype(np.complex128)
+        for i, s in enumerate(shapes):
+            ref = O.cart_normal(xs[i], sens[i], masks[i]) / L[i]
+            g = got[b.image_off[i]:b.image_off[i + 1]].reshape(s)
+            assert np.linalg.norm(g - ref) <= TOL_APPLY * np.linalg.norm(ref)
+    finally:
+        b.destroy()
