@@ -10,6 +10,7 @@ first call raises.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 from typing import Optional, Sequence
 
@@ -172,12 +173,12 @@ def _numel(t, n: int, what: str):
 
 
 def _img(plan, t, what):
-    _numel(t, int(np.prod(plan.shape)), what)
+    _numel(t, int(math.prod(plan.shape)), what)
     return _dev_ptr(t, what)
 
 
 def _ksp(plan, t, what):
-    _numel(t, int(np.prod(plan.kspace_shape)), what)
+    _numel(t, int(math.prod(plan.kspace_shape)), what)
     return _dev_ptr(t, what)
 
 
