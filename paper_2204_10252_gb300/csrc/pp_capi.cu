@@ -592,6 +592,21 @@ static pp_status build_noncartesian(Plan& p, const pp_sampling* s) {
             wy[j] = st[k].wy;
             kx[j] = make_int2(k, cell[k] % Gx);
         }
+        // the spread's 4 x 4 tiles by the samples that reach them, most first: the
+        // long ones of a trajectory start first, each in a CTA of its own
+        const int ntx = (Gx + 3) / 4, nty = (Gy + 3) / 4;
+        std::vector<int> count(ntx * nty), order(ntx * nty);
+        for (int t = 0; t < ntx * nty; ++t) {
+            const int ty = 4 * (t / ntx), tx = 4 * (t % ntx);
+            for (int y = ty - 3; y <= std::min(ty + 3, Gy - 1); ++y) {
+                const int* row = start.data() + (size_t)wrap_host(y, Gy) * Gx;
+                count[t] += row[std::min(tx + 4, Gx)] - row[std::max(tx - 3, 0)];
+                if (tx < 3) count[t] += row[Gx] - row[Gx + tx - 3];
+            }
+            order[t] = t;
+        }
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return count[a] / 8 > count[b] / 8; });
+        PP_TRY(upload(p, &p.tile_order, order));
         PP_TRY(upload(p, &p.cell_start, start));
         PP_TRY(upload(p, &p.sort_wx, wx));
         PP_TRY(upload(p, &p.sort_wy, wy));

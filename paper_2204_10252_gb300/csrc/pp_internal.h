@@ -156,6 +156,7 @@ struct Plan {
     int* cell_start = nullptr;   // [G_y * G_x + 1]
     float4 *sort_wx = nullptr, *sort_wy = nullptr;   // [K] tap weights
     int2* sort_kx = nullptr;     // [K] (sample, first tap's column)
+    int* tile_order = nullptr;   // 4 x 4 tiles of grid points, those with most samples first
     float2* ksp_t = nullptr;     // [K][C rounded up] transposed k-space
     SampleTaps* samp = nullptr;  // [K]
     float* gtg = nullptr;        // [(2W-1)^2][G_y][G_x] stencil of G^T G

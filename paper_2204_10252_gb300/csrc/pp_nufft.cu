@@ -2,18 +2,23 @@
 // G^T (spread, of the adjoint) and G (interpolation, of the forward model).
 //
 // Spread by gathering.  The samples are sorted by the grid cell of their first
-// tap (plan time), so the samples that reach grid point (gy, gx), those whose
-// first tap lies in rows gy-3 .. gy and columns gx-3 .. gx (periodic), are at
-// most two contiguous runs a row: eight runs a point.  A group of LC lanes owns
-// a point, one coil a lane; it fetches LC entries' (sample, weight) at a time,
-// a lane each, and broadcasts them while every lane reads its own coil's
-// value.  With the k-space transposed to [sample][coil] each read is one
-// contiguous run, and a point's sum needs neither atomics nor a fixed tile.
+// tap (plan time), so the samples that reach a 4 x 4 tile of grid points are those
+// of 7 x 7 cells (periodic): seven contiguous runs, and seven more where the tile
+// touches column 0.  A group of LC lanes owns a tile, one coil a lane and the 16
+// points' sums in registers; it prepares LC entries' weights at a time, a lane
+// each, and then reads the coils' values of one sample after another.  With the
+// k-space transposed to [sample][coil] each read is one contiguous run, and the
+// sums need no atomics and have a fixed order.
 //
-// What bounds it: L2 reads of 16 values per sample and coil (268 MB at 65 536
-// samples, 32 coils).  The scatter form it replaces (a CTA per 32 x 32 tile,
-// shared-memory atomics) took 459 us there: a spiral puts a tenth of its samples
-// into the four centre tiles, whose CTAs ran long after the others had ended.
+// What bounds it: latency of the reads (cell starts, entries, weights, samples in
+// turn), 16 warps an SM.  At 65 536 samples on a 320 x 320 grid, 32 coils, a
+// sample's values are read three times on average (51 MB); a group that owned one
+// point read them 16 times (268 MB), 119 us against 33 us here.  The scatter form
+// before that (a CTA per 32 x 32 tile, shared-memory atomics) took 459 us.  85
+// registers a thread for three CTAs an SM: 38 us.
+//
+// Tiles go by the samples that reach them, most first: 50 us in grid order, where
+// the centre of a spiral starts late and its neighbours share a CTA.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -42,25 +47,21 @@ ksp_transpose_kernel(const float2* __restrict__ ksp, int K, int C, int Cp, float
     }
 }
 
-// The eight runs of sorted samples that reach grid point `lin`, one a lane (lanes
-// l < 8 of a group of LC): its start `s` and the inclusive prefix `pre` of the
-// lengths; returns their total.  All 32 lanes of the warp call it.
+// Rows of 7 cells whose samples reach a 4 x 4 tile of grid points at (ty, tx), one
+// a lane (lanes l < 7 of a group of LC): the run's start `s` in the sorted samples
+// and the inclusive prefix `pre` of the lengths; returns their total.  wrap: the
+// cells left of column 0 (tx < 3) in place of the others; cells right of the tile's
+// last column, or below its last row, reach none of its points.  All 32 lanes of
+// the warp call it.
 template <int LC>
-__device__ __forceinline__ int spread_runs(const int* __restrict__ cell_start, int Gx, int Gy, int lin,
-                                           bool live, int l, int* s, int* pre) {
-    const int gy = lin / Gx, gx = lin - gy * Gx;
+__device__ __forceinline__ int spread_runs(const int* __restrict__ cell_start, int Gx, int Gy, int ty,
+                                           int tx, bool live, bool wrap, int l, int* s, int* pre) {
     int st = 0, len = 0;
-    if (live && l < 8) {
-        int row = gy - (l >> 1);
+    int row = ty + l - 3;
+    if (live && l < 7 && row < Gy) {
         if (row < 0) row += Gy;
-        int lo = 1, hi = 0;
-        if ((l & 1) == 0) {
-            lo = gx > 3 ? gx - 3 : 0;
-            hi = gx;
-        } else if (gx < 3) {
-            lo = Gx + gx - 3;
-            hi = Gx - 1;
-        }
+        const int lo = wrap ? Gx + tx - 3 : max(tx - 3, 0);
+        const int hi = wrap ? Gx - 1 : min(tx + 3, Gx - 1);
         if (lo <= hi) {
             const int* cp = cell_start + (int64_t)row * Gx;
             st = cp[lo];
@@ -77,23 +78,33 @@ __device__ __forceinline__ int spread_runs(const int* __restrict__ cell_start, i
     return __shfl_sync(0xffffffffu, len, 7, LC);
 }
 
-// Sum of weight * sample over entries base0 .. base0 + LC, base0 + step .. of the
-// point's n entries, for this lane's coil (kc, NULL: none).  A lane fetches one
-// entry, then all lanes read their coil's value of each; eight reads in flight.
-// nmax: the largest n of the warp's groups.
+struct SpreadTables {
+    const int* cell_start;
+    const float *wx, *wy;   // [K][4], sorted
+    const int2* kx;         // (sample, first-tap column), sorted
+    const int* order;       // tiles, those with most entries first
+    int Gx, Gy;
+};
+
+// One entry of a group's work list: the weights of tile columns 0 .. 3 and rows
+// 0 .. 3, each twice (for packed multiplies), zero where the sample does not reach.
+struct SpreadEntry {
+    float4 x01, x23, y01, y23;
+};
+
+// acc[4 b + a] += wy_b wx_a * sample over entries base0 .. base0 + LC,
+// base0 + step .. of the n entries of the tile's runs, for this lane's coil (kc,
+// NULL: none).  A lane prepares one entry, then all lanes read their coil's value
+// of each; eight reads in flight.  nmax: the largest n of the warp's groups.
 template <int LC>
-__device__ __forceinline__ float2 spread_sum(const float* __restrict__ wxf, const float* __restrict__ wyf,
-                                             const int2* __restrict__ kx, int Gx, int gx, int l, int s,
-                                             int pre, int n, int nmax, int base0, int step,
-                                             const float2* kc, int64_t ks) {
-    float2 acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = make_float2(0.f, 0.f);
+__device__ __forceinline__ void spread_sum(float2 (&acc)[16], const SpreadTables& T, int tx, bool wrap,
+                                           int l, int s, int pre, int n, int nmax, int base0, int step,
+                                           const float2* kc, int64_t ks, SpreadEntry* ent, int* ek) {
     for (int base = base0; base < nmax; base += step) {
         const int t = base + l;
         int idx = 0, before = 0;
 #pragma unroll
-        for (int r = 0; r < 7; ++r) {
+        for (int r = 0; r < 6; ++r) {
             const int pr = __shfl_sync(0xffffffffu, pre, r, LC);
             if (t >= pr) {
                 idx = r + 1;
@@ -102,105 +113,154 @@ __device__ __forceinline__ float2 spread_sum(const float* __restrict__ wxf, cons
         }
         const int sr = __shfl_sync(0xffffffffu, s, idx, LC);
         int k = 0;
-        float w = 0.f;
+        float x[4] = {0.f, 0.f, 0.f, 0.f}, y[4] = {0.f, 0.f, 0.f, 0.f};
         if (t < n) {
             const int j = sr + t - before;
-            const int2 e = kx[j];
-            int a = gx - e.y;
-            if (a < 0) a += Gx;
+            const int2 e = T.kx[j];
+            const int dx = tx - e.y + (wrap ? T.Gx : 0), dy = 3 - idx;
+            const float *wx = T.wx + 4 * (int64_t)j, *wy = T.wy + 4 * (int64_t)j;
             k = e.x;
-            w = wxf[4 * (int64_t)j + a] * wyf[4 * (int64_t)j + (idx >> 1)];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if ((unsigned)(a + dx) < 4u) x[a] = wx[a + dx];
+                if ((unsigned)(a + dy) < 4u) y[a] = wy[a + dy];
+            }
         }
+        __syncwarp();
+        ent[l].x01 = make_float4(x[0], x[0], x[1], x[1]);
+        ent[l].x23 = make_float4(x[2], x[2], x[3], x[3]);
+        ent[l].y01 = make_float4(y[0], y[0], y[1], y[1]);
+        ent[l].y23 = make_float4(y[2], y[2], y[3], y[3]);
+        ek[l] = k;
+        __syncwarp();
         const int m = n - base;
         const int mw = nmax - base < LC ? nmax - base : LC;
         for (int u0 = 0; u0 < mw; u0 += 8) {
             float2 v[8];
-            float ww[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                v[u] = u0 + u < m && kc ? kc[ek[u0 + u] * ks] : make_float2(0.f, 0.f);
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int kk = __shfl_sync(0xffffffffu, k, (u0 + u) & (LC - 1), LC);
-                ww[u] = __shfl_sync(0xffffffffu, w, (u0 + u) & (LC - 1), LC);
-                const bool on = u0 + u < m && kc;
-                if (!on) ww[u] = 0.f;
-                v[u] = on ? kc[kk * ks] : make_float2(0.f, 0.f);
-            }
+                const SpreadEntry& e = ent[u0 + u];
+                const float4 x01 = e.x01, x23 = e.x23, y01 = e.y01, y23 = e.y23;
+                const float2 z = make_float2(0.f, 0.f);
+                const float2 w[4] = {__ffma2_rn(make_float2(x01.x, x01.y), v[u], z),
+                                     __ffma2_rn(make_float2(x01.z, x01.w), v[u], z),
+                                     __ffma2_rn(make_float2(x23.x, x23.y), v[u], z),
+                                     __ffma2_rn(make_float2(x23.z, x23.w), v[u], z)};
+                const float2 yy[4] = {make_float2(y01.x, y01.y), make_float2(y01.z, y01.w),
+                                      make_float2(y23.x, y23.y), make_float2(y23.z, y23.w)};
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                acc[u & 3].x = fmaf(ww[u], v[u].x, acc[u & 3].x);
-                acc[u & 3].y = fmaf(ww[u], v[u].y, acc[u & 3].y);
+                for (int p = 0; p < 16; ++p) acc[p] = __ffma2_rn(yy[p >> 2], w[p & 3], acc[p]);
             }
         }
     }
-    return cadd(cadd(acc[0], acc[1]), cadd(acc[2], acc[3]));
 }
 
-// Every point is written once.  Sample k of coil c is ksp[c * cs + k * ks].  CI:
-// grid_out[point][32] (zero at or past C), else grid_out[c][point].  A point with
-// more than kHeavy entries (the centre of a spiral holds a thousand: one group
-// would need 40 us for it) is summed by all groups of its CTA together: forward +
-// adjoint of a 256 x 256 spiral, 32 coils, 208 -> 198 us, and no longer 290 where
-// the heavy points meet in one SM.
+// Entries above which all groups of a CTA share a tile: 35 us at 64, 34 at 96, 33 at
+// 128, 34 at 192 (the 320 x 320 grid above; its centre tile has 1400).
 constexpr int kHeavy = 128;
 
+// Every point is written once.  Sample k of coil c is ksp[c * cs + k * ks].  CI:
+// grid_out[point][32] (zero at or past C), else grid_out[c][point].  A CTA's groups
+// take a tile each, gridDim.x apart in the order, so that the dense ones fall to
+// different CTAs; a tile with more than kHeavy
+// entries is summed by all groups of its CTA together, one chunk of LC entries at
+// a time in turn.
 template <int LC, bool CI>
-__global__ void __launch_bounds__(256)
-nufft_spread_kernel(const int* __restrict__ cell_start, const float4* __restrict__ wx,
-                    const float4* __restrict__ wy, const int2* __restrict__ kx, int Gx, int Gy, int C,
-                    const float2* __restrict__ ksp, int64_t cs, int64_t ks,
+__global__ void __launch_bounds__(256, 2)
+nufft_spread_kernel(const SpreadTables T, int C, const float2* __restrict__ ksp, int64_t cs, int64_t ks,
                     float2* __restrict__ grid_out) {
-    constexpr int NG = 256 / LC;   // groups (points in flight) per CTA
-    static_assert(LC >= 8, "a group finds its eight runs one a lane");
-    __shared__ float2 tile[CI ? 1 : LC][PT + 1];
-    __shared__ float2 part[NG][LC];
-    __shared__ int heavy[PT], nheavy;
+    constexpr int NG = 256 / LC;   // groups (tiles in flight) per CTA
+    static_assert(LC >= 8, "a group finds its seven runs one a lane");
+    union Shared {
+        struct {
+            SpreadEntry ent[256];
+            int ek[256];
+        } w;
+        float2 part[16][256];
+    };
+    __shared__ Shared sh;
+    __shared__ int heavy[NG], nheavy;
     const int l = threadIdx.x & (LC - 1), g = threadIdx.x / LC;
     const int c = blockIdx.y * LC + l;
-    const int np = Gx * Gy;
-    const float* wxf = reinterpret_cast<const float*>(wx);
-    const float* wyf = reinterpret_cast<const float*>(wy);
+    const int Gx = T.Gx, Gy = T.Gy;
+    const int ntx = (Gx + 3) >> 2, ntiles = ntx * ((Gy + 3) >> 2);
+    const int64_t np = (int64_t)Gx * Gy;
     const float2* kc = c < C ? ksp + c * cs : nullptr;
+    SpreadEntry* ent = sh.w.ent + g * LC;
+    int* ek = sh.w.ek + g * LC;
     if (threadIdx.x == 0) nheavy = 0;
     __syncthreads();
-#pragma unroll 1
-    for (int q = 0; q < PT / NG; ++q) {
-        const int pt = q * NG + g, lin = blockIdx.x * PT + pt;
-        const bool live = lin < np;
-        int s, pre;
-        int n = spread_runs<LC>(cell_start, Gx, Gy, lin, live, l, &s, &pre);
-        const bool big = n > kHeavy;
-        if (big && l == 0) heavy[atomicAdd(&nheavy, 1)] = pt;
-        if (big) n = 0;
+    {
+        const int place = g * gridDim.x + blockIdx.x;
+        const bool live = place < ntiles;
+        const int tile = live ? T.order[place] : 0;
+        const int ty = 4 * (tile / ntx), tx = 4 * (tile % ntx);
+        int s, pre, s2 = 0, pre2 = 0, n2 = 0;
+        int n = spread_runs<LC>(T.cell_start, Gx, Gy, ty, tx, live, false, l, &s, &pre);
+        const bool edge = __any_sync(0xffffffffu, live && tx < 3);
+        if (edge) n2 = spread_runs<LC>(T.cell_start, Gx, Gy, ty, tx, live && tx < 3, true, l, &s2, &pre2);
+        const bool big = n + n2 > kHeavy;
+        if (big && l == 0) heavy[atomicAdd(&nheavy, 1)] = tile;
+        if (big) n = n2 = 0;
+        float2 acc[16];
+#pragma unroll
+        for (int p = 0; p < 16; ++p) acc[p] = make_float2(0.f, 0.f);
         const int nmax = LC < 32 ? __reduce_max_sync(0xffffffffu, n) : n;
-        const float2 sum = spread_sum<LC>(wxf, wyf, kx, Gx, lin % Gx, l, s, pre, n, nmax, 0, LC, kc, ks);
-        if (big || !live) continue;
-        if (CI) grid_out[(int64_t)lin * 32 + l] = sum;
-        else tile[l][pt] = sum;
+        spread_sum<LC>(acc, T, tx, false, l, s, pre, n, nmax, 0, LC, kc, ks, ent, ek);
+        if (edge) {
+            const int nmax2 = LC < 32 ? __reduce_max_sync(0xffffffffu, n2) : n2;
+            spread_sum<LC>(acc, T, tx, true, l, s2, pre2, n2, nmax2, 0, LC, kc, ks, ent, ek);
+        }
+        if (live && !big) {
+            if (CI) {
+                float2* o = grid_out + ((int64_t)ty * Gx + tx) * 32 + l;
+#pragma unroll
+                for (int p = 0; p < 16; ++p)
+                    if (ty + (p >> 2) < Gy && tx + (p & 3) < Gx) o[((p >> 2) * Gx + (p & 3)) * 32] = acc[p];
+            } else if (c < C) {
+                float2* o = grid_out + c * np + (int64_t)ty * Gx + tx;
+#pragma unroll
+                for (int p = 0; p < 16; p += 2)   // plans have even grids, 16-byte aligned
+                    if (ty + (p >> 2) < Gy && tx + (p & 3) < Gx)
+                        *reinterpret_cast<float4*>(o + (p >> 2) * Gx + (p & 3)) =
+                            make_float4(acc[p].x, acc[p].y, acc[p + 1].x, acc[p + 1].y);
+            }
+        }
     }
     __syncthreads();
     const int nh = nheavy;
     for (int h = 0; h < nh; ++h) {
-        const int pt = heavy[h], lin = blockIdx.x * PT + pt;
-        int s, pre;
-        const int n = spread_runs<LC>(cell_start, Gx, Gy, lin, true, l, &s, &pre);
-        // every group of a warp takes the same number of turns
-        const int turns = (n + NG * LC - 1) / (NG * LC);
-        part[g][l] = spread_sum<LC>(wxf, wyf, kx, Gx, lin % Gx, l, s, pre, n,
-                                    g * LC + (turns - 1) * NG * LC + LC, g * LC, NG * LC, kc, ks);
+        const int tile = heavy[h];
+        const int ty = 4 * (tile / ntx), tx = 4 * (tile % ntx);
+        float2 acc[16];
+#pragma unroll
+        for (int p = 0; p < 16; ++p) acc[p] = make_float2(0.f, 0.f);
+        for (int wrap = 0; wrap < (tx < 3 ? 2 : 1); ++wrap) {
+            int s, pre;
+            const int n = spread_runs<LC>(T.cell_start, Gx, Gy, ty, tx, true, wrap != 0, l, &s, &pre);
+            // every group of a warp takes the same number of turns
+            const int turns = (n + NG * LC - 1) / (NG * LC);
+            spread_sum<LC>(acc, T, tx, wrap != 0, l, s, pre, n, g * LC + turns * NG * LC, g * LC, NG * LC,
+                           kc, ks, ent, ek);
+        }
+        __syncthreads();   // the entries and the parts share their memory
+#pragma unroll
+        for (int p = 0; p < 16; ++p) sh.part[p][threadIdx.x] = acc[p];
         __syncthreads();
-        if (g == 0) {
-            float2 sum = part[0][l];
-            for (int p = 1; p < NG; ++p) sum = cadd(sum, part[p][l]);
-            if (CI) grid_out[(int64_t)lin * 32 + l] = sum;
-            else tile[l][pt] = sum;
+        for (int e = threadIdx.x; e < 16 * LC; e += 256) {
+            const int p = e / LC, ll = e - p * LC, cc = blockIdx.y * LC + ll;
+            const int gy = ty + (p >> 2), gx = tx + (p & 3);
+            float2 sum = sh.part[p][ll];
+            for (int q = 1; q < NG; ++q) sum = cadd(sum, sh.part[p][q * LC + ll]);
+            if (gy >= Gy || gx >= Gx) continue;
+            const int64_t lin = (int64_t)gy * Gx + gx;
+            if (CI) grid_out[lin * 32 + ll] = sum;
+            else if (cc < C) grid_out[cc * np + lin] = sum;
         }
         __syncthreads();
-    }
-    if (!CI) {
-        const int tx = threadIdx.x & 31, lin = blockIdx.x * PT + tx;
-        for (int cc = threadIdx.x >> 5; cc < LC; cc += 8) {
-            const int cg = blockIdx.y * LC + cc;
-            if (cg < C && lin < np) grid_out[(int64_t)cg * np + lin] = tile[cc][tx];
-        }
     }
 }
 
@@ -301,9 +361,12 @@ pp_status transpose_ksp(const Plan& p, int lc, const float2* ksp, int Cp, float2
 template <int LC, bool CI>
 pp_status spread(const Plan& p, const float2* ksp, int64_t cs, int64_t ks, float2* grid_out,
                  cudaStream_t st) {
-    const dim3 g((p.G_x * p.G_y + PT - 1) / PT, (p.C + LC - 1) / LC);
-    nufft_spread_kernel<LC, CI><<<g, 256, 0, st>>>(p.cell_start, p.sort_wx, p.sort_wy, p.sort_kx, p.G_x,
-                                                   p.G_y, p.C, ksp, cs, ks, grid_out);
+    const int ntiles = ((p.G_x + 3) / 4) * ((p.G_y + 3) / 4), ng = 256 / LC;
+    const dim3 g((ntiles + ng - 1) / ng, (p.C + LC - 1) / LC);
+    const SpreadTables T{p.cell_start, reinterpret_cast<const float*>(p.sort_wx),
+                         reinterpret_cast<const float*>(p.sort_wy), p.sort_kx, p.tile_order,
+                         p.G_x, p.G_y};
+    nufft_spread_kernel<LC, CI><<<g, 256, 0, st>>>(T, p.C, ksp, cs, ks, grid_out);
     return check_nufft("nufft_spread_kernel");
 }
 
