@@ -470,8 +470,13 @@ static pp_status build_cartesian(Plan& p, const uint8_t* mask) {
     } else if (p.ndim == 2) {
         PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.C * p.nimg));
     } else {
-        // coils whose planes fill about half of the L2 (129 MB) together
-        p.c3_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(p.C, (72ll << 20) / (8 * p.nimg)));
+        // Coils of one launch of each stage: 512 MB of planes.  Planes that fit L2
+        // together (72 MB) leave each launch short: the stages read little back from
+        // L2 (26 % hits), and every launch ends in a part wave and, in the adjoint,
+        // adds to the image.  80 x 180 x 200 x 12, forward + adjoint / normal: 862 /
+        // 502 us at 72 MB, 789 / - at 200, 746 / 429 at 512 and above; 128 x 200 x 200
+        // x 9, normal: 1090 -> 650.
+        p.c3_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(p.C, (512ll << 20) / (8 * p.nimg)));
         PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.c3_chunk * p.nimg));
         PP_TRY(alloc_n(p, &p.wk_b, (size_t)p.nimg));
     }

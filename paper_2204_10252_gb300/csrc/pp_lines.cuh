@@ -3,7 +3,9 @@
 // two-factor decomposition of pp_fft4.cuh: n = N1 N2, N1 <= N2 <= 32, input
 // m = N2 m1 + m2, output k = k1 + N1 k2; one shared-memory transpose a transform,
 // all global loads of a thread issued together, every twiddle from the table.
-// Same index maps as the Stockham kernels of pp_kernels.cu (RowArgs, ColArgs).
+// Same index maps as the Stockham kernels of pp_kernels.cu (RowArgs, ColArgs).  In
+// the row stages the second half's (line, k1) pairs are packed into the first
+// RBG N1 threads, so that it runs in N1 / N2 of the warps.
 //
 // What bounds them: one read and one write per element, N1 loads in flight a
 // thread.  A kernel that switches on the two factors at run time moves the same
@@ -322,8 +324,7 @@ __global__ void __launch_bounds__(RBG * N2, line_min_ctas(RBG * N2)) line_rows_f
     const int b = threadIdx.x / N2, r = threadIdx.x - b * N2;
     float2* Y = sm + n + b * N1 * P;
     const int row = blockIdx.x * RBG + b;
-    const bool live = row < nrows;
-    const int lrow = live ? row : nrows - 1;
+    const int lrow = row < nrows ? row : nrows - 1;
     const float2* xr = xs + (int64_t)lrow * a.n;
     const float2* sr = ss ? ss + (int64_t)lrow * a.n : nullptr;
     const float wr = a.scale * (L.wrow ? L.wrow[lrow] : 1.f);
@@ -365,16 +366,19 @@ __global__ void __launch_bounds__(RBG * N2, line_min_ctas(RBG * N2)) line_rows_f
         for (int k1 = 0; k1 < N1; ++k1) Y[k1 * P + r] = v[k1];
     }
     __syncthreads();
-    if (r < N1) {
-        float2* o = od + (int64_t)lrow * n;
+    if (threadIdx.x < RBG * N1) {
+        const int b2 = N1 == N2 ? b : threadIdx.x / N1, k1 = N1 == N2 ? r : threadIdx.x - b2 * N1;
+        const int row2 = blockIdx.x * RBG + b2;
+        const float2* Y2 = sm + n + (b2 * N1 + k1) * P;
         float2 u[N2];
 #pragma unroll
-        for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y[r * P + m2];
+        for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y2[m2];
         RegFft<N2, false>::run(u, tws, N1);
-        if (live) {
+        if (row2 < nrows) {
+            float2* o = od + (int64_t)row2 * n;
 #pragma unroll
             for (int k2 = 0; k2 < N2; ++k2) {
-                int q = r + N1 * k2 + a.off_out;
+                int q = k1 + N1 * k2 + a.off_out;
                 if (q >= n) q -= n;
                 o[q] = u[k2];
             }
@@ -410,23 +414,37 @@ __global__ void __launch_bounds__(RBG * N2, line_min_ctas(RBG * N2)) line_rows_a
         cstride = (int64_t)nrows * a.n;
     }
     load_tw(tws, L.tw, n);
+    // (line, m2) in the first half, (line, k1) on the first RBG N1 threads after it
     const int b = threadIdx.x / N2, r = threadIdx.x - b * N2;
-    const int slot = b / rb, lrow = b - slot * rb;
+    const int b2 = N1 == N2 ? b : threadIdx.x / N1, k1 = N1 == N2 ? r : threadIdx.x - b2 * N1;
+    // r < N1 holds where N1 = N2; written out it keeps the map's loads behind the
+    // first half (in front of it, 18 x 18 and 20 x 20 spill 140 to 220 bytes)
+    const bool second = N1 == N2 ? r < N1 : threadIdx.x < RBG * N1;
     float2* Y = sm + n + b * N1 * P;
+    const float2* Y2 = sm + n + (b2 * N1 + k1) * P;
     float2* accs = sm + n + RBG * N1 * P;
-    float2* acc = accs + b * a.n;
+    float2* acc = accs + b2 * a.n;
     for (int e = threadIdx.x; e < RBG * a.n; e += blockDim.x) accs[e] = make_float2(0.f, 0.f);
-    const int row = blockIdx.x * rb + lrow;
-    const float wr = (L.wrow && row < nrows) ? L.wrow[row] : 1.f;
+    const int slot = b / rb, row = blockIdx.x * rb + b - slot * rb;
+    const int slot2 = N1 == N2 ? slot : b2 / rb, row2 = N1 == N2 ? row : blockIdx.x * rb + b2 - slot2 * rb;
+    const float wr = (L.wrow && second && row2 < nrows) ? L.wrow[row2] : 1.f;
     int r0 = r + a.off_in;
     if (r0 >= n) r0 -= n;
     __syncthreads();
     for (int c0 = 0; c0 < ncoils; c0 += cb) {
-        const int c = c0 + slot;
-        const bool live = row < nrows && c < ncoils;
-        const float2* sc = sens ? sens + c * cstride + (int64_t)row * a.n : nullptr;
-        float2 s[N2];   // the map, read while the transform's first half runs
-        if (live) {
+        const int c = c0 + slot, c2 = c0 + slot2;
+        const bool live2 = second && row2 < nrows && c2 < ncoils;
+        const float2* sc = sens ? sens + c2 * cstride + (int64_t)row2 * a.n : nullptr;
+        float2 s[N2];   // the map, read across the barrier
+        auto read_map = [&] {
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) {
+                int i = k1 + N1 * k2 + a.off_out;
+                if (i >= n) i -= n;
+                s[k2] = i < a.n ? sc[i] : make_float2(0.f, 0.f);
+            }
+        };
+        if (row < nrows && c < ncoils) {
             const float2* sr = src + ((int64_t)c * nrows + row) * n;
             float2 v[N1];
 #pragma unroll
@@ -438,20 +456,14 @@ __global__ void __launch_bounds__(RBG * N2, line_min_ctas(RBG * N2)) line_rows_a
             fft4_phase1_exact<N1, N2, true>(v, r, tws);
 #pragma unroll
             for (int k1 = 0; k1 < N1; ++k1) Y[k1 * P + r] = v[k1];
-            if (sc && r < N1) {
-#pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) {
-                    int i = r + N1 * k2 + a.off_out;
-                    if (i >= n) i -= n;
-                    s[k2] = i < a.n ? sc[i] : make_float2(0.f, 0.f);
-                }
-            }
+            if (N1 == N2 && sc && second) read_map();
         }
+        if (N1 != N2 && sc && live2) read_map();
         __syncthreads();
-        if (live && r < N1) {
+        if (live2) {
             float2 u[N2];
 #pragma unroll
-            for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y[r * P + m2];
+            for (int m2 = 0; m2 < N2; ++m2) u[m2] = Y2[m2];
             RegFft<N2, true>::run(u, tws, N1);
             if (sc) {
 #pragma unroll
@@ -459,23 +471,36 @@ __global__ void __launch_bounds__(RBG * N2, line_min_ctas(RBG * N2)) line_rows_a
             }
 #pragma unroll
             for (int k2 = 0; k2 < N2; ++k2) {
-                int i = r + N1 * k2 + a.off_out;
+                int i = k1 + N1 * k2 + a.off_out;
                 if (i >= n) i -= n;
                 if (i < a.n) acc[i] = cadd(acc[i], cscale(u[k2], L.wcol ? wr * L.wcol[i] : wr));
             }
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < rb * a.n; e += blockDim.x) {
-        const int lr = e / a.n, i = e - lr * a.n;
-        const int orow = blockIdx.x * rb + lr;
-        if (orow >= nrows) continue;
-        float2 v = accs[lr * a.n + i];
-        for (int s = 1; s < cb; ++s) v = cadd(v, accs[(s * rb + lr) * a.n + i]);
-        const int64_t o = (int64_t)orow * a.n + i;
-        v = cscale(v, scale);
-        if (L.operand) v = cadd(v, cscale(L.operand[o], L.alpha));
-        out[o] = v;
+    // the CTA's rows are contiguous in the image; eight loads of the operand in
+    // flight (one at a time they took 26 us of a 68 us launch)
+    const int64_t o0 = (int64_t)blockIdx.x * rb * a.n;
+    const int ne = min(rb, nrows - (int)blockIdx.x * rb) * a.n, sn = rb * a.n;
+    for (int e0 = threadIdx.x; e0 < ne; e0 += 8 * blockDim.x) {
+        float2 op[8];
+        if (L.operand) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int e = e0 + u * blockDim.x;
+                if (e < ne) op[u] = L.operand[o0 + e];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int e = e0 + u * blockDim.x;
+            if (e >= ne) break;
+            float2 v = accs[e];
+            for (int s = 1; s < cb; ++s) v = cadd(v, accs[s * sn + e]);
+            v = cscale(v, scale);
+            if (L.operand) v = cadd(v, cscale(op[u], L.alpha));
+            out[o0 + e] = v;
+        }
     }
 }
 
