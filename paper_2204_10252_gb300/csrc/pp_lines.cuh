@@ -73,6 +73,16 @@ template <int N1, int N2> struct Line {
 // At most 128 registers a thread, and 8 CTAs an SM of the small blocks.
 __host__ __device__ constexpr int line_min_ctas(int threads) { return threads < 512 ? 512 / threads : 1; }
 
+// The round trip holds one transform at a time: 80 registers are enough up to
+// N2 = 16 and 102 up to 20 without spilling (32 bytes at 16 x 16), and half as many
+// threads more an SM: 148 -> 134 us at 12 x 80 x 180 x 200, whole normal operator of
+// 100 x 256 x 108 x 7 256 -> 240 us.  The inverse y stage with the same cap spills
+// 150 bytes and more (156 -> 181 us).
+__host__ __device__ constexpr int roundtrip_min_ctas(int threads) {
+    const int t = threads <= 128 ? 768 : (threads <= 160 ? 640 : 512);
+    return threads < t ? t / threads : 1;
+}
+
 __device__ __forceinline__ float2 tw_of(const float2* tws, int t, bool inv) {
     float2 w = tws[t];
     if (inv) w.y = -w.y;
@@ -251,7 +261,7 @@ __global__ void __launch_bounds__(TXG * N2, line_min_ctas(TXG * N2)) line_yinv_k
 // length-N2 DFT over k2 and twiddle W^-(m2 k1) feed the (m2) threads' inverse
 // length-N1 DFT.  src == dst is allowed.
 template <int N1, int N2>
-__global__ void __launch_bounds__(TXG * N2, line_min_ctas(TXG * N2)) line_roundtrip_kernel(const LineCols L) {
+__global__ void __launch_bounds__(TXG * N2, roundtrip_min_ctas(TXG * N2)) line_roundtrip_kernel(const LineCols L) {
     constexpr int n = N1 * N2, P = N2 | 1;
     extern __shared__ float2 sm[];
     float2* tws = sm;
