@@ -301,17 +301,23 @@ nufft_degrid_kernel(const SampleTaps* __restrict__ st, int K, int Gx, int Gy,
 
 // The same from the coil-innermost grid [Gy][Gx][32]: a warp takes 4 samples in
 // turn, one coil a lane (256-byte rows, which neighbouring samples of a readout
-// find in L1); 32 samples x 32 coils are transposed through shared memory.
+// find in L1); 32 samples x 32 coils are transposed through shared memory.  26.6 us
+// at 65 536 samples with a sample's taps and values in turn, 25.5 us with the taps of
+// all four first and two samples' values in flight.
 __global__ void __launch_bounds__(256)
 ci_degrid_kernel(const SampleTaps* __restrict__ st, int K, int Gx, int Gy, int C,
                  const float2* __restrict__ grid, float2* __restrict__ ksp) {
     __shared__ float2 tile[32][PT + 1];
+    __shared__ SampleTaps taps[PT];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll 1
+    // a warp's four samples' taps at once (past the last sample: the last again,
+    // not stored), then 32 grid values in flight
+    if (lane < 4) taps[4 * w + lane] = st[min((int)blockIdx.x * PT + 4 * w + lane, K - 1)];
+    __syncwarp();
+#pragma unroll 2
     for (int q = 0; q < 4; ++q) {
-        const int kk = 4 * w + q, k = blockIdx.x * PT + kk;
-        if (k >= K) break;
-        const SampleTaps s = st[k];
+        const int kk = 4 * w + q;
+        const SampleTaps s = taps[kk];
         const float wx[4] = {s.wx.x, s.wx.y, s.wx.z, s.wx.w};
         const float wy[4] = {s.wy.x, s.wy.y, s.wy.z, s.wy.w};
         const int y0 = wrapG(s.iy0, Gy), x0 = wrapG(s.ix0, Gx);
