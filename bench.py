@@ -219,8 +219,9 @@ def kernel_flops(c, K, toeplitz=False):
         "ci_sum_kernel": 4.0 * 2.0 * n,
         "rows_adj_cb_kernel": C * ny * fft(G) + 10.0 * C * n,
         "rows_adj_kernel": C * ny * fft(G) + 10.0 * C * n,
-        "rows4_fwd_kernel": C * ny * fft(G) + 8.0 * C * n,
-        "cols4_kernel": C * G * fft(G),
+        "line_rows_fwd_kernel": C * ny * fft(G) + 8.0 * C * n,
+        "line_cols_kernel": C * G * fft(G),
+        "line_rows_adj_kernel": C * ny * fft(G) + 10.0 * C * n,
         "rows4_adj_kernel": C * ny * fft(G) + 10.0 * C * n,
         "rows4_adj_cl_kernel": C * ny * fft(G) + 10.0 * C * n,
         "rows4_inv_kernel": C * ny * fft(G) + 8.0 * C * n,
@@ -531,7 +532,7 @@ def main():
     apply_ms = sum(stages.values())
     flops = kernel_flops(c, K, toep)
     # cols_kernel runs twice per apply (forward and inverse): per-launch time is half
-    launches_per_apply = {"cols_kernel": 2, "cols4_kernel": 2, "ci_cols_kernel": 2}
+    launches_per_apply = {"cols_kernel": 2, "line_cols_kernel": 2, "ci_cols_kernel": 2}
     per_launch_ms = {k: v / launches_per_apply.get(k, 1) for k, v in stages.items()}
     dom = max(stages, key=stages.get)
     peak_tflops, peak_src = fp32_peak(dev, clocks)

@@ -184,7 +184,7 @@ def cart3d(args, pp, rank, world, local):
                                "hbm_frac": llr_gbs / peak, "bytes_per_call": llr_bytes,
                                "ms_per_call": llr_ms / llr_calls,
                                "timing": "back-to-back calls alternating over two 335 MB input/output "
-                                         "pairs (1.3 GB, larger than L2); one-sided Jacobi SVD per "
+                                         "pairs (1.3 GB, larger than L2); Gram-matrix SVD per "
                                          "512 x 5 block, instruction bound"}})
 
 
@@ -231,7 +231,7 @@ def batched(args, pp, rank, world, local):
                   "coil_map_bytes": 8 * sum(C * s[0] * s[1] for C, s in zip(coils, shapes)),
                   "d": c["d"], "iters": c["iters"], "l2": "inputs larger than L2; flushed between steps",
                   "autotuned_cols_per_cta": tile, "persistent_ctas": grid, "setup_s": setup_s}, clk,
-                 {"roofline": {"bound": "hbm", "kernel": "cart2d_batch_normal_kernel (one launch per apply)",
+                 {"roofline": {"bound": "hbm", "kernel": "cart_stream_kernel / cart_cols_kernel (side by side per size)",
                                "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
                                "traffic": bench.ncu_traffic("cart2d_batch_normal", "ncu_traffic_batched.json"),
                                "peak_source": src,
