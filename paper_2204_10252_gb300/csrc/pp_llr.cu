@@ -19,7 +19,7 @@
 // T'-1 rounds of every sweep, and are rotated twice instead of in every round:
 // five images of 128 x 256 x 256 with 8^3 blocks (0.67 GB in and out) took
 // 877 us with one-sided Jacobi over the rows (issue bound: 60 % of issue slots)
-// and take 369 us (1820 GB/s).
+// and take 348 us (1930 GB/s).
 //
 // The T x T eigenproblems run in one warp, a lane per matrix element: the
 // rounds of disjoint pairs (round-robin schedule, T' = T rounded up to even)
@@ -211,12 +211,25 @@ __device__ __forceinline__ int64_t llr_voxel(const LlrArgs& a, int b, int row) {
 // gave wrong results (the tests hold every compiled form to the oracle).
 __host__ __device__ constexpr int llr_min_ctas(int nt) { return nt > 32 ? 65536 / (nt * 80) : 0; }
 
+// A trace of the Gram matrix whose reciprocal, or whose terms, leave the range of
+// FP32: the first product only scales the rows, by this, and the second Gram matrix
+// is the only one.  2^100: no |x| is above 1e-14 there, and the squares of the
+// smallest FP32 numbers become 2^-98; 2^-80: the largest become 2^96.  A trace of 0
+// needs nothing (every output is 0), and a NaN stays one.  All of it is the first
+// warp's: forming the Gram matrix once more instead cost 3 to 15 % of the prox
+// (registers), this nothing to 2 % (five images 128 x 256 x 256: 355 -> 348 us, two
+// images 64 x 256 x 256: 57.4 -> 58.9).
+__device__ __forceinline__ float llr_unit(float trace) {
+    if (trace > 0.f && trace < 1e-28f) return 0x1p100f;
+    return trace == __int_as_float(0x7f800000) ? 0x1p-80f : 1.f;
+}
+
 template <int T, int RPT, int NT>
 __global__ void __launch_bounds__(NT, llr_min_ctas(NT)) llr_prox_kernel(LlrArgs a) {
     __shared__ float part[NT / 32][64];
     __shared__ float2 A[2][T][T], V0[2][T][T], V1[2][T][T];
     __shared__ float4 W[T][T];   // (x, x, -y, y) of the T x T factor applied to the rows
-    __shared__ float trace;
+    __shared__ float trace, unit;
     const int b = blockIdx.x;
     const int lane = threadIdx.x & 31;
     float2 m[RPT][T];
@@ -249,19 +262,24 @@ __global__ void __launch_bounds__(NT, llr_min_ctas(NT)) llr_prox_kernel(LlrArgs 
                 g[q] = acc;
                 if (e < T * T && e / T == e % T) tr += acc;
             }
-            if (pass == 0) {
+            if (pass == 0 || unit != 1.f) {
 #pragma unroll
                 for (int o = 16; o; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-                if (lane == 0) trace = tr;
+                __syncwarp();
+                if (lane == 0) {
+                    trace = tr;
+                    if (pass == 0) unit = llr_unit(tr);
+                }
                 __syncwarp();
             }
             tr = trace;
             const float sc = tr > 0.f ? 1.f / tr : (tr == 0.f ? 0.f : tr);
+            const bool skip = pass == 0 && unit != 1.f;   // A = 0: no rotations, V0 = I
 #pragma unroll
             for (int q = 0; q < (T * T + 31) / 32; ++q) {
                 const int e = lane + 32 * q, i = e / T, k = e - i * T;
                 if (e < T * T) {
-                    const float v = g[q] * sc;
+                    const float v = skip ? 0.f : g[q] * sc;
                     if (i == k) {
                         A[0][i][i] = make_float2(v, 0.f);
                     } else if (i < k) {
@@ -282,12 +300,13 @@ __global__ void __launch_bounds__(NT, llr_min_ctas(NT)) llr_prox_kernel(LlrArgs 
                 for (int q = 0; q < (T * T + 31) / 32; ++q) {
                     const int e = lane + 32 * q;
                     if (e < T * T) {
-                        const float2 v = (&V0[c0][0][0])[e];
+                        const float2 v = cscale((&V0[c0][0][0])[e], unit);
                         (&W[0][0])[e] = make_float4(v.x, v.x, -v.y, v.y);
                     }
                 }
             } else {
                 const int c1 = warp_jacobi<T>(A, V1, tol, 1e-3f);
+                const float lam = a.lam * unit, back = 1.f / unit;
                 // W = V1 F V^H with V = V0 V1; V goes to the buffer of A not in use
 #pragma unroll
                 for (int q = 0; q < (T * T + 31) / 32; ++q) {
@@ -310,7 +329,7 @@ __global__ void __launch_bounds__(NT, llr_min_ctas(NT)) llr_prox_kernel(LlrArgs 
                             // s <= lambda (also s = 0) -> 0; a NaN fails the test and stays NaN
                             const float d = A[c1][l][l].x * tr;
                             const float sg = d < 0.f ? 0.f : sqrtf(d);
-                            const float f = sg <= a.lam ? 0.f : 1.f - a.lam / sg;
+                            const float f = sg <= lam ? 0.f : (1.f - lam / sg) * back;
                             const float2 v = A[c1 ^ 1][k][l];
                             s = cadd(s, cscale(cmulc(v, V1[c1][i][l]), f));
                         }

@@ -137,3 +137,43 @@ def test_llr_prox_graded_spectrum(pp, shape, block, T):
     out = torch.empty_like(xin)
     pp.pp_prox_llr(shape, T, block, lam, xin, out)
     assert rel(host(out), ref) <= 6e-6
+
+
+@pytest.mark.parametrize("T", [1, 5, 8])
+@pytest.mark.parametrize("shape,block", [((8, 8, 8), 8), ((16, 16), 16), ((4, 4, 4), 4), ((4, 4), 4)],
+                         ids=["512rows", "256rows", "64rows", "16rows"])
+@pytest.mark.parametrize("mag", [1e-18, 1e-20, 1e-21, 1e-22, 1e16, 1e18, 3e19])
+def test_llr_prox_at_the_ends_of_the_range(pp, shape, block, T, mag):
+    """Blocks whose Gram matrix leaves the FP32 range although the block does
+    not: every entry near `mag`, one image zero (T > 1), and a block that is zero
+    but for three voxels of one image.  The bound is that of the graded spectra:
+    a power-of-two scale adds no rounding to normal numbers."""
+    import torch
+    rng = np.random.default_rng(7 * T + int(np.prod(shape)))
+    x = (rng.standard_normal((T,) + shape) + 1j * rng.standard_normal((T,) + shape)) * mag
+    if T > 1:
+        x[T // 2] = 0
+    tail = np.zeros_like(x)
+    tail.reshape(T, -1)[T - 1, :3] = mag * np.array([1.0, -2.0, 0.5j])
+    for v in (x.astype(np.complex64), tail.astype(np.complex64)):
+        top = float(np.linalg.norm(v.astype(np.complex128)))   # no singular value is above it
+        xin = dev(v)
+        out = torch.empty_like(xin)
+        for lam in (0.0, float(np.float32(0.3 * top / np.sqrt(T)))):
+            pp.pp_prox_llr(shape, T, block, lam, xin, out)
+            assert rel(host(out) / mag, O.prox_llr(v.astype(np.complex128), lam, block) / mag) <= 6e-6, lam
+        pp.pp_prox_llr(shape, T, block, 1.1 * top, xin, out)
+        assert np.all(host(out) == 0)
+
+
+@pytest.mark.parametrize("T", [1, 5])
+def test_llr_prox_below_the_range_is_finite(pp, T):
+    """Squares that underflow altogether: finite, and no larger than the input."""
+    import torch
+    x = np.full((T, 8, 8), 1e-24 + 1e-24j, np.complex64)
+    xin = dev(x)
+    out = torch.empty_like(xin)
+    for lam in (0.0, 1e-3):
+        pp.pp_prox_llr((8, 8), T, 8, lam, xin, out)
+        got = host(out)
+        assert np.all(np.isfinite(got)) and np.all(np.abs(got) <= 2e-24)
