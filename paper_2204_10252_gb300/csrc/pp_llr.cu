@@ -207,8 +207,10 @@ __device__ __forceinline__ int64_t llr_voxel(const LlrArgs& a, int b, int row) {
 }
 
 // At most 80 registers a thread: 6 CTAs of 128 threads an SM.  One-warp CTAs are
-// left uncapped: capped at 80, their seven- and eight-image forms spill and
-// gave wrong results (the tests hold every compiled form to the oracle).
+// left uncapped (up to 103 registers).  Capped, their results are the same; a few
+// blocks take longer (256 x 240 in 8 x 8 blocks: 30.7 -> 32.9 us for seven images,
+// 32.9 -> 35.0 for eight) and many are faster (64 x 256 x 256 in 4^3 blocks: 1004 ->
+// 935 us for seven, 1008 -> 910 for eight).
 __host__ __device__ constexpr int llr_min_ctas(int nt) { return nt > 32 ? 65536 / (nt * 80) : 0; }
 
 // A trace of the Gram matrix whose reciprocal, or whose terms, leave the range of
