@@ -21,6 +21,7 @@
 #include "pp_batch.h"
 #include "pp_fft4.cuh"
 #include "pp_internal.h"
+#include "pp_twiddles.h"
 
 namespace pp {
 
@@ -88,70 +89,6 @@ static pp_status alloc_n(Plan& p, T** ptr, size_t n) {
     return dev_alloc(p, reinterpret_cast<void**>(ptr), n * sizeof(T));
 }
 
-// Mean of |w|^2 - 1 that the FP32 constants of a register DFT leave in its output
-// energy (pp_fft.cuh, pp_fft4.cuh, pp_fftgen.cuh): the radix kernels' own
-// constants, and the inner twiddles of a composite A * B.
-static double reg_dft_gain(int N) {
-    auto sq = [](double v) { const double f = (float)v; return f * f; };
-    if (N <= 2 || N == 4) return 0.0;
-    if (N == 3) return (3.0 + 2.0 * (1.0 + 2.0 * (0.25 + sq(sqrt(3.0) / 2.0)))) / 9.0 - 1.0;
-    if (N == 5) {
-        double e = 0.0;
-        for (int q = 1; q <= 2; ++q) e += sq(cos(2.0 * M_PI * q / 5.0)) + sq(sin(2.0 * M_PI * q / 5.0));
-        return (5.0 + 4.0 * (1.0 + 2.0 * e)) / 25.0 - 1.0;
-    }
-    if (N == 8) return 0.25 * (2.0 * sq(sqrt(0.5)) - 1.0);   // two of the eight inner products
-    static const int ab[][2] = {{3, 2}, {3, 3}, {5, 2}, {4, 3}, {5, 3}, {4, 4}, {9, 2}, {4, 5}, {8, 3}, {5, 5}, {9, 3}, {10, 3}, {8, 4}};
-    for (const auto& f : ab) {
-        const int A = f[0], B = f[1];
-        if (A * B != N) continue;
-        double g = 0.0;
-        for (int b = 0; b < B; ++b)
-            for (int k = 0; k < A; ++k)
-                g += sq(cos(2.0 * M_PI * b * k / N)) + sq(sin(2.0 * M_PI * b * k / N)) - 1.0;
-        return reg_dft_gain(A) + reg_dft_gain(B) + g / N;
-    }
-    return 0.0;
-}
-
-// Twiddles of the two-factor kernels (n = n1 n2, W_n^(m2 k1)).  Rounding them and
-// the register DFTs' constants to FP32 changes the transform's mean output energy
-// by some 5e-8, always the same way, so that it adds up over the transforms of a
-// solve where rounding does not.  The table is scaled by the one factor that
-// brings the mean to 1 - 1e-8 (bisection: entries round one by one), the value at
-// which the coefficient gradients of a 3-iteration unrolled solve, which are
-// differences of large sums, were least off their 64-bit values: 6e-7 relative on
-// eight 256 x 256 slices, 9e-7 at a mean of 1 and 2e-6 with the plain table.
-static std::vector<float2> balanced_twiddles(int n) {
-    const GenSplit g = gen_split_of(n);
-    if (!g.n1) return {};
-    const double reg = reg_dft_gain(g.n1) + reg_dft_gain(g.n2);
-    auto table = [&](double scale) {
-        std::vector<float2> tw(n);
-        for (int t = 0; t < n; ++t) {
-            const double a = -2.0 * M_PI * (double)t / (double)n;
-            tw[t] = make_float2((float)(scale * cos(a)), (float)(scale * sin(a)));
-        }
-        tw[0] = make_float2(1.f, 0.f);
-        return tw;
-    };
-    auto gain = [&](const std::vector<float2>& tw) {
-        double e = 0.0;
-        for (int m = 0; m < g.n2; ++m)
-            for (int k = 0; k < g.n1; ++k) {
-                const float2 w = tw[m * k];
-                e += (double)w.x * w.x + (double)w.y * w.y - 1.0;
-            }
-        return reg + e / n;
-    };
-    double lo = 1.0 - 5e-7, hi = 1.0 + 5e-7;
-    for (int it = 0; it < 20; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        (gain(table(mid)) > -1e-8 ? hi : lo) = mid;
-    }
-    return table(0.5 * (lo + hi));
-}
-
 static pp_status make_fft(Plan& p, int n, DevFft& f) {
     if (!factorize(n, f.d)) {
         set_error("FFT length %d has a prime factor above 5", n);
@@ -164,9 +101,10 @@ static pp_status make_fft(Plan& p, int n, DevFft& f) {
     }
     PP_TRY(alloc_n(p, &f.tw, n));
     PP_TRY_CUDA(cudaMemcpy(f.tw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
-    const std::vector<float2> twb = balanced_twiddles(n);
+    const GenSplit g = gen_split_of(n);
     f.twb = f.tw;
-    if (!twb.empty()) {
+    if (g.n1) {
+        const std::vector<Twiddle> twb = balanced_twiddles(g.n1, g.n2);
         PP_TRY(alloc_n(p, &f.twb, n));
         PP_TRY_CUDA(cudaMemcpy(f.twb, twb.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
     }
