@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import glob
 import os
+import re
 import shutil
 import subprocess
 from concurrent.futures import ThreadPoolExecutor
@@ -27,6 +28,24 @@ def _newest(paths):
     return max(os.path.getmtime(p) for p in paths)
 
 
+def units():
+    """(source, defines, object) of every translation unit: one for each csrc/*.cu, and
+    one for each length of the two that are compiled length by length."""
+    lengths = {}
+    with open(os.path.join(CSRC, "pp_lines_lengths.h")) as f:
+        for block in f.read().split("#define ")[1:]:
+            lengths[block.split("(")[0]] = re.findall(r"X\((\d+), (\d+), (\d+)\)", block)
+    each = {"pp_lines_unit.cu": "PP_LINE_LENGTHS", "pp_cart_unit.cu": "PP_CART_LENGTHS"}
+    out = []
+    # the longest lengths first: their kernels take the longest to compile
+    for name, group in each.items():
+        for n, n1, n2 in sorted(lengths[group], key=lambda t: -int(t[0])):
+            out.append((os.path.join(CSRC, name), ["-DPP_N1=" + n1, "-DPP_N2=" + n2],
+                        os.path.join(BUILD, "%s_%s.o" % (name[:-3], n))))
+    whole = [s for s in sorted(glob.glob(os.path.join(CSRC, "*.cu"))) if os.path.basename(s) not in each]
+    return [(s, [], os.path.join(BUILD, os.path.basename(s)[:-3] + ".o")) for s in whole] + out
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compile every csrc/*.cu in parallel and link libpp.so; returns its path."""
     nvcc = _nvcc()
@@ -36,11 +55,12 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         glob.glob(os.path.join(ROOT, "include", "*.h"))
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest(deps):
         return LIB
-    objs = [os.path.join(BUILD, os.path.basename(s)[:-3] + ".o") for s in srcs]
+    jobs = units()
+    objs = [obj for _, _, obj in jobs]
 
-    def compile_one(pair):
-        src, obj = pair
-        cmd = [nvcc, *ARCH, *FLAGS, "-c", src, "-o", obj]
+    def compile_one(job):
+        src, defines, obj = job
+        cmd = [nvcc, *ARCH, *FLAGS, *defines, "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("nvcc failed for %s:\n%s%s" % (src, r.stdout, r.stderr))
@@ -48,8 +68,8 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
             print(" ".join(cmd))
         return obj
 
-    with ThreadPoolExecutor(max_workers=max(1, min(len(srcs), os.cpu_count() or 1))) as ex:
-        list(ex.map(compile_one, zip(srcs, objs)))
+    with ThreadPoolExecutor(max_workers=max(1, min(len(jobs), os.cpu_count() or 1))) as ex:
+        list(ex.map(compile_one, jobs))
     tmp = LIB + ".tmp"
     cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-cudart", "static"]
     r = subprocess.run(cmd, capture_output=True, text=True)

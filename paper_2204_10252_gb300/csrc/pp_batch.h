@@ -102,6 +102,13 @@ struct RevCombine {
 size_t batch_normal_smem(int ny_max, int lgt);
 void* batch_normal_fn(int km, int lgt);
 pp_status configure_batch_kernels();
+// Columns per CTA that are compiled: 4 where the tile of one coil group leaves
+// room for two map buffers (n <= 256).
+// 8: the streaming form.
+constexpr bool cart_width_ok(int n, int W) { return W == 1 || W == 2 || W == 8 || (W == 4 && n <= 256); }
+// One launch for the length of (N1, N2); defined in that length's unit.
+template <int N1, int N2>
+cudaError_t cart_cols_launch(const CartLaunch& L, const float2* x, const CartChain& ch, cudaStream_t st);
 // Whether the column-resident kernel is compiled for length n and W columns.
 bool cart_cols_width_ok(int n, int W);
 pp_status launch_cart_cols(int n, CartLaunch L, const float2* x, const CartChain& ch, cudaStream_t st);

@@ -1,7 +1,8 @@
 // Choice and launch of the column-resident Cartesian kernels (pp_cart_cols.cuh).
 #include <algorithm>
 
-#include "pp_cart_cols.cuh"
+#include "pp_batch.h"
+#include "pp_lines_lengths.h"
 
 namespace pp {
 
@@ -9,9 +10,10 @@ namespace {
 
 struct Len {
     int n, n1, n2;
+    cudaError_t (*launch)(const CartLaunch&, const float2*, const CartChain&, cudaStream_t);
 };
-#define PP_LEN_ROW(n, a, b) {n, a, b},
-const Len kLens[] = {PP_CART_A(PP_LEN_ROW) PP_CART_B(PP_LEN_ROW) PP_CART_C(PP_LEN_ROW) PP_CART_D(PP_LEN_ROW)};
+#define PP_LEN_ROW(n, a, b) {n, a, b, cart_cols_launch<a, b>},
+const Len kLens[] = {PP_CART_LENGTHS(PP_LEN_ROW)};
 #undef PP_LEN_ROW
 
 const Len* find(int n) {
@@ -48,13 +50,7 @@ pp_status launch_cart_cols(int n, CartLaunch L, const float2* x, const CartChain
         const int ctas = L.items ? L.nitems : (L.one.nx + 7) / 8;
         while (L.slots < 4 && ctas * L.slots * 8 * l->n2 < 152 * 512 && L.max_coils >= 4 * L.slots) L.slots *= 2;
     }
-    cudaError_t e = cudaErrorInvalidValue;
-    if (l) {
-        e = cart_cols_launch_a(n, L, x, ch, st);
-        if (e == cudaErrorInvalidValue) e = cart_cols_launch_b(n, L, x, ch, st);
-        if (e == cudaErrorInvalidValue) e = cart_cols_launch_c(n, L, x, ch, st);
-        if (e == cudaErrorInvalidValue) e = cart_cols_launch_d(n, L, x, ch, st);
-    }
+    cudaError_t e = l ? l->launch(L, x, ch, st) : cudaErrorInvalidValue;
     if (e != cudaSuccess) return cuda_status(e, "cart_cols_kernel launch");
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e, "cart_cols_kernel");

@@ -352,11 +352,6 @@ cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
     if (follows) pdl_wait();
 }
 
-// Columns per CTA that are compiled: 4 where the tile of one coil group leaves
-// room for two map buffers (n <= 256).
-// 8: the streaming form.
-constexpr bool cart_width_ok(int n, int W) { return W == 1 || W == 2 || W == 8 || (W == 4 && n <= 256); }
-
 template <int N1, int N2>
 cudaError_t cart_cols_launch(const CartLaunch& L, const float2* x, const CartChain& ch, cudaStream_t st) {
     using K = CartCols<N1, N2>;
@@ -391,28 +386,5 @@ cudaError_t cart_cols_launch(const CartLaunch& L, const float2* x, const CartCha
         return go(cart_cols_kernel<N1, N2, 4>, allow_smem<cart_cols_kernel<N1, N2, 4>, kCartSmem>());
     return cudaErrorInvalidValue;
 }
-
-// (n, N1, N2) of every length with a compiled kernel, in four translation units
-#define PP_CART_A(X) X(32, 4, 8) X(36, 6, 6) X(40, 5, 8) X(48, 6, 8) X(60, 6, 10) X(64, 8, 8) X(72, 8, 9) X(80, 8, 10) X(96, 8, 12) X(100, 10, 10) X(108, 9, 12) X(120, 10, 12)
-#define PP_CART_B(X) X(128, 8, 16) X(144, 12, 12) X(160, 10, 16) X(180, 12, 15) X(192, 12, 16) X(200, 10, 20) X(216, 12, 18) X(240, 15, 16)
-#define PP_CART_C(X) X(256, 16, 16) X(288, 16, 18) X(300, 15, 20) X(320, 16, 20) X(324, 18, 18) X(360, 18, 20)
-#define PP_CART_D(X) X(384, 16, 24) X(400, 20, 20) X(432, 18, 24) X(480, 20, 24) X(500, 20, 25) X(512, 16, 32)
-
-// One of the four: launch or configure; cudaErrorInvalidValue where n is not in it.
-#define PP_CART_UNIT(NAME, LIST)                                                                   \
-    cudaError_t cart_cols_launch_##NAME(int n, const CartLaunch& L, const float2* x,               \
-                                        const CartChain& ch, cudaStream_t st) {                    \
-        switch (n) {                                                                               \
-            LIST(PP_CART_LAUNCH) default : return cudaErrorInvalidValue;                           \
-        }                                                                                          \
-    }
-#define PP_CART_LAUNCH(n, a, b) \
-    case n: return cart_cols_launch<a, b>(L, x, ch, st);
-
-#define PP_CART_DECL(NAME)                                                                       \
-    cudaError_t cart_cols_launch_##NAME(int n, const CartLaunch& L, const float2* x,             \
-                                        const CartChain& ch, cudaStream_t st);
-PP_CART_DECL(a) PP_CART_DECL(b) PP_CART_DECL(c) PP_CART_DECL(d)
-#undef PP_CART_DECL
 
 }  // namespace pp

@@ -1,14 +1,18 @@
 // Choice and launch of the compiled row and column FFT stages (pp_lines.cuh).
-#include "pp_lines.cuh"
+#include <algorithm>
+
+#include "pp_lines.h"
+#include "pp_lines_lengths.h"
 
 namespace pp {
 namespace {
 
 struct Len {
     int n, n1, n2;
+    cudaError_t (*launch)(LineOp, const LineUnion&, dim3, cudaStream_t);
 };
-#define PP_LINE_ROW(n, a, b) {n, a, b},
-const Len kLens[] = {PP_LINES_A(PP_LINE_ROW) PP_LINES_B(PP_LINE_ROW) PP_LINES_C(PP_LINE_ROW) PP_LINES_D(PP_LINE_ROW)};
+#define PP_LINE_ROW(n, a, b) {n, a, b, line_launch<a, b>},
+const Len kLens[] = {PP_LINE_LENGTHS(PP_LINE_ROW)};
 #undef PP_LINE_ROW
 
 const Len* find(int n) {
@@ -18,10 +22,7 @@ const Len* find(int n) {
 }
 
 pp_status go(const char* what, int n, LineOp op, const LineUnion& u, dim3 grid, cudaStream_t st) {
-    cudaError_t e = line_launch_a(n, op, u, grid, st);
-    if (e == cudaErrorInvalidValue) e = line_launch_b(n, op, u, grid, st);
-    if (e == cudaErrorInvalidValue) e = line_launch_c(n, op, u, grid, st);
-    if (e == cudaErrorInvalidValue) e = line_launch_d(n, op, u, grid, st);
+    cudaError_t e = find(n)->launch(op, u, grid, st);
     if (e != cudaSuccess) return cuda_status(e, what);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e, what);

@@ -15,52 +15,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <algorithm>
-
 #include "pp_fftgen.cuh"
-#include "pp_internal.h"
+#include "pp_lines.h"
 
 namespace pp {
-
-constexpr int TXG = 8;   // columns per CTA
-constexpr int RBG = 8;   // lines (rows, or rows x coils) per CTA in the row stages
-
-struct LineCols {
-    const float2* tw;
-    ColArgs a;
-    const ColItem* items;     // one per batch, or NULL: a's strides
-    const float2* src;
-    float2* dst;
-    const float2* ximg;       // XIMG: image multiplied into the input (batch b: image b % nimgs)
-    int nimgs;
-};
-struct LineRows {
-    const float2* tw;
-    RowArgs a;
-    const RowItem* items;     // one per (slice, coil) (forward) or slice (adjoint), or NULL
-    const float2* src;
-    int64_t src_batch_stride;
-    const float2* sens;
-    const float* wrow;
-    const float* wcol;
-    float2* dst;
-    const float2* operand;
-    float alpha;
-    int ncoils, rb;
-};
-struct LineYinv {
-    const float2* tw;
-    int nx;
-    int64_t nimg;
-    int ncoils;
-    const float2* W;
-    const float2* S;
-    float2* out;
-    int first, last;
-    float scale;
-    const float2* operand;
-    float alpha;
-};
 
 template <int N1, int N2> struct Line {
     static constexpr int n = N1 * N2, P = N2 | 1;
@@ -514,13 +472,6 @@ __global__ void __launch_bounds__(RBG * N2, line_min_ctas(RBG * N2)) line_rows_a
     }
 }
 
-// One launch of a stage for the length of (N1, N2).
-enum class LineOp { ColsFwd, ColsInv, ColsFwdImg, RoundTrip, Yinv, RowsFwd, RowsAdj };
-union LineUnion {
-    const LineCols* cols;
-    const LineRows* rows;
-    const LineYinv* yinv;
-};
 constexpr int kLineSmem = 200 * 1024;
 
 template <auto Kernel, class Args>
@@ -540,38 +491,24 @@ template <int N1, int N2> cudaError_t line_launch(LineOp op, const LineUnion& u,
             return line_go<line_cols_kernel<N1, N2, false, false>>(grid, K::cols_threads, K::cols_smem, st, *u.cols);
         case LineOp::ColsInv:
             return line_go<line_cols_kernel<N1, N2, true, false>>(grid, K::cols_threads, K::cols_smem, st, *u.cols);
+        case LineOp::RowsFwd:
+            return line_go<line_rows_fwd_kernel<N1, N2>>(grid, K::rows_threads, K::rows_smem, st, *u.rows);
+        case LineOp::RowsAdj:
+            return line_go<line_rows_adj_kernel<N1, N2>>(grid, K::rows_threads, K::rows_adj_smem(u.rows->a.n), st,
+                                                         *u.rows);
+        default: break;
+    }
+    // the 3-D normal operator's: image axes end at 512, only grids are longer
+    if constexpr (K::n <= 512) switch (op) {
         case LineOp::ColsFwdImg:
             return line_go<line_cols_kernel<N1, N2, false, true>>(grid, K::cols_threads, K::cols_smem, st, *u.cols);
         case LineOp::RoundTrip:
             return line_go<line_roundtrip_kernel<N1, N2>>(grid, K::cols_threads, K::cols_smem, st, *u.cols);
         case LineOp::Yinv:
             return line_go<line_yinv_kernel<N1, N2>>(grid, K::cols_threads, K::yinv_smem, st, *u.yinv);
-        case LineOp::RowsFwd:
-            return line_go<line_rows_fwd_kernel<N1, N2>>(grid, K::rows_threads, K::rows_smem, st, *u.rows);
-        default:
-            return line_go<line_rows_adj_kernel<N1, N2>>(grid, K::rows_threads, K::rows_adj_smem(u.rows->a.n), st,
-                                                         *u.rows);
+        default: break;
     }
+    return cudaErrorInvalidValue;
 }
-
-// (n, N1, N2) of every compiled length, in four translation units
-#define PP_LINES_A(X) X(16, 4, 4) X(18, 3, 6) X(20, 4, 5) X(24, 4, 6) X(30, 5, 6) X(32, 4, 8) X(36, 6, 6) X(40, 5, 8) X(48, 6, 8) X(50, 5, 10) X(54, 6, 9) X(60, 6, 10) X(64, 8, 8) X(72, 8, 9) X(80, 8, 10) X(90, 9, 10) X(96, 8, 12) X(100, 10, 10) X(108, 9, 12) X(120, 10, 12)
-#define PP_LINES_B(X) X(128, 8, 16) X(144, 12, 12) X(150, 10, 15) X(160, 10, 16) X(162, 9, 18) X(180, 12, 15) X(192, 12, 16) X(200, 10, 20) X(216, 12, 18) X(240, 15, 16) X(250, 10, 25) X(256, 16, 16) X(270, 15, 18)
-#define PP_LINES_C(X) X(288, 16, 18) X(300, 15, 20) X(320, 16, 20) X(324, 18, 18) X(360, 18, 20) X(384, 16, 24) X(400, 20, 20) X(432, 18, 24) X(450, 18, 25) X(480, 20, 24) X(486, 18, 27) X(500, 20, 25) X(512, 16, 32)
-#define PP_LINES_D(X) X(540, 20, 27) X(576, 24, 24) X(600, 24, 25) X(640, 20, 32) X(648, 24, 27) X(720, 24, 30) X(750, 25, 30) X(768, 24, 32) X(800, 25, 32) X(810, 27, 30) X(864, 27, 32) X(900, 30, 30) X(960, 30, 32) X(1024, 32, 32)
-
-#define PP_LINES_CASE(n, a, b) \
-    case n: return line_launch<a, b>(op, u, grid, st);
-// cudaErrorInvalidValue where n is not in the unit
-#define PP_LINES_UNIT(NAME, LIST)                                                                         \
-    cudaError_t line_launch_##NAME(int n, LineOp op, const LineUnion& u, dim3 grid, cudaStream_t st) {    \
-        switch (n) {                                                                                      \
-            LIST(PP_LINES_CASE) default : return cudaErrorInvalidValue;                                   \
-        }                                                                                                 \
-    }
-cudaError_t line_launch_a(int n, LineOp op, const LineUnion& u, dim3 grid, cudaStream_t st);
-cudaError_t line_launch_b(int n, LineOp op, const LineUnion& u, dim3 grid, cudaStream_t st);
-cudaError_t line_launch_c(int n, LineOp op, const LineUnion& u, dim3 grid, cudaStream_t st);
-cudaError_t line_launch_d(int n, LineOp op, const LineUnion& u, dim3 grid, cudaStream_t st);
 
 }  // namespace pp
