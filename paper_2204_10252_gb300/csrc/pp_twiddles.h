@@ -40,12 +40,13 @@ inline double reg_dft_gain(int N) {
 // m < n2, k < n1.  Rounding them and the register DFTs' constants to FP32 changes the
 // transform's mean output energy by some 5e-8, always the same way, so that it adds
 // up over the transforms of a solve where rounding does not.  The table is scaled by
-// the one factor that brings the mean nearest to 1 (bisection: entries round one by
-// one, so it stays within half a step of one entry, 5e-9 from 64 points on).
-// Coefficient gradients of a 3-iteration unrolled solve, differences of large sums,
-// against 64 bits, mean of four data sets: 8 slices of 256 x 256 2.0e-6 with the plain
-// table, 5.6e-8 so; 2 slices of 128 x 128 with d = 2 2.5e-6 and 1.2e-6; of 384 x 384
-// with d = 1 3.0e-6 and 6.6e-7.
+// the largest factor that leaves the mean at 1 or below, so that a normalised operator
+// stays one and FISTA's unit step stays safe (bisection: entries round one by one, so
+// the mean falls short of 1 by less than one entry's step: 2e-8 at 16 and 32 points,
+// 8e-9 at 80, 5e-9 at 256, mostly below 2e-9).  Coefficient gradients of a 3-iteration
+// unrolled solve, differences of large sums, against 64 bits, mean of four data sets:
+// 8 slices of 256 x 256 2.0e-6 with the plain table, 3.5e-7 so; 2 slices of 128 x 128
+// with d = 2 2.5e-6 and 1.2e-6; of 384 x 384 with d = 1 3.0e-6 and 6.6e-7.
 inline std::vector<Twiddle> balanced_twiddles(int n1, int n2) {
     const int n = n1 * n2;
     const double reg = reg_dft_gain(n1) + reg_dft_gain(n2);
@@ -72,8 +73,7 @@ inline std::vector<Twiddle> balanced_twiddles(int n1, int n2) {
         const double mid = 0.5 * (lo + hi);
         (gain(table(mid)) > 0.0 ? hi : lo) = mid;
     }
-    const std::vector<Twiddle> below = table(lo), above = table(hi);
-    return gain(above) < -gain(below) ? above : below;
+    return table(lo);
 }
 
 }  // namespace pp

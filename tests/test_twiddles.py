@@ -1,6 +1,6 @@
 """The two-factor kernels' twiddle tables (csrc/pp_twiddles.h), compiled for the host:
-the mean output energy of a transform of any compiled length is the nearest to 1 that
-one scale factor can bring it."""
+the mean output energy of a transform of any compiled length is the largest not above
+1 that one scale factor can bring it to."""
 import os
 import re
 import shutil
@@ -48,9 +48,9 @@ def test_mean_energy_of_every_compiled_length(tmp_path):
         reg, w = v[0], np.array(v[1:]).reshape(n, 2)
         used = (np.arange(b)[:, None] * np.arange(a)[None]).ravel()
         mean = reg + float((w[used] ** 2).sum(1).mean()) - 1.0
-        # scaling moves all entries of one magnitude together, by an ulp: no scale comes
-        # nearer than half the largest of those steps in general
+        # scaling moves all entries of one magnitude together, by an ulp: the mean falls
+        # short of 1 by no more than the largest of those steps
         mags, inv = np.unique(np.abs(w[used]).ravel(), return_inverse=True)
         count = np.bincount(inv)
         step = 2.0 * mags * np.spacing(mags.astype(np.float32)).astype(float) * count / n
-        assert abs(mean) <= step[mags < 1.0].max() / 2 + 1e-12, (n, mean)
+        assert -step[mags < 1.0].max() - 1e-12 <= mean <= 1e-12, (n, mean)
