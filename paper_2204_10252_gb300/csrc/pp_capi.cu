@@ -89,6 +89,17 @@ static pp_status alloc_n(Plan& p, T** ptr, size_t n) {
     return dev_alloc(p, reinterpret_cast<void**>(ptr), n * sizeof(T));
 }
 
+// The balanced table of a length, kept for the life of the process (60 lengths at
+// most): a batch makes two a slice.
+static const std::vector<Twiddle>& twiddles_of(int n, const GenSplit& g) {
+    static std::mutex mu;
+    static std::map<int, std::vector<Twiddle>> kept;
+    std::lock_guard<std::mutex> lock(mu);
+    std::vector<Twiddle>& tw = kept[n];
+    if (tw.empty()) tw = balanced_twiddles(g.n1, g.n2);
+    return tw;
+}
+
 static pp_status make_fft(Plan& p, int n, DevFft& f) {
     if (!factorize(n, f.d)) {
         set_error("FFT length %d has a prime factor above 5", n);
@@ -99,15 +110,12 @@ static pp_status make_fft(Plan& p, int n, DevFft& f) {
         const double a = -2.0 * M_PI * (double)t / (double)n;
         tw[t] = make_float2((float)cos(a), (float)sin(a));
     }
-    PP_TRY(alloc_n(p, &f.tw, n));
-    PP_TRY_CUDA(cudaMemcpy(f.tw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
     const GenSplit g = gen_split_of(n);
-    f.twb = f.tw;
-    if (g.n1) {
-        const std::vector<Twiddle> twb = balanced_twiddles(g.n1, g.n2);
-        PP_TRY(alloc_n(p, &f.twb, n));
-        PP_TRY_CUDA(cudaMemcpy(f.twb, twb.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
-    }
+    if (g.n1)   // both tables in one array
+        for (const Twiddle& w : twiddles_of(n, g)) tw.push_back(make_float2(w.x, w.y));
+    PP_TRY(alloc_n(p, &f.tw, tw.size()));
+    PP_TRY_CUDA(cudaMemcpy(f.tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice));
+    f.twb = g.n1 ? f.tw + n : f.tw;
     return PP_OK;
 }
 
@@ -801,7 +809,8 @@ static pp_status tune_cart3d(Plan& p, cudaStream_t st) {
 
 // 2-D Cartesian: the columns per CTA of the column-resident kernel, timed on the
 // plan's buffers as one application and as a chain of three (a preconditioned
-// gradient of degree 2); the fastest sum is kept.
+// gradient of degree 2); the fastest sum is kept.  A second round re-times the
+// candidates within 10 % of the first one's best.
 static pp_status tune_cart2d(Plan& p, cudaStream_t st) {
     p.cols = cart_cols_width_ok(p.ny, 1);
     if (!p.cols) return PP_OK;   // the Stockham kernel
@@ -818,21 +827,25 @@ static pp_status tune_cart2d(Plan& p, cudaStream_t st) {
     three.v_first = 1;
     three.J = 3;
     for (int j = 0; j < 3; ++j) three.sc[j] = three.al[j] = 1.f;
-    for (int round = 0; round < 3; ++round)
+    auto pass = [&]() {
+        PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
+        return cart_chain(p, p.v, three, st);
+    };
+    for (int round = 0; round < 2; ++round) {
+        const float cut = round == 0 ? 2e30f : 1.1f * *std::min_element(best.begin(), best.end());
         for (size_t i = 0; i < cand.size(); ++i) {
+            if (best[i] > cut) continue;
             p.tune_c2 = cand[i];
-            PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
+            PP_TRY(pass());
             PP_TRY_CUDA(cudaEventRecord(e0, st));
-            for (int r = 0; r < 5; ++r) {
-                PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
-                PP_TRY(cart_chain(p, p.v, three, st));
-            }
+            for (int r = 0; r < 4; ++r) PP_TRY(pass());
             PP_TRY_CUDA(cudaEventRecord(e1, st));
             PP_TRY_CUDA(cudaEventSynchronize(e1));
             float ms = 0.f;
             PP_TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
             best[i] = std::min(best[i], ms);
         }
+    }
     p.tune_c2 = cand[std::min_element(best.begin(), best.end()) - best.begin()];
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1252,17 +1265,15 @@ static bool cols_supported(const Batch& b) {
         if (!cart_cols_width_ok(d.ny, 1)) return false;
     return !b.hdesc.empty();
 }
-static void drop_groups(Batch& b) {
-    for (CartGroup& g : b.dev.groups)
-        if (g.items) {
-            cudaFree(g.items);
-            b.allocs.erase(std::remove(b.allocs.begin(), b.allocs.end(), (void*)g.items), b.allocs.end());
-        }
-    b.dev.groups.clear();
-    b.dev.cols = 0;
+// One upload holds the lists of all lengths: groups[0].items is its start.
+static void free_groups(Batch& b, std::vector<CartGroup>& groups) {
+    if (!groups.empty()) {
+        cudaFree(groups[0].items);
+        b.allocs.erase(std::remove(b.allocs.begin(), b.allocs.end(), (void*)groups[0].items), b.allocs.end());
+    }
+    groups.clear();
 }
-static pp_status set_cols(Batch& b, int W) {
-    drop_groups(b);
+static pp_status make_groups(Batch& b, int W, std::vector<CartGroup>* out) {
     std::map<int, std::vector<std::pair<int, int2>>, std::greater<int>> by_len;
     std::map<int, CartGroup> info;
     for (int s = 0; s < b.n; ++s) {
@@ -1274,32 +1285,51 @@ static pp_status set_cols(Batch& b, int W) {
         g.max_coils = std::max(g.max_coils, d.C);
         for (int c0 = 0; c0 < d.nx; c0 += g.W) by_len[d.ny].push_back({d.C, make_int2(s, c0)});
     }
-    int total = 0;
+    std::vector<int2> items;
+    std::vector<CartGroup> groups;
     for (auto& e : by_len) {
         std::stable_sort(e.second.begin(), e.second.end(),
                          [](const std::pair<int, int2>& a, const std::pair<int, int2>& c) {
                              return a.first > c.first;
                          });
-        std::vector<int2> items;
         for (auto& it : e.second) items.push_back(it.second);
         CartGroup g = info[e.first];
-        g.nitems = (int)items.size();
-        total += g.nitems;
-        PP_TRY(bupload(b, &g.items, items));
-        b.dev.groups.push_back(g);
+        g.nitems = (int)e.second.size();
+        groups.push_back(g);
     }
-    b.dev.cols = W;
-    b.dev.grid = total;
+    int2* all = nullptr;
+    PP_TRY(bupload(b, &all, items));
+    for (CartGroup& g : groups) {
+        g.items = all;
+        all += g.nitems;
+    }
+    *out = groups;
+    return PP_OK;
+}
+static void use_groups(Batch& b, int W, const std::vector<CartGroup>& groups) {
+    b.dev.groups = groups;
+    b.dev.cols = groups.empty() ? 0 : W;
+    b.dev.grid = 0;
+    for (const CartGroup& g : groups) b.dev.grid += g.nitems;
+}
+static void drop_groups(Batch& b) {
+    free_groups(b, b.dev.groups);
+    b.dev.cols = 0;
+}
+static pp_status set_cols(Batch& b, int W) {
+    std::vector<CartGroup> groups;
+    PP_TRY(make_groups(b, W, &groups));
+    drop_groups(b);
+    use_groups(b, W, groups);
     return PP_OK;
 }
 
 // Batch autotuner: the columns per CTA of the column-resident kernels (one
 // application and a chain of three, as for a single plan) where every slice
-// length has one, else the tile width of the Stockham kernel.
+// length has one, else the tile width of the Stockham kernel.  One pass each, then
+// about 0.4 ms of passes for those within 20 % of the best.
 static pp_status autotune(Batch& b, cudaStream_t st) {
     std::vector<int2> items;
-    int best = -1;
-    float best_ms = 1e30f;
     cudaEvent_t e0, e1;
     PP_TRY_CUDA(cudaEventCreate(&e0));
     PP_TRY_CUDA(cudaEventCreate(&e1));
@@ -1309,36 +1339,46 @@ static pp_status autotune(Batch& b, cudaStream_t st) {
     three.v_first = 1;
     three.J = 3;
     for (int j = 0; j < 3; ++j) three.sc[j] = three.al[j] = 1.f;
-    for (int v : cols ? std::vector<int>{1, 4, 8} : std::vector<int>{2, 3, 4}) {
-        if (cols) {
-            PP_TRY(set_cols(b, v));
-        } else {
-            if (!km_for(b.dev.ny_max, v)) continue;
-            PP_TRY(set_items(b, v, &items));
-        }
-        auto pass = [&]() {
-            PP_TRY(launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st));
-            return cols ? launch_batch_chain(b.dev, b.v, three, st) : PP_OK;
-        };
-        PP_TRY(pass());
-        PP_TRY_CUDA(cudaEventRecord(e0, st));
-        for (int r = 0; r < 3; ++r) PP_TRY(pass());
-        PP_TRY_CUDA(cudaEventRecord(e1, st));
-        PP_TRY_CUDA(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best_ms) {
-            best_ms = ms;
-            best = v;
+    std::vector<int> cand;
+    for (int v : cols ? std::vector<int>{1, 4, 8} : std::vector<int>{2, 3, 4})
+        if (cols || km_for(b.dev.ny_max, v)) cand.push_back(v);
+    if (cand.empty()) {
+        set_error("no batched kernel fits ny_max = %d", b.dev.ny_max);
+        return PP_ERR_UNSUPPORTED;
+    }
+    std::vector<std::vector<CartGroup>> lists(cand.size());
+    if (cols)
+        for (size_t i = 0; i < cand.size(); ++i) PP_TRY(make_groups(b, cand[i], &lists[i]));
+    auto pass = [&]() {
+        PP_TRY(launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st));
+        return cols ? launch_batch_chain(b.dev, b.v, three, st) : PP_OK;
+    };
+    std::vector<float> best(cand.size(), 1e30f);
+    for (int round = 0; round < 2; ++round) {
+        const float lead = *std::min_element(best.begin(), best.end());
+        const int reps = round == 0 ? 1 : std::max(1, std::min(8, (int)(0.4f / lead)));
+        for (size_t i = 0; i < cand.size(); ++i) {
+            if (round > 0 && best[i] > 1.2f * lead) continue;
+            if (cols) use_groups(b, cand[i], lists[i]);
+            else PP_TRY(set_items(b, cand[i], &items));
+            if (round == 0) PP_TRY(pass());
+            PP_TRY_CUDA(cudaEventRecord(e0, st));
+            for (int r = 0; r < reps; ++r) PP_TRY(pass());
+            PP_TRY_CUDA(cudaEventRecord(e1, st));
+            PP_TRY_CUDA(cudaEventSynchronize(e1));
+            float ms = 0.f;
+            PP_TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+            best[i] = std::min(best[i], ms / reps);
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (best < 0) {
-        set_error("no batched kernel fits ny_max = %d", b.dev.ny_max);
-        return PP_ERR_UNSUPPORTED;
-    }
-    return cols ? set_cols(b, best) : set_items(b, best, &items);
+    const size_t win = std::min_element(best.begin(), best.end()) - best.begin();
+    if (!cols) return set_items(b, cand[win], &items);
+    use_groups(b, cand[win], lists[win]);
+    for (size_t i = 0; i < cand.size(); ++i)
+        if (i != win) free_groups(b, lists[i]);
+    return PP_OK;
 }
 
 static pp_status batch_power_iteration(Batch& b, uint64_t seed, int iters, cudaStream_t st) {

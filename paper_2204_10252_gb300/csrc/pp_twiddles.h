@@ -50,22 +50,25 @@ inline double reg_dft_gain(int N) {
 inline std::vector<Twiddle> balanced_twiddles(int n1, int n2) {
     const int n = n1 * n2;
     const double reg = reg_dft_gain(n1) + reg_dft_gain(n2);
+    std::vector<double> c(n), s(n);
+    std::vector<int> used(n, 0);   // products that take entry t
+    for (int t = 0; t < n; ++t) {
+        const double a = -2.0 * 3.14159265358979323846 * (double)t / (double)n;
+        c[t] = std::cos(a);
+        s[t] = std::sin(a);
+    }
+    for (int m = 0; m < n2; ++m)
+        for (int k = 0; k < n1; ++k) ++used[m * k];
     auto table = [&](double scale) {
         std::vector<Twiddle> tw(n);
-        for (int t = 0; t < n; ++t) {
-            const double a = -2.0 * 3.14159265358979323846 * (double)t / (double)n;
-            tw[t] = {(float)(scale * std::cos(a)), (float)(scale * std::sin(a))};
-        }
+        for (int t = 0; t < n; ++t) tw[t] = {(float)(scale * c[t]), (float)(scale * s[t])};
         tw[0] = {1.f, 0.f};
         return tw;
     };
     auto gain = [&](const std::vector<Twiddle>& tw) {
         double e = 0.0;
-        for (int m = 0; m < n2; ++m)
-            for (int k = 0; k < n1; ++k) {
-                const Twiddle w = tw[m * k];
-                e += (double)w.x * w.x + (double)w.y * w.y - 1.0;
-            }
+        for (int t = 0; t < n; ++t)
+            e += used[t] * ((double)tw[t].x * tw[t].x + (double)tw[t].y * tw[t].y - 1.0);
         return reg + e / n;
     };
     double lo = 1.0 - 5e-7, hi = 1.0 + 5e-7;
