@@ -1878,9 +1878,9 @@ pp_status pp_plan_create(pp_plan** out, pp_dims dims, int coils, const pp_c64* s
         set_error("pp_plan_create: unknown sampling kind %d", s->kind);
         return PP_ERR_INVALID_ARG;
     }
-    static std::once_flag once;
-    static pp_status cfg = PP_OK;
-    std::call_once(once, [] { cfg = configure_kernels(); });
+    static PerDevice configured;
+    pp_status cfg = PP_OK;
+    configured.get(current_device(), [&] { return (cfg = configure_kernels()) == PP_OK ? 0 : -1; });
     if (cfg != PP_OK) return cfg;
 
     pp_plan* h = new pp_plan();
@@ -2557,11 +2557,12 @@ pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, cons
             return PP_ERR_UNSUPPORTED;
         }
     }
-    static std::once_flag once;
-    static pp_status cfg = PP_OK;
-    std::call_once(once, [] {
+    static PerDevice configured;
+    pp_status cfg = PP_OK;
+    configured.get(current_device(), [&] {
         cfg = configure_kernels();
         if (cfg == PP_OK) cfg = configure_batch_kernels();
+        return cfg == PP_OK ? 0 : -1;
     });
     if (cfg != PP_OK) return cfg;
     cudaStream_t st = (cudaStream_t)stream;

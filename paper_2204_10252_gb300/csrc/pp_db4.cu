@@ -370,21 +370,17 @@ size_t db4_cluster_smem(int nx, int ny, int levels, int R) {
     const int units = ny >> levels, slab = ((units + R - 1) / R) << levels;
     return sizeof(float2) * ((size_t)2 * slab * nx + (size_t)4 * levels * nx);
 }
-int db4_cluster_size(int nx, int ny, int levels) {
-    constexpr int kSmem = 220 * 1024;
-    static const cudaError_t allowed = [] {
-        cudaError_t e = cudaFuncSetAttribute(db4_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+constexpr int kDb4Smem = 220 * 1024;
+// Largest cluster that the current device takes: 16, 8 (the portable size), or 0
+// when the kernel's attributes are refused.
+int db4_largest_cluster() {
+    static PerDevice largest;
+    return largest.get(current_device(), [] {
+        cudaError_t e = cudaFuncSetAttribute(db4_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDb4Smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(db4_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaGetLastError();
-        return e;
-    }();
-    if (allowed != cudaSuccess) return 0;
-    const int units = ny >> levels;
-    int R = (int64_t)nx * ny > 128 * 128 ? 16 : 8;
-    while (R > units) R >>= 1;
-    if (db4_cluster_smem(nx, ny, levels, R) > (size_t)kSmem) return 0;
-    static const bool sixteen = [] {
+        if (e != cudaSuccess) return 0;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -392,19 +388,22 @@ int db4_cluster_size(int nx, int ny, int levels) {
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(16);
         cfg.blockDim = dim3(kDb4Threads);
-        cfg.dynamicSmemBytes = kSmem;
+        cfg.dynamicSmemBytes = kDb4Smem;
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, db4_cluster_kernel, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&n, db4_cluster_kernel, &cfg);
         cudaGetLastError();
-        return e == cudaSuccess && n > 0;
-    }();
-    if (R == 16 && !sixteen) {
-        R = 8;
-        if (db4_cluster_smem(nx, ny, levels, R) > (size_t)kSmem) return 0;
-    }
-    return R;
+        return e == cudaSuccess && n > 0 ? 16 : 8;
+    });
+}
+int db4_cluster_size(int nx, int ny, int levels) {
+    const int largest = db4_largest_cluster();
+    if (!largest) return 0;
+    const int units = ny >> levels;
+    int R = (int64_t)nx * ny > 128 * 128 ? largest : 8;
+    while (R > units) R >>= 1;
+    return db4_cluster_smem(nx, ny, levels, R) <= (size_t)kDb4Smem ? R : 0;
 }
 
 pp_status check_db4(const char* what) {
@@ -461,7 +460,7 @@ pp_status db4_prox(int nx, int ny, int levels, float lambda, const float2* in, c
 
 }  // namespace
 
-void db4_prepare() { (void)db4_cluster_size(64, 64, 1); }
+void db4_prepare() { (void)db4_largest_cluster(); }
 
 bool db4_supported(int ndim, int nx, int ny, int levels) {
     return ndim == 2 && levels >= 1 && levels <= 4 && nx <= MAXN && ny <= MAXN && nx > 0 && ny > 0 &&

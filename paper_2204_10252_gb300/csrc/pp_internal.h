@@ -9,6 +9,7 @@
 
 #include "pp.h"
 #include "pp_fft.cuh"
+#include "pp_per_device.h"
 
 namespace pp {
 
@@ -69,9 +70,19 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Raises a kernel's dynamic shared memory limit to `bytes`, once.
+inline int current_device() {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+
+// Raises a kernel's dynamic shared memory limit to `bytes`, once on each device.
 template <auto Kernel, int bytes> cudaError_t allow_smem() {
-    static const cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    static PerDevice done;
+    cudaError_t e = cudaSuccess;
+    done.get(current_device(), [&] {
+        e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        return e == cudaSuccess ? 0 : -1;
+    });
     return e;
 }
 
