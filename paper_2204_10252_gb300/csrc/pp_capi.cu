@@ -41,6 +41,7 @@ void set_error(const char* fmt, ...) {
 
 pp_status cuda_status(cudaError_t e, const char* what) {
     set_error("%s: %s", what, cudaGetErrorString(e));
+    cudaGetLastError();   // a refused launch is not to be found by the next one's check
     return e == cudaErrorMemoryAllocation ? PP_ERR_OOM : PP_ERR_CUDA;
 }
 
