@@ -122,6 +122,16 @@ typedef struct pp_plan pp_plan;
  * trajectory's or the mask's bytes), so a later plan of the same geometry
  * takes it without timing again.  Non-Cartesian set-up computes the
  * per-sample gridding taps and tile lists on up to 16 host threads.
+ * Device memory beside `sens`: 8 images, and
+ *   2-D Cartesian    the k-space, 8*C*ny*nx bytes;
+ *   3-D              the planes of as many coils as fit 512 MB (one at least), fewer
+ *                    where those would take over half of the free memory; one more
+ *                    volume when ny or nz is below 16; the dataflow operator's slots;
+ *   non-Cartesian    8*C*Gx*(ny + 2*Gy), the weight planes (about 400*Gx*Gy), 80 bytes
+ *                    a sample, and a transposed k-space of 8 bytes a sample and coil
+ *                    (coils rounded up to 8, 16 or a multiple of 32) unless that would
+ *                    take over half of the free memory; up to 32 coils on
+ *                    register-FFT grids also coil-innermost copies.
  * Synchronises `stream` (the set-up work is complete on return).  On
  * failure *out is NULL. */
 pp_status pp_plan_create(pp_plan** out, pp_dims dims, int coils, const pp_c64* sens,
@@ -389,7 +399,10 @@ pp_status pp_fista_solve_prox(pp_plan* plan, const pp_c64* b, const pp_c64* v, d
 typedef struct pp_batch pp_batch;
 
 /* Build a batch; power_iters > 0 estimates every L_s (one seed per slice:
- * seed + s).  Synchronises `stream`. */
+ * seed + s).  Device memory: 8 images of the whole batch and an adjoint workspace of
+ * 72 MB or the batch's k-space, whichever is less, but at least the largest slice's
+ * k-space (and no more than that where 72 MB is over half of what is free).
+ * Synchronises `stream`. */
 pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, const int* coils,
                           const pp_c64* const* sens, const uint8_t* const* masks, uint64_t seed,
                           int power_iters, pp_stream stream);

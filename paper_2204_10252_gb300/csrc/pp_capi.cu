@@ -90,6 +90,17 @@ static pp_status alloc_n(Plan& p, T** ptr, size_t n) {
     return dev_alloc(p, reinterpret_cast<void**>(ptr), n * sizeof(T));
 }
 
+// A workspace that only makes things faster: NULL, and no error, where it would take
+// more than half of the free memory.
+static void* spare_alloc(size_t bytes) {
+    size_t room = 0, total = 0;
+    void* ptr = nullptr;
+    if (cudaMemGetInfo(&room, &total) == cudaSuccess && bytes <= room / 2 && cudaMalloc(&ptr, bytes) == cudaSuccess)
+        return ptr;
+    cudaGetLastError();
+    return nullptr;
+}
+
 // The balanced table of a length, kept for the life of the process (60 lengths at
 // most): a batch makes two a slice.
 static const std::vector<Twiddle>& twiddles_of(int n, const GenSplit& g) {
@@ -417,18 +428,30 @@ static pp_status build_cartesian(Plan& p, const uint8_t* mask) {
     } else if (p.ndim == 2) {
         PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.C * p.nimg));
     } else {
-        // Coils of one launch of each stage: 512 MB of planes.  Planes that fit L2
-        // together (72 MB) leave each launch short: the stages read little back from
-        // L2 (26 % hits), and every launch ends in a part wave and, in the adjoint,
-        // adds to the image.  80 x 180 x 200 x 12, forward + adjoint / normal: 862 /
-        // 502 us at 72 MB, 789 / - at 200, 746 / 429 at 512 and above; 128 x 200 x 200
-        // x 9, normal: 1090 -> 650.
-        p.c3_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(p.C, (512ll << 20) / (8 * p.nimg)));
-        PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.c3_chunk * p.nimg));
-        PP_TRY(alloc_n(p, &p.wk_b, (size_t)p.nimg));
+        PP_TRY(alloc_n(p, &p.wk_a, (size_t)p.nimg));   // see widen_c3
+        // the passes for axes without compiled stages alternate between two volumes
+        if (!lines_have(ny) || !lines_have(nz)) PP_TRY(alloc_n(p, &p.wk_b, (size_t)p.nimg));
     }
     p.nksp = (int64_t)p.C * p.nimg;
     return PP_OK;
+}
+
+// 3-D: coils of one launch of each stage, 512 MB of planes, or the half, the quarter ..
+// of them where the memory is short.  Planes that fit L2 together (72 MB) leave each
+// launch short: the stages read little back from L2 (26 % hits), and every launch ends
+// in a part wave and, in the adjoint, adds to the image.  80 x 180 x 200 x 12, forward +
+// adjoint / normal: 862 / 502 us at 72 MB, 789 / - at 200, 746 / 429 at 512 and above;
+// 128 x 200 x 200 x 9, normal: 1090 -> 650.
+static void widen_c3(Plan& p) {
+    const int64_t volume = p.nimg * (int64_t)sizeof(float2);
+    for (int c = (int)std::min<int64_t>(p.C, (512ll << 20) / volume); c > 1; c = (c + 1) / 2)
+        if (void* w = spare_alloc((size_t)(c * volume))) {
+            cudaFree(p.wk_a);
+            std::replace(p.allocs.begin(), p.allocs.end(), (void*)p.wk_a, w);
+            p.wk_a = static_cast<float2*>(w);
+            p.c3_chunk = c;
+            return;
+        }
 }
 
 static pp_status build_noncartesian(Plan& p, const pp_sampling* s) {
@@ -563,7 +586,6 @@ static pp_status build_noncartesian(Plan& p, const pp_sampling* s) {
         PP_TRY(upload(p, &p.sort_wx, wx));
         PP_TRY(upload(p, &p.sort_wy, wy));
         PP_TRY(upload(p, &p.sort_kx, kx));
-        PP_TRY(alloc_n(p, &p.ksp_t, nufft_transposed_elems(p)));
     }
     // G^T G as (2W-1)^2 weight planes (FP64 sums of the taps' pairwise
     // products, stored FP32), in both layouts, built on the device
@@ -1933,10 +1955,18 @@ pp_status pp_plan_create(pp_plan** out, pp_dims dims, int coils, const pp_c64* s
                          ? PP_OK : cuda_status(cudaGetLastError(), "cudaMemsetAsync");
             p.c3df_cg = std::min(4, p.C);
         }
+        if (rc == PP_OK) widen_c3(p);
         if (rc == PP_OK && !(tuned = tune_lookup(tkey, p))) rc = tune_cart3d(p, st);
     }
     if (rc == PP_OK && p.kind == PP_NONCARTESIAN) rc = setup_ci(p, st);
     if (rc == PP_OK && p.toep) rc = setup_toeplitz(p, s, st);
+    if (rc == PP_OK && p.kind == PP_NONCARTESIAN) {
+        // the spread's transposed k-space; without it the spread reads [C][K] in place
+        if (void* w = spare_alloc(nufft_transposed_elems(p) * sizeof(float2))) {
+            p.allocs.push_back(w);
+            p.ksp_t = static_cast<float2*>(w);
+        }
+    }
     if (rc == PP_OK && p.kind == PP_NONCARTESIAN && !p.toep && !(tuned = tune_lookup(tkey, p)))
         rc = tune_noncartesian(p, st);
     if (rc == PP_OK && !tuned) tune_store(tkey, p);
@@ -2599,11 +2629,6 @@ pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, cons
     }
     b.nimg = b.img_off[nslices];
     b.nksp = b.ksp_off[nslices];
-    // adjoint workspace: the largest slice, and more of them up to half of the L2
-    const size_t wk = std::max(wk_max, std::min((size_t)b.nksp, (size_t)(72 << 20) / sizeof(float2)));
-    if (rc == PP_OK) rc = balloc(b, &b.wk, wk);
-    if (rc == PP_OK)
-        for (Plan* p : b.sub) p->wk_a = b.wk;
     const size_t n = (size_t)b.nimg;
     if (rc == PP_OK && (rc = balloc(b, &b.z, n)) == PP_OK && (rc = balloc(b, &b.y, n)) == PP_OK &&
         (rc = balloc(b, &b.g, n)) == PP_OK && (rc = balloc(b, &b.u, n)) == PP_OK &&
@@ -2626,6 +2651,19 @@ pp_status pp_batch_create(pp_batch** out, int nslices, const pp_dims* dims, cons
     if (rc == PP_OK) {
         cudaError_t e = cudaMemsetAsync(b.v, 0, n * sizeof(float2), st);
         if (e != cudaSuccess) rc = cuda_status(e, "cudaMemsetAsync");
+    }
+    // adjoint workspace: as many slices as fit half of the L2 together, where there is
+    // memory for them, but at least the largest
+    size_t wk = std::max(wk_max, std::min((size_t)b.nksp, (size_t)(72 << 20) / sizeof(float2)));
+    if (rc == PP_OK) {
+        if (void* w = wk > wk_max ? spare_alloc(wk * sizeof(float2)) : nullptr) {
+            b.allocs.push_back(w);
+            b.wk = static_cast<float2*>(w);
+        } else {
+            wk = wk_max;
+            rc = balloc(b, &b.wk, wk);
+        }
+        for (Plan* p : b.sub) p->wk_a = b.wk;
     }
     if (rc == PP_OK) rc = plan_lines(b, wk);
     if (rc == PP_OK) rc = autotune(b, st);
