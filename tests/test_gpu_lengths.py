@@ -108,3 +108,85 @@ def test_column_resident_batch_of_mixed_lengths(pp, tile):
             assert np.linalg.norm(g - ref) <= TOL_APPLY * np.linalg.norm(ref)
     finally:
         b.destroy()
+
+
+# image axes (multiples of 4 up to 512), and the other compiled lengths as grids of an
+# image axis n oversampled by s: (length, n, s, n and length of the other axis)
+AXES = [16, 20, 24, 32, 36, 40, 48, 60, 64, 72, 80, 96, 100, 108, 120, 128, 144, 160, 180, 192, 200, 216, 240, 256, 288,
+        300, 320, 324, 360, 384, 400, 432, 480, 500, 512]
+GRIDS = [(50, 40, 1.25), (54, 48, 1.125), (90, 72, 1.25), (150, 120, 1.25), (162, 144, 1.125), (250, 200, 1.25),
+         (270, 240, 1.125), (450, 360, 1.25), (486, 432, 1.125), (540, 480, 1.125), (576, 512, 1.125), (600, 480, 1.25),
+         (640, 512, 1.25), (648, 324, 2.0), (720, 360, 2.0), (750, 500, 1.5), (768, 384, 2.0), (800, 400, 2.0),
+         (810, 432, 1.875), (864, 432, 2.0), (900, 480, 1.875), (960, 480, 2.0), (1024, 512, 2.0)]
+
+
+@pytest.mark.parametrize("n", AXES)
+def test_row_and_column_stages_at_every_image_length(pp, n):
+    """Forward and adjoint with rows and with columns of every compiled image length,
+    beside 20 points (three rows or columns past a group of eight), three coils."""
+    import torch
+    for shape in ((n, 20), (20, n)):
+        sens = synth.coil_maps(shape, 3, 31)
+        mask = synth.line_mask(shape, 2, 4, 32)
+        x, y = synth.crandn(shape, 33), synth.crandn((3,) + shape, 34)
+        with pp.pp_plan_create(shape, 3, dev(sens), mask=mask, power_iters=0) as plan:
+            gy = torch.empty((3,) + shape, dtype=torch.complex64, device="cuda")
+            gx = torch.empty(shape, dtype=torch.complex64, device="cuda")
+            pp.pp_forward_apply(plan, dev(x), gy)
+            pp.pp_adjoint_apply(plan, dev(y), gx)
+            assert err(gy, O.cart_forward(x, sens, mask)) <= TOL_APPLY, shape
+            assert err(gx, O.cart_adjoint(y, sens, mask)) <= TOL_APPLY, shape
+
+
+@pytest.mark.parametrize("length,n,s", GRIDS)
+def test_row_and_column_stages_at_every_grid_length(pp, length, n, s):
+    """The same for the lengths that only oversampled grids have."""
+    import torch
+    assert int(n * s) == length
+    for shape in ((n, 64), (64, n)):
+        sens = synth.coil_maps(shape, 2, 41)
+        traj = (np.random.default_rng(42).uniform(-0.499, 0.499, (301, 2)) * [shape[1], shape[0]]).astype(np.float32)
+        x, y = synth.crandn(shape, 43), synth.crandn((2, len(traj)), 44)
+        with pp.pp_plan_create(shape, 2, dev(sens), traj=traj, oversamp=s, power_iters=0) as plan:
+            gy = torch.empty((2, len(traj)), dtype=torch.complex64, device="cuda")
+            gx = torch.empty(shape, dtype=torch.complex64, device="cuda")
+            pp.pp_forward_apply(plan, dev(x), gy)
+            pp.pp_adjoint_apply(plan, dev(y), gx)
+            assert err(gy, O.nc_forward(x, sens, traj, 4, s)) <= TOL_APPLY, shape
+            assert err(gx, O.nc_adjoint(y, sens, traj, 4, s)) <= TOL_APPLY, shape
+
+
+@pytest.mark.parametrize("coils", [3, 5, 9, 27])
+@pytest.mark.parametrize("ny", [64, 128, 300, 500])
+def test_gradient_and_horner_chain_in_every_form(pp, ny, coils):
+    """A preconditioned solve (gradient and Horner recursion in one launch, the
+    gradient re-read by the streamed form) with every width, as a plan and as a batch
+    of two lengths; 3, 5 and 9 coils give the streamed form 1, 2 and 4 slots where they
+    fit.  Tolerance of the repository's solves, 1e-4."""
+    import torch
+    iters, lam, c = 4, 1e-3, [float(v) for v in O.poly_coeffs_l2(2)]
+    shapes = [(ny, 20), (96, 12)]
+    sens = [synth.coil_maps(s, coils, 51 + i) for i, s in enumerate(shapes)]
+    masks = [synth.line_mask(s, 2, 6, 53 + i) for i, s in enumerate(shapes)]
+    ys = [(synth.crandn((coils,) + s, 55 + i) * m[None]).astype(np.complex64) for i, (s, m) in enumerate(zip(shapes, masks))]
+    refs = [O.pfista(lambda v: O.cart_normal(v, s, m), lambda y: O.cart_adjoint(y, s, m), y.astype(np.complex128), lam, c,
+                     iters, 1.1) for s, m, y in zip(sens, masks, ys)]
+    with pp.pp_plan_create(shapes[0], coils, dev(sens[0]), mask=masks[0], power_iters=0) as plan:
+        pp.pp_plan_set_scale(plan, 1.1)
+        out = torch.empty(shapes[0], dtype=torch.complex64, device="cuda")
+        for w in (1, 2, 4, 8):
+            pp.pp_plan_set_tuning(plan, w, 0, 8)
+            pp.pp_fista_solve(plan, dev(ys[0]), lam, iters, c, 2, out)
+            assert err(out, refs[0]) <= 1e-4, w
+    b = pp.pp_batch_create(shapes, [coils] * 2, [dev(s) for s in sens], masks, power_iters=0)
+    try:
+        pp.pp_batch_set_scales(b, np.full(2, 1.1))
+        y = dev(np.concatenate([v.ravel() for v in ys]))
+        for tile in (-8, -16, -32):
+            pp.pp_batch_set_tile(b, tile)
+            out = torch.empty(int(b.image_off[-1]), dtype=torch.complex64, device="cuda")
+            pp.pp_batch_fista_solve(b, y, lam, iters, c, 2, out)
+            for i, s in enumerate(shapes):
+                assert err(out[b.image_off[i]:b.image_off[i + 1]].view(s), refs[i]) <= 1e-4, (tile, i)
+    finally:
+        b.destroy()
