@@ -179,8 +179,11 @@ pp_status pp_plan_sizes(const pp_plan* plan, int64_t* image_elems, int64_t* kspa
  *    into two shared buffers by tensor-map bulk copies (TMA), 3 = the same
  *    with one buffer and three blocks per SM, 4 or 5 = 0 or 1 with two z
  *    planes per y-FFT item and two line units per z item); for 2-D
- *    Cartesian plans 1, 2, 4 or 8
- *    = CTAs per 8-column group, the coils split over a cluster of that size;
+ *    Cartesian plans 1, 2, 4 or 8 = image columns per CTA: up to 4 with the
+ *    columns' intermediates in shared memory through a whole chain of
+ *    applications (4 only up to ny = 256, else the next lower width runs), 8 =
+ *    the streaming form, coils one after another; without effect where ny has no
+ *    compiled chain (see pp_batch_set_tile for the lengths);
  *  - stencil_kind: the G^T G stencil kernel (0 = one output per thread,
  *    1 = two outputs per thread, both staging one coil at a time with
  *    stencil_coils coils per CTA; 2..5 = register-blocked, a thread holding
@@ -219,9 +222,10 @@ pp_status pp_adjoint_apply(const pp_plan* plan, const pp_c64* y, pp_c64* x, pp_s
  * its own pool (an allocation behind its back can fail or upset the host's
  * accounting), or a real-time loop that forbids allocation after start-up
  * (an allocation can stall or fail on fragmented memory).  The plan is built
- * beforehand with pp_plan_create.  Runs the [coil][row][col] kernels of
- * pp_adjoint_apply (which may choose the coil-innermost ones: the results
- * then agree to rounding).  The paper has no counterpart.
+ * beforehand with pp_plan_create.  Runs the [coil][row][col] kernels, one coil
+ * of a volume at a time; pp_adjoint_apply may run the coil-innermost ones and
+ * takes several coils of a volume together, so that its sums over coils group
+ * otherwise: the results agree to rounding.  The paper has no counterpart.
  *  - Plans whose adjoint needs more than 16 MiB of scratch (Cartesian 2-D:
  *    8*C*ny*nx bytes; 3-D: 16*nz*ny*nx; non-Cartesian: 8*C*G*(ny+G))
  *    return PP_ERR_UNSUPPORTED.
@@ -301,8 +305,10 @@ pp_status pp_prox_l1_haar(pp_dims dims, int levels, float lambda, const pp_c64* 
  *   dims    2-D only; nx, ny <= 512 and multiples of 2^levels; levels 1..4
  *           (else PP_ERR_UNSUPPORTED).
  *   in/out  device [ny][nx] complex64; out may equal in.
- * Runs as 4 * levels kernels on `stream` (each level couples neighbouring
- * rows and columns, so the transform is not tile-local like the Haar). */
+ * Runs as one kernel of one thread-block cluster where the image fits its shared
+ * memory (up to about 430 x 430 at two levels, 16 CTAs), else as 4 * levels kernels (each
+ * level couples neighbouring rows and columns, so the transform is not tile-local
+ * like the Haar). */
 pp_status pp_prox_l1_db4(pp_dims dims, int levels, float lambda, const pp_c64* in, pp_c64* out,
                          pp_stream stream);
 
@@ -318,7 +324,10 @@ pp_status pp_prox_l1_db4(pp_dims dims, int levels, float lambda, const pp_c64* i
  *   shift   host int[3] (x, y, z) or NULL: the block grid starts at voxel
  *           shift (circularly), so a caller can move it between iterations.
  *   in/out  device [T][nz][ny][nx] complex64; out may equal in.
- * FP32 one-sided Jacobi SVD per block (one thread block each); else
+ * FP32, one thread block each: the singular values and vectors through the T x T
+ * Gram matrix, formed twice so that small singular values keep their accuracy;
+ * blocks near either end of the FP32 range are scaled by a power of two first, and
+ * those whose squares underflow altogether give 0.  Other sizes:
  * PP_ERR_UNSUPPORTED. */
 pp_status pp_prox_llr(pp_dims dims, int T, int block, const int* shift, float lambda,
                       const pp_c64* in, pp_c64* out, pp_stream stream);
@@ -393,9 +402,11 @@ pp_status pp_fista_solve_prox(pp_plan* plan, const pp_c64* b, const pp_c64* v, d
  * <= 5, at most 512), coils[s] coils (1..64), borrowed 16-byte aligned device maps
  * sens[s] [C_s][ny_s][nx_s] and a host line mask masks[s] [ny_s][nx_s] constant along
  * x.  Images, k-space and solutions are concatenated in slice order; the
- * offsets come from pp_batch_offsets.  Every stage of an iteration is one
- * persistent kernel launch over a work list of (slice, column tile) items,
- * and the tile width is chosen at creation by timing the candidates. */
+ * offsets come from pp_batch_offsets.  The normal operator runs over work lists
+ * of (slice, columns) items, one launch for each distinct ny, side by side (one
+ * persistent launch for all when some ny has no compiled chain); the other
+ * stages of an iteration are one launch each.  The columns per item are chosen at
+ * creation by timing the candidates. */
 typedef struct pp_batch pp_batch;
 
 /* Build a batch; power_iters > 0 estimates every L_s (one seed per slice:
@@ -412,19 +423,26 @@ pp_status pp_batch_offsets(const pp_batch* batch, int64_t* image_off, int64_t* k
 /* host double [nslices] */
 pp_status pp_batch_scales(const pp_batch* batch, double* L);
 pp_status pp_batch_set_scales(pp_batch* batch, const double* L);
-/* autotuned column tile width and persistent grid size (either may be NULL);
- * a positive width is the shared-memory Stockham kernel's columns per item;
- * -8, -16, -32 mean the register four-step FFT kernel on 8-column items
- * with 1, 2 or 4 CTAs per item (the item's coils split over a thread-block
- * cluster) */
+/* autotuned form of the normal operator and its grid size (either may be NULL);
+ * a positive number is the shared-memory Stockham kernel's columns per item;
+ * -8, -16, -32 mean the compiled column chains: -8 the streaming form on 8
+ * columns, -16 one column and -32 four columns per CTA (two where ny > 256),
+ * their intermediates in shared memory through a chain of applications.  (The
+ * numbers once stood for other kernels: one kept from such a version selects
+ * another form, with the same results up to rounding.) */
 pp_status pp_batch_tile(const pp_batch* batch, int* cols_per_cta, int* persistent_ctas);
-/* override the autotuner: 4, 8 or 16 (Stockham) or -8, -16, -32 (register
- * four-step, every slice length must be 16 * {8, 12, 16, 20, 24}) */
+/* override the autotuner: 4, 8 or 16 (Stockham) or -8, -16, -32 (the column
+ * chains: every slice's ny must be one of 32, 36, 40, 48, 60, 64, 72, 80, 96, 100,
+ * 108, 120, 128, 144, 160, 180, 192, 200, 216, 240, 256, 288, 300, 320, 324, 360,
+ * 384, 400, 432, 480, 500, 512, else PP_ERR_UNSUPPORTED) */
 pp_status pp_batch_set_tile(pp_batch* batch, int cols_per_cta);
-/* per-slice A x and A^H y (one launch sequence per slice; set-up work) */
+/* per-slice A x and A^H y: one launch for each distinct ny and nx (the adjoint in
+ * chunks of slices that fit its workspace), or slice by slice when some length has
+ * no compiled stage */
 pp_status pp_batch_forward_apply(const pp_batch* batch, const pp_c64* x, pp_c64* y, pp_stream stream);
 pp_status pp_batch_adjoint_apply(const pp_batch* batch, const pp_c64* y, pp_c64* x, pp_stream stream);
-/* y_s = (A_s^H A_s / L_s) x_s for every slice in one launch */
+/* y_s = (A_s^H A_s / L_s) x_s for every slice: one launch for each distinct ny, side
+ * by side */
 pp_status pp_batch_normal_apply(const pp_batch* batch, const pp_c64* x, pp_c64* y, pp_stream stream);
 /* Algorithm "pfista" on every slice's normalised problem, one shared lambda,
  * iteration count and polynomial; as pp_fista_solve otherwise (history sums

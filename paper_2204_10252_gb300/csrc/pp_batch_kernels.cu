@@ -7,8 +7,6 @@
 
 #include <algorithm>
 
-#include <cooperative_groups.h>
-
 #include "pp_batch.h"
 #include "pp_fft4.cuh"
 
@@ -482,8 +480,6 @@ pp_status configure_batch_kernels() {
     return PP_OK;
 }
 
-
-// Persistent grid of the uniform-length kernel (0 when n2 has none).
 pp_status launch_batch_chain(const BatchDev& b, const float2* x, const CartChain& ch, cudaStream_t st) {
     // one launch per length; each after the first may start while its
     // predecessor's last CTAs run (same input, other slices)

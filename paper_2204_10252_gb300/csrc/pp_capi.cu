@@ -1494,7 +1494,7 @@ static pp_status batch_iterations(Batch& b, float lambda, int iters, const doubl
 // fixed), Algorithm "pfista" for a fixed iteration count, checkpoints
 // (y_k, z_k) every `ce` iterations, and the reverse pass.
 // Arena layout (image-sized vectors): [0] ahb, [1 .. 2*ncp] checkpoints,
-// then 3*ce segment vectors (z_k, g_k, w_k), d+2 Horner-adjoint vectors and
+// then 2*ce segment vectors (g_k, w_k), d+2 Horner-adjoint vectors and
 // Ybar, Zbar, wbar, ahb_bar, yw, zw.
 // ---------------------------------------------------------------------------
 static pp_status ensure_arena(Batch& b, size_t vecs, size_t slots) {
@@ -1526,7 +1526,7 @@ static inline float2* avec(Batch& b, size_t i) { return b.arena + i * (size_t)b.
 
 static size_t unrolled_vecs(int iters, int ce, int d) {
     const size_t ncp = (size_t)((iters + ce - 1) / ce);
-    return 1 + 2 * ncp + 3 * (size_t)ce + (size_t)(d + 2) + 6;
+    return 1 + 2 * ncp + 2 * (size_t)ce + (size_t)(d + 2) + 6;
 }
 
 static pp_status unrolled_step(Batch& b, const double* c, int d, float lambda, int k, float2* z,
@@ -1567,7 +1567,7 @@ static pp_status unrolled_backward(Batch& b, float lambda, int iters, const doub
                                    int ce, const float2* gout, float2* grad_b, double* grad_lam,
                                    double* grad_c, cudaStream_t st) {
     const size_t ncp = (size_t)((iters + ce - 1) / ce);
-    const size_t seg0 = 1 + 2 * ncp, v0 = seg0 + 3 * (size_t)ce, r0 = v0 + (size_t)(d + 2);
+    const size_t seg0 = 1 + 2 * ncp, v0 = seg0 + 2 * (size_t)ce, r0 = v0 + (size_t)(d + 2);
     float2 *Ybar = avec(b, r0), *Zbar = avec(b, r0 + 1), *wbar = avec(b, r0 + 2),
            *ahb_bar = avec(b, r0 + 3), *yw = avec(b, r0 + 4), *zw = avec(b, r0 + 5);
     const size_t bytes = (size_t)b.nimg * sizeof(float2);
@@ -1584,13 +1584,13 @@ static pp_status unrolled_backward(Batch& b, float lambda, int iters, const doub
         PP_TRY_CUDA(cudaMemcpyAsync(zw, avec(b, 2 + 2 * sg), bytes, cudaMemcpyDeviceToDevice, st));
         for (int k = k0; k < k1; ++k) {
             const int j = k - k0;
-            PP_TRY(unrolled_step(b, c, d, lambda, k, zw, yw, avec(b, seg0 + 3 * j + 1),
-                                 avec(b, seg0 + 3 * j + 2), st));
+            PP_TRY(unrolled_step(b, c, d, lambda, k, zw, yw, avec(b, seg0 + 2 * j),
+                                 avec(b, seg0 + 2 * j + 1), st));
         }
         for (int k = k1 - 1; k >= k0; --k) {
             const int j = k - k0;
             const float beta = (float)((double)k / (k + 3.0));
-            PP_TRY(launch_batch_prox_vjp(b.dev, lambda, beta, avec(b, seg0 + 3 * j + 2), Ybar, Zbar,
+            PP_TRY(launch_batch_prox_vjp(b.dev, lambda, beta, avec(b, seg0 + 2 * j + 1), Ybar, Zbar,
                                          wbar, lam_bar, st));
             // v_0 = wbar, v_i = N_hat v_{i-1}, i = 1..d+1
             if (b.dev.cols > 0) {
@@ -1610,7 +1610,7 @@ static pp_status unrolled_backward(Batch& b, float lambda, int iters, const doub
                     prev = avec(b, v0 + i);
                 }
             }
-            const float2* gk = avec(b, seg0 + 3 * j + 1);
+            const float2* gk = avec(b, seg0 + 2 * j);
             // dots_i = Re<v_i, g_k>;  Zbar = wbar - sum_i c_i v_{i+1};  ahb_bar += sum_i c_i v_i
             RevCombine rc;
             rc.d = d;
@@ -2081,7 +2081,7 @@ pp_status pp_plan_set_tuning(pp_plan* plan, int row_ifft_variant, int stencil_ki
         return PP_ERR_UNSUPPORTED;
     }
     if (row_ifft_variant == 8 && !(p.kind == PP_CARTESIAN && p.ndim == 2)) {
-        set_error("pp_plan_set_tuning: row variant 8 (coils split over 8-CTA clusters) applies to "
+        set_error("pp_plan_set_tuning: row variant 8 (the streaming form on 8 columns) applies to "
                   "2-D Cartesian plans");
         return PP_ERR_UNSUPPORTED;
     }
@@ -2089,7 +2089,8 @@ pp_status pp_plan_set_tuning(pp_plan* plan, int row_ifft_variant, int stencil_ki
         p.tune_c3 = row_ifft_variant == 16 ? 1 : (row_ifft_variant == -16 ? 2 : 0);
     if (p.kind == PP_CARTESIAN && p.ndim == 2) {
         if (row_ifft_variant == -1 || row_ifft_variant == 16 || row_ifft_variant == -16) {
-            set_error("pp_plan_set_tuning: 2-D Cartesian plans take row variant 1, 2, 4 or 8");
+            set_error("pp_plan_set_tuning: 2-D Cartesian plans take row variant 1, 2, 4 or 8 (image "
+                      "columns per CTA)");
             return PP_ERR_UNSUPPORTED;
         }
         p.tune_c2 = row_ifft_variant;
@@ -2763,7 +2764,7 @@ pp_status pp_batch_set_tile(pp_batch* batch, int cols_per_cta) {
     if (cols_per_cta == -8 || cols_per_cta == -16 || cols_per_cta == -32) {
         for (const SliceDesc& d : b.hdesc)
             if (!cart_cols_width_ok(d.ny, 1)) {
-                set_error("pp_batch_set_tile: slice length %d has no register FFT kernel", d.ny);
+                set_error("pp_batch_set_tile: slice length %d has no compiled column chain", d.ny);
                 return PP_ERR_UNSUPPORTED;
             }
         PP_TRY(set_cols(b, cols_per_cta == -8 ? 8 : (cols_per_cta == -16 ? 1 : 4)));

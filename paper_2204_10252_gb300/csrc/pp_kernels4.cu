@@ -16,8 +16,6 @@ namespace pp {
 namespace {
 
 constexpr int N1 = 16;
-constexpr int TXF = 8;      // columns per CTA (column stage)
-constexpr int LGTXF = 3;
 constexpr int RBF = 8;      // rows / coils per CTA (row stages)
 
 

@@ -32,10 +32,12 @@ template <int N1, int N2> struct Line {
 __host__ __device__ constexpr int line_min_ctas(int threads) { return threads < 512 ? 512 / threads : 1; }
 
 // The round trip holds one transform at a time: 80 registers are enough up to
-// N2 = 16 and 102 up to 20 without spilling (32 bytes at 16 x 16), and half as many
-// threads more an SM: 148 -> 134 us at 12 x 80 x 180 x 200, whole normal operator of
-// 100 x 256 x 108 x 7 256 -> 240 us.  The inverse y stage with the same cap spills
-// 150 bytes and more (156 -> 181 us).
+// N2 = 16 and 102 up to 20 (32 bytes spilled at 16 x 16, 40 at 20 x 20), and half as
+// many threads more an SM: 148 -> 134 us at 12 x 80 x 180 x 200, whole normal operator
+// of 100 x 256 x 108 x 7 256 -> 240 us.  The inverse y stage, which holds the map's N2
+// values across the barrier as well, spills at 128 registers already (stores of 30 to
+// 260 bytes for most lengths from 80 points on, 300 to 460 for N2 = 25 and 27 and at
+// 10 x 20, 720 at 16 x 32) and took 156 -> 181 us under this cap.
 __host__ __device__ constexpr int roundtrip_min_ctas(int threads) {
     const int t = threads <= 128 ? 768 : (threads <= 160 ? 640 : 512);
     return threads < t ? t / threads : 1;

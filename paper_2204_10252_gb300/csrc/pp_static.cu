@@ -8,9 +8,10 @@
 // no-allocation rule after start-up (an allocation can stall or fail when
 // memory is fragmented).  Such callers build their plan during start-up and
 // later call pp_adjoint_apply_static instead of pp_adjoint_apply, which
-// writes its intermediates into the plan's own workspace.  Both run the same
-// kernel sequence (adjoint_ws).  The paper has no counterpart: this is an
-// interface concern.
+// writes its intermediates into the plan's own workspace.  Both are adjoint_ws,
+// here with one coil of a volume at a time; pp_adjoint_apply may also take the
+// coil-innermost arrays, which do not fit 16 MiB.  The paper has no counterpart:
+// this is an interface concern.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -62,7 +63,7 @@ void scratch_elems(const Plan& p, int64_t* wa, int64_t* wb) {
         *wb = 0;
     } else if (p.kind == PP_CARTESIAN) {
         *wa = p.nimg;
-        *wb = p.nimg;
+        *wb = p.nimg;   // not used: the limit of the calls that are taken stays where it was
     } else {
         *wa = (int64_t)p.C * p.ny * p.G_x;
         *wb = (int64_t)p.C * p.G_y * p.G_x;
