@@ -182,7 +182,9 @@ pp_status pp_plan_sizes(const pp_plan* plan, int64_t* image_elems, int64_t* kspa
  *    Cartesian plans 1, 2, 4 or 8 = image columns per CTA: up to 4 with the
  *    columns' intermediates in shared memory through a whole chain of
  *    applications (4 only up to ny = 256, else the next lower width runs), 8 =
- *    the streaming form, coils one after another; without effect where ny has no
+ *    the streaming form, coils one after another, split over a cluster of CTAs where
+ *    the columns are few; the number is the chains' (a single application is timed by
+ *    itself, and pp_plan_set_tuning sets both); without effect where ny has no
  *    compiled chain (see pp_batch_set_tile for the lengths);
  *  - stencil_kind: the G^T G stencil kernel (0 = one output per thread,
  *    1 = two outputs per thread, both staging one coil at a time with

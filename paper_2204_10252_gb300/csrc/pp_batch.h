@@ -51,6 +51,8 @@ struct CartLaunch {
     int nitems = 0;
     int W = 1;                       // columns per CTA: 1, 2, 4 (column-resident) or 8 (streaming)
     int slots = 1;                   // coils side by side in a streaming CTA
+    int split = 1;                   // CTAs of a cluster that share a streaming item's coils
+    int beside = 0;                  // items of the launches that run beside this one
     int max_coils = 1;               // largest coil count of the slices
     int resident = 1;                // maps of all coil groups in shared memory
     bool pdl = false;

@@ -491,6 +491,7 @@ pp_status launch_batch_chain(const BatchDev& b, const float2* x, const CartChain
         L.nitems = g.nitems;
         L.W = g.W;
         L.max_coils = g.max_coils;
+        L.beside = b.grid - g.nitems;
         L.pdl = L.follows = !first;
         PP_TRY(launch_cart_cols(g.n, L, x, ch, st));
         first = false;

@@ -221,7 +221,7 @@ static pp_status cart_chain(const Plan& p, const float2* x, const CartChain& ch,
     L.one.twb = p.fy.twb; L.one.sens = p.sens; L.one.mask_fo = p.mask_fo;
     L.one.ny = p.ny; L.one.nx = p.nx; L.one.C = p.C; L.one.img_off = 0; L.one.invL = 1.f;
     L.max_coils = p.C;
-    L.W = p.tune_c2;
+    L.W = ch.J > 1 ? p.tune_c2 : p.tune_c2_one;
     while (L.W > 1 && !cart_cols_width_ok(p.ny, L.W)) L.W >>= 1;
     L.pdl = p.pdl != 0;
     return launch_cart_cols(p.ny, L, x, ch, st);
@@ -740,7 +740,7 @@ struct TuneKey {
     }
 };
 struct TuneVal {
-    int rows_adj_cl, stencil_kind, stencil_cpc, c3, c3df_cg, c3df_hi, c2;
+    int rows_adj_cl, stencil_kind, stencil_cpc, c3, c3df_cg, c3df_hi, c2, c2_one;
 };
 static std::mutex g_tune_mu;
 static std::map<TuneKey, TuneVal> g_tune_cache;
@@ -766,13 +766,13 @@ static bool tune_lookup(const TuneKey& k, Plan& p) {
     const TuneVal& v = it->second;
     p.tune_rows_adj_cl = v.rows_adj_cl; p.tune_stencil_kind = v.stencil_kind;
     p.tune_stencil_cpc = v.stencil_cpc; p.tune_c3 = v.c3; p.c3df_cg = v.c3df_cg;
-    p.c3df_hi = v.c3df_hi; p.tune_c2 = v.c2;
+    p.c3df_hi = v.c3df_hi; p.tune_c2 = v.c2; p.tune_c2_one = v.c2_one;
     return true;
 }
 static void tune_store(const TuneKey& k, const Plan& p) {
     std::lock_guard<std::mutex> g(g_tune_mu);
     g_tune_cache[k] = TuneVal{p.tune_rows_adj_cl, p.tune_stencil_kind, p.tune_stencil_cpc, p.tune_c3,
-                              p.c3df_cg, p.c3df_hi, p.tune_c2};
+                              p.c3df_cg, p.c3df_hi, p.tune_c2, p.tune_c2_one};
 }
 
 // 3-D Cartesian: the three passes per coil, the one-kernel cluster operator
@@ -830,48 +830,50 @@ static pp_status tune_cart3d(Plan& p, cudaStream_t st) {
     return PP_OK;
 }
 
-// 2-D Cartesian: the columns per CTA of the column-resident kernel, timed on the
-// plan's buffers as one application and as a chain of three (a preconditioned
-// gradient of degree 2); the fastest sum is kept.  A second round re-times the
+// 2-D Cartesian: the columns per CTA of the column kernels, timed on the plan's
+// buffers for one application and for a chain of three (a preconditioned gradient of
+// degree 2); the fastest of each is kept (256 x 256 x 32: 14.7 us streaming and 17.7 on
+// two columns for one, 42 and 29 for the chain).  A second round re-times the
 // candidates within 10 % of the first one's best.
 static pp_status tune_cart2d(Plan& p, cudaStream_t st) {
     p.cols = cart_cols_width_ok(p.ny, 1);
     if (!p.cols) return PP_OK;   // the Stockham kernel
-    cudaEvent_t e0, e1;
-    PP_TRY_CUDA(cudaEventCreate(&e0));
-    PP_TRY_CUDA(cudaEventCreate(&e1));
+    cudaEvent_t ev[3];
+    for (cudaEvent_t& e : ev) PP_TRY_CUDA(cudaEventCreate(&e));
     PP_TRY_CUDA(cudaMemsetAsync(p.v, 0, sizeof(float2) * (size_t)p.nimg, st));
     std::vector<int> cand;
     for (int w : {1, 2, 4, 8})
         if (cart_cols_width_ok(p.ny, w)) cand.push_back(w);
-    std::vector<float> best(cand.size(), 1e30f);
+    std::vector<float> one(cand.size(), 1e30f), chain(cand.size(), 1e30f);
     CartChain three;
     three.out = p.t;
     three.v_first = 1;
     three.J = 3;
     for (int j = 0; j < 3; ++j) three.sc[j] = three.al[j] = 1.f;
-    auto pass = [&]() {
-        PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
-        return cart_chain(p, p.v, three, st);
-    };
     for (int round = 0; round < 2; ++round) {
-        const float cut = round == 0 ? 2e30f : 1.1f * *std::min_element(best.begin(), best.end());
+        const float one0 = *std::min_element(one.begin(), one.end()),
+                    chain0 = *std::min_element(chain.begin(), chain.end());
         for (size_t i = 0; i < cand.size(); ++i) {
-            if (best[i] > cut) continue;
-            p.tune_c2 = cand[i];
-            PP_TRY(pass());
-            PP_TRY_CUDA(cudaEventRecord(e0, st));
-            for (int r = 0; r < 4; ++r) PP_TRY(pass());
-            PP_TRY_CUDA(cudaEventRecord(e1, st));
-            PP_TRY_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            PP_TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-            best[i] = std::min(best[i], ms);
+            if (round > 0 && one[i] > 1.1f * one0 && chain[i] > 1.1f * chain0) continue;
+            p.tune_c2 = p.tune_c2_one = cand[i];
+            PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
+            PP_TRY(cart_chain(p, p.v, three, st));
+            PP_TRY_CUDA(cudaEventRecord(ev[0], st));
+            for (int r = 0; r < 4; ++r) PP_TRY(normal_into(p, p.v, p.t, 1.f, nullptr, 0.f, st));
+            PP_TRY_CUDA(cudaEventRecord(ev[1], st));
+            for (int r = 0; r < 4; ++r) PP_TRY(cart_chain(p, p.v, three, st));
+            PP_TRY_CUDA(cudaEventRecord(ev[2], st));
+            PP_TRY_CUDA(cudaEventSynchronize(ev[2]));
+            float a = 0.f, b = 0.f;
+            PP_TRY_CUDA(cudaEventElapsedTime(&a, ev[0], ev[1]));
+            PP_TRY_CUDA(cudaEventElapsedTime(&b, ev[1], ev[2]));
+            one[i] = std::min(one[i], a);
+            chain[i] = std::min(chain[i], b);
         }
     }
-    p.tune_c2 = cand[std::min_element(best.begin(), best.end()) - best.begin()];
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    p.tune_c2_one = cand[std::min_element(one.begin(), one.end()) - one.begin()];
+    p.tune_c2 = cand[std::min_element(chain.begin(), chain.end()) - chain.begin()];
+    for (cudaEvent_t e : ev) cudaEventDestroy(e);
     return PP_OK;
 }
 
@@ -2093,7 +2095,7 @@ pp_status pp_plan_set_tuning(pp_plan* plan, int row_ifft_variant, int stencil_ki
                       "columns per CTA)");
             return PP_ERR_UNSUPPORTED;
         }
-        p.tune_c2 = row_ifft_variant;
+        p.tune_c2 = p.tune_c2_one = row_ifft_variant;
         p.gkey.clear();
         return PP_OK;
     }

@@ -38,6 +38,16 @@ template <int N1, int N2> struct CartCols {
     }
 };
 
+// *p of the same shared variable in CTA `rank` of the cluster
+__device__ __forceinline__ float2 cluster_load(const float2* p, int rank) {
+    unsigned remote;
+    float2 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+                 : "=r"(remote) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(remote) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ void cpa8(void* smem, const void* gmem, bool valid) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem),
@@ -218,10 +228,14 @@ template <int Q, int TS> __device__ __forceinline__ void slot_sync(int q) {
     else asm volatile("barrier.cta.sync %0, %1;\n" ::"r"(q + 1), "n"(TS) : "memory");
 }
 
-template <int N1, int N2, int Q>
+// SPLIT: a cluster of R CTAs owns the columns and splits the coils.  After each
+// application every CTA adds the R partial sums in rank order, each slot a share of
+// the rows, so that all of them hold the same next image.  (A form of its own: the
+// exchange costs the unsplit one registers, 16 x 16 and longer spill.)
+template <int N1, int N2, int Q, bool SPLIT>
 __global__ void __launch_bounds__(8 * N2 * Q, stream_min_ctas(8 * N2 * Q))
 cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
-                   const int2* __restrict__ items, int follows, const float2* x, const CartChain ch) {
+                   const int2* __restrict__ items, int follows, int R, const float2* x, const CartChain ch) {
     using K = CartStream<N1, N2>;
     constexpr int n = K::n, P = K::P, TS = 8 * N2;
     extern __shared__ float2 sm[];
@@ -231,16 +245,19 @@ cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
     const int lane = t & 7, r = t >> 3;
     float2* Y = sm + n + n / 2 + q * K::slot;
     float2* Sb = Y + N1 * P * 8 + r * 8 + lane;
-    const int2 item = items ? items[blockIdx.x] : make_int2(0, blockIdx.x * 8);
+    const int rank = SPLIT ? blockIdx.x % R : 0, group = SPLIT ? blockIdx.x / R : blockIdx.x;
+    const int2 item = items ? items[group] : make_int2(0, group * 8);
     const SliceDesc D = items ? descs[item.x] : one;
     const int nx = D.nx, col = item.y + lane;
     const bool colok = col < nx;
     const int64_t cs = (int64_t)n * nx;
     const float2* Sg = D.sens + (int64_t)r * nx + (colok ? col : 0);
-    const int steps = (D.C + Q - 1) / Q;
+    // this CTA's coils; a CTA without any takes one step of zeros
+    const int c0 = SPLIT ? D.C * rank / R : 0, c1 = SPLIT ? D.C * (rank + 1) / R : D.C;
+    const int steps = SPLIT ? max(1, (c1 - c0 + Q - 1) / Q) : (D.C + Q - 1) / Q;
     auto stage = [&](int step, int b) {
-        const int c = step * Q + q;
-        const bool ok = c < D.C && colok;
+        const int c = c0 + step * Q + q;
+        const bool ok = c < c1 && colok;
         const float2* s = ok ? Sg + c * cs : Sg;
 #pragma unroll
         for (int m1 = 0; m1 < N1; ++m1) cpa8(Sb + (b * n + N2 * m1) * 8, s + N2 * m1 * nx, ok);
@@ -306,7 +323,49 @@ cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
             }
             // the next phase 1 writes the elements of Y that this thread just read
         }
-        if (Q > 1) {
+        if constexpr (SPLIT) {
+            float2* const Y0 = sm + n + n / 2 + r * 8 + lane;
+            __syncthreads();   // Y is free
+#pragma unroll
+            for (int m1 = 0; m1 < N1; ++m1) Y[(N2 * m1 + r) * 8 + lane] = acc[m1];
+            constexpr int RQ = (N1 + Q - 1) / Q;   // rows q, q + Q, .. belong to slot q here
+            float2* const Yr = Y0 + N2 * q * 8;
+            if constexpr (Q > 1) {
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < RQ; ++i) {
+                    if (q + Q * i >= N1) break;
+                    float2 a = Yr[N2 * Q * i * 8];
+#pragma unroll
+                    for (int p = 1; p < Q; ++p) a = cadd(a, Yr[p * K::slot + N2 * Q * i * 8]);
+                    Yr[N2 * Q * i * 8] = a;
+                }
+            }
+            cluster_arrive_release();
+            cluster_wait_acquire();
+            float2 a[RQ];
+            for (int k = 0; k < R; ++k) {
+                float2 t[RQ];
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+                    t[i] = q + Q * i < N1 ? cluster_load(Yr + N2 * Q * i * 8, k) : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < RQ; ++i) a[i] = k ? cadd(a[i], t[i]) : t[i];
+            }
+            if constexpr (Q > 1) {
+                // through slot 1, whose part is not read from outside
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+                    if (q + Q * i < N1) Yr[K::slot + N2 * Q * i * 8] = a[i];
+                __syncthreads();
+#pragma unroll
+                for (int m1 = 0; m1 < N1; ++m1) acc[m1] = Y0[K::slot + N2 * m1 * 8];
+            } else {
+#pragma unroll
+                for (int m1 = 0; m1 < N1; ++m1) acc[m1] = a[m1];
+            }
+            cluster_arrive_release();   // Y may be written again once all have waited for this
+        } else if constexpr (Q > 1) {
             // the slots' sums meet in Y, in slot order
             __syncthreads();
 #pragma unroll
@@ -331,7 +390,7 @@ cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
 #pragma unroll
             for (int m1 = 0; m1 < N1; ++m1) xr[m1] = cadd(xr[m1], cscale(op[o0 + N2 * m1 * nx], al));
         }
-        if (q == 0 && colok) {
+        if (q == 0 && rank == 0 && colok) {
             float2* out0 = j == 0 ? ch.first_out : nullptr;
             if (out0) {
 #pragma unroll
@@ -348,6 +407,7 @@ cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
                 for (int m1 = 0; m1 < N1; ++m1) out2[o0 + N2 * m1 * nx] = xr[m1];
             }
         }
+        if constexpr (SPLIT) cluster_wait_acquire();
     }
     if (follows) pdl_wait();
 }
@@ -357,19 +417,20 @@ cudaError_t cart_cols_launch(const CartLaunch& L, const float2* x, const CartCha
     using K = CartCols<N1, N2>;
     if (L.W == 8) {
         using KS = CartStream<N1, N2>;
-        const int grid = L.items ? L.nitems : (L.one.nx + 7) / 8;
+        const int grid = (L.items ? L.nitems : (L.one.nx + 7) / 8) * L.split;
         auto go = [&](auto kernel, int Q, cudaError_t allowed) {
             if (allowed != cudaSuccess) return allowed;
-            return launch_ex(kernel, dim3(grid), dim3(8 * N2 * Q), KS::smem(Q), st, L.pdl, 0, L.one,
-                             L.descs, L.items, (int)L.follows, x, ch);
+            return launch_ex(kernel, dim3(grid), dim3(8 * N2 * Q), KS::smem(Q), st, L.pdl, L.split > 1 ? L.split : 0,
+                             L.one, L.descs, L.items, (int)L.follows, L.split, x, ch);
         };
+#define PP_GO(Q, SPLIT)                                        \
+    go(cart_stream_kernel<N1, N2, Q, SPLIT>, Q, allow_smem<cart_stream_kernel<N1, N2, Q, SPLIT>, kCartSmem>())
         if constexpr (KS::smem(4) <= (size_t)kCartSmem && 32 * N2 <= 512)
-            if (L.slots == 4)
-                return go(cart_stream_kernel<N1, N2, 4>, 4, allow_smem<cart_stream_kernel<N1, N2, 4>, kCartSmem>());
+            if (L.slots == 4) return L.split > 1 ? PP_GO(4, true) : PP_GO(4, false);
         if constexpr (KS::smem(2) <= (size_t)kCartSmem)
-            if (L.slots >= 2)
-                return go(cart_stream_kernel<N1, N2, 2>, 2, allow_smem<cart_stream_kernel<N1, N2, 2>, kCartSmem>());
-        return go(cart_stream_kernel<N1, N2, 1>, 1, allow_smem<cart_stream_kernel<N1, N2, 1>, kCartSmem>());
+            if (L.slots >= 2) return L.split > 1 ? PP_GO(2, true) : PP_GO(2, false);
+        return L.split > 1 ? PP_GO(1, true) : PP_GO(1, false);
+#undef PP_GO
     }
     const int groups = (L.max_coils + 7) / 8, NB = L.resident || groups < 2 ? groups : 2;
     const size_t smem = sizeof(float2) * K::elems(L.W, NB);

@@ -232,7 +232,8 @@ struct Plan {
                                 //      with 4 / 2 columns per task
     int pdl = 1;                // programmatic dependent launch in the solve's kernel chain
     bool cols = false;          // 2-D Cartesian: the column-resident kernels run (ny has one)
-    int tune_c2 = 1;            //   columns per CTA: 1, 2, 4 (fewer where not compiled), 8 streaming
+    int tune_c2 = 1;            //   columns per CTA: 1, 2, 4 (fewer where not compiled), 8 streaming,
+    int tune_c2_one = 1;        //   of a chain and of a single application
     std::vector<void*> allocs;
 };
 

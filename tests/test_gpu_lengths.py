@@ -190,3 +190,35 @@ def test_gradient_and_horner_chain_in_every_form(pp, ny, coils):
                 assert err(out[b.image_off[i]:b.image_off[i + 1]].view(s), refs[i]) <= 1e-4, (tile, i)
     finally:
         b.destroy()
+
+
+def test_coils_split_over_more_ctas_than_a_slice_has(pp):
+    """Slices of one length with 1, 27 and 2 coils: the streamed form splits the coils of
+    all of them over four CTAs, some of which then have none."""
+    import torch
+    shapes, coils, c = [(96, 20), (96, 12), (96, 8)], [1, 27, 2], [1.5, -2.0, 1.25]
+    sens = [synth.coil_maps(s, n, 61 + i) for i, (s, n) in enumerate(zip(shapes, coils))]
+    masks = [synth.line_mask(s, 2, 6, 64 + i) for i, s in enumerate(shapes)]
+    xs = [synth.crandn(s, 67 + i) for i, s in enumerate(shapes)]
+    b = pp.pp_batch_create(shapes, coils, [dev(s) for s in sens], masks, power_iters=0)
+    try:
+        pp.pp_batch_set_tile(b, -8)
+        pp.pp_batch_set_scales(b, np.full(3, 1.25))
+        x = dev(np.concatenate([v.ravel() for v in xs]))
+        out = torch.empty_like(x)
+        for _ in range(3):
+            pp.pp_batch_normal_apply(b, x, out)
+        # the chain of the unrolled solve's reverse pass (every result kept) and of its steps
+        y = torch.empty(int(b.kspace_off[-1]), dtype=torch.complex64, device="cuda")
+        pp.pp_batch_forward_apply(b, x, y)
+        sol = torch.empty_like(x)
+        pp.pp_batch_fista_solve(b, y, 1e-3, 3, c, 2, sol)
+        for i, s in enumerate(shapes):
+            lo, hi = b.image_off[i], b.image_off[i + 1]
+            nrm = lambda v: O.cart_normal(v, sens[i], masks[i])  # noqa: E731
+            assert err(out[lo:hi].view(s), nrm(xs[i]) / 1.25) <= TOL_APPLY
+            ref = O.pfista(nrm, lambda v: O.cart_adjoint(v, sens[i], masks[i]), O.cart_forward(xs[i], sens[i], masks[i]),
+                           1e-3, c, 3, 1.25)
+            assert err(sol[lo:hi].view(s), ref) <= 1e-4
+    finally:
+        b.destroy()
