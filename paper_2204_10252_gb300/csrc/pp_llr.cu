@@ -61,18 +61,20 @@ __device__ __forceinline__ int rr_partner(int r, int i) {
 }
 
 // The T^2 floats of the Gram matrix of the block's rows, as a T x T array:
-// |a_i|^2 at (i, i), Re a_i^H a_j at (i, j) and Im a_i^H a_j at (j, i), i < j.
-// Within a warp a butterfly reduce-scatter halves the values each step (31
-// shuffles for 32 values instead of 5 for each), which leaves value l of a
-// chunk with lane l; one row a warp in `buf`.
+// |a_i|^2 at (i, i), Re a_i^H a_j at (i, j) and Im a_i^H a_j at (j, i), i < j; one row
+// a warp in `buf`.  Within a warp a butterfly reduce-scatter halves the values each
+// step (31 shuffles for 32 values instead of 5 for each), which leaves value l of a
+// chunk with lane l; the 1 or 4 values of one or two images go to the lowest lanes,
+// and the others' sums are added (5 or 6 shuffles).
 template <int T, int RPT, int NT>
 __device__ __forceinline__ void gram_partials(const float2 (&m)[RPT][T], float (*buf)[64]) {
+    constexpr int NV = T <= 2 ? T * T : 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int base = 0; base < T * T; base += 32) {
-        float t[32];
+    for (int base = 0; base < T * T; base += NV) {
+        float t[NV];
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
+        for (int e = 0; e < NV; ++e) {
             const int i = (base + e) / T, j = (base + e) % T;
             float acc = 0.f;
             if (base + e < T * T && i <= j) {
@@ -88,7 +90,7 @@ __device__ __forceinline__ void gram_partials(const float2 (&m)[RPT][T], float (
             t[e] = acc;
         }
 #pragma unroll
-        for (int h = 16; h >= 1; h >>= 1) {
+        for (int h = NV / 2; h >= 1; h >>= 1) {
             const bool up = (lane & h) != 0;
 #pragma unroll
             for (int i = 0; i < h; ++i) {
@@ -97,7 +99,9 @@ __device__ __forceinline__ void gram_partials(const float2 (&m)[RPT][T], float (
                 t[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
             }
         }
-        buf[w][base + lane] = t[0];
+#pragma unroll
+        for (int h = NV; h < 32; h <<= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], h);
+        if (lane < NV) buf[w][base + lane] = t[0];
     }
 }
 
@@ -224,6 +228,169 @@ __host__ __device__ constexpr int llr_min_ctas(int nt) { return nt > 32 ? 65536 
 __device__ __forceinline__ float llr_unit(float trace) {
     if (trace > 0.f && trace < 1e-28f) return 0x1p100f;
     return trace == __int_as_float(0x7f800000) ? 0x1p-80f : 1.f;
+}
+
+// The same for one or two images, whose T x T problem is at most one rotation: every
+// thread solves it in its own registers, so that no warp waits for the first one's and
+// a pass has one barrier, and one image takes one pass.  us, one-sided Jacobi over the
+// rows / llr_prox_kernel / here: 64 x 256 x 256 in 8^3 blocks, one image 20.2 / 35.2 / 21.1,
+// two 41.6 / 58.1 / 41.7; in 4^3 blocks 37.5 / 48.7 / 37.8 and 74.0 / 91.2 / 54.1; 1024 x 1024
+// in 4 x 4 blocks, two 37.3 / 66.2 / 39.5.  Error against 64 bits: 1.1e-7 to 1.4e-7 for
+// two images (1.1e-7 to 1.6e-7 before).  Three images so (with sweeps): 102 -> 174 us in
+// 8^3 blocks, 190 -> 238 in 4 x 4; these, alone, stay slower than with one-sided
+// Jacobi in 4 x 4 blocks (136 us), whose error was 2.8e-7 against 2.3e-7.
+template <int T> struct LlrSmall {
+    float2 A[T][T], V[T][T];   // Hermitian matrix; its eigenvectors in V's columns
+
+    __device__ __forceinline__ void set(const float (&g)[T * T], float sc) {
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int k = i; k < T; ++k) {
+                const float2 v = make_float2(g[i * T + k] * sc, i == k ? 0.f : g[k * T + i] * sc);
+                A[i][k] = v;
+                A[k][i] = make_float2(v.x, -v.y);
+            }
+        identity();
+    }
+    __device__ __forceinline__ void identity() {
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int k = 0; k < T; ++k) V[i][k] = make_float2(i == k ? 1.f : 0.f, 0.f);
+    }
+    // A <- J^H A J, V = J for the rotation that makes a 2 x 2 matrix diagonal
+    __device__ __forceinline__ void rotate(float tol) {
+        constexpr int j = T - 1;
+        float2 ai, bi, aj, bj;
+        jacobi_pair<T>(A, 0, j, tol, &ai, &bi);
+        jacobi_pair<T>(A, j, 0, tol, &aj, &bj);
+        V[0][0] = ai;
+        V[j][0] = bi;
+        V[0][j] = bj;
+        V[j][j] = aj;
+#pragma unroll
+        for (int k = 0; k < T; ++k) {
+            const float2 p = A[k][0], q = A[k][j];
+            A[k][0] = cadd(cmul(p, ai), cmul(q, bi));
+            A[k][j] = cadd(cmul(q, aj), cmul(p, bj));
+        }
+#pragma unroll
+        for (int k = 0; k < T; ++k) {
+            const float2 p = A[0][k], q = A[j][k];
+            A[0][k] = cadd(cmulc(ai, p), cmulc(bi, q));
+            A[j][k] = cadd(cmulc(aj, q), cmulc(bj, p));
+        }
+    }
+};
+
+template <int T, int RPT, int NT>
+__device__ __forceinline__ void gram_sums(const float2 (&m)[RPT][T], float (*part)[64], float (&g)[T * T]) {
+    gram_partials<T, RPT, NT>(m, part);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < T * T; ++e) {
+        g[e] = part[0][e];
+#pragma unroll
+        for (int w = 1; w < NT / 32; ++w) g[e] += part[w][e];
+    }
+}
+
+template <int T, int RPT, int NT>
+__global__ void __launch_bounds__(NT) llr_small_kernel(LlrArgs a) {
+    __shared__ float part[2][NT / 32][64];
+    float2 m[RPT][T];
+    int64_t off[RPT];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int row = threadIdx.x + q * NT;
+        off[q] = row < a.R ? llr_voxel(a, blockIdx.x, row) : -1;
+#pragma unroll
+        for (int t = 0; t < T; ++t)
+            m[q][t] = off[q] >= 0 ? a.in[t * a.nimg + off[q]] : make_float2(0.f, 0.f);
+    }
+    const float tol = sqrtf((float)a.R) * 5.9604645e-8f;
+    auto trace_of = [](const float (&g)[T * T]) {
+        float tr = g[0];
+#pragma unroll
+        for (int i = 1; i < T; ++i) tr += g[i * T + i];
+        return tr;
+    };
+    auto inverse = [](float tr) { return tr > 0.f ? 1.f / tr : (tr == 0.f ? 0.f : tr); };
+    float g[T * T];
+    gram_sums<T, RPT, NT>(m, part[0], g);
+    float tr = trace_of(g);
+    const float unit = llr_unit(tr);
+    LlrSmall<T> H;
+    float2 V0[T][T];
+    H.set(g, inverse(tr));
+    if (unit != 1.f) {   // the first pass only scales, as in llr_prox_kernel
+#pragma unroll
+        for (int q = 0; q < RPT; ++q)
+#pragma unroll
+            for (int k = 0; k < T; ++k) m[q][k] = cscale(m[q][k], unit);
+    } else if (T > 1) {
+        H.rotate(tol);
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            float2 y[T];
+#pragma unroll
+            for (int k = 0; k < T; ++k) {
+                y[k] = cmul(m[q][0], H.V[0][k]);
+#pragma unroll
+                for (int i = 1; i < T; ++i) y[k] = cadd(y[k], cmul(m[q][i], H.V[i][k]));
+            }
+#pragma unroll
+            for (int k = 0; k < T; ++k) m[q][k] = y[k];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < T; ++i)
+#pragma unroll
+        for (int k = 0; k < T; ++k) V0[i][k] = H.V[i][k];
+    if (T > 1 || unit != 1.f) {
+        gram_sums<T, RPT, NT>(m, part[1], g);
+        tr = trace_of(g);
+        H.set(g, inverse(tr));
+        if (T > 1) H.rotate(tol);
+    }
+    const float lam = a.lam * unit, back = 1.f / unit;
+    float2 Q[T][T];   // V1 F V^H with V = V0 V1
+    float f[T];
+#pragma unroll
+    for (int l = 0; l < T; ++l) {
+        // s <= lambda (also s = 0) -> 0; a NaN fails the test and stays NaN
+        const float d = H.A[l][l].x * tr;
+        const float sg = d < 0.f ? 0.f : sqrtf(d);
+        f[l] = sg <= lam ? 0.f : (1.f - lam / sg) * back;
+    }
+#pragma unroll
+    for (int k = 0; k < T; ++k) {
+        float2 v[T];
+#pragma unroll
+        for (int l = 0; l < T; ++l) {
+            v[l] = cmul(V0[k][0], H.V[0][l]);
+#pragma unroll
+            for (int i = 1; i < T; ++i) v[l] = cadd(v[l], cmul(V0[k][i], H.V[i][l]));
+        }
+#pragma unroll
+        for (int i = 0; i < T; ++i) {
+            Q[i][k] = cscale(cmulc(v[0], H.V[i][0]), f[0]);
+#pragma unroll
+            for (int l = 1; l < T; ++l) Q[i][k] = cadd(Q[i][k], cscale(cmulc(v[l], H.V[i][l]), f[l]));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        if (off[q] < 0) continue;
+#pragma unroll
+        for (int k = 0; k < T; ++k) {
+            float2 y = cmul(m[q][0], Q[0][k]);
+#pragma unroll
+            for (int i = 1; i < T; ++i) y = cadd(y, cmul(m[q][i], Q[i][k]));
+            a.out[k * a.nimg + off[q]] = y;
+        }
+    }
 }
 
 template <int T, int RPT, int NT>
@@ -372,20 +539,28 @@ __global__ void __launch_bounds__(NT, llr_min_ctas(NT)) llr_prox_kernel(LlrArgs 
 
 template <int T>
 cudaError_t llr_launch_t(const LlrArgs& a, int nblocks, cudaStream_t st) {
-    // R = 512, 256, 64 or 16 rows: few warps a block, so that few wait for the
-    // one that solves the eigenproblems; up to 20 matrix elements a thread
-    if (a.R > 256) {
-        if constexpr (T <= 5) llr_prox_kernel<T, 4, 128><<<nblocks, 128, 0, st>>>(a);
-        else llr_prox_kernel<T, 2, 256><<<nblocks, 256, 0, st>>>(a);
-    } else if (a.R > 64) {
-        if constexpr (T <= 5) llr_prox_kernel<T, 4, 64><<<nblocks, 64, 0, st>>>(a);
-        else llr_prox_kernel<T, 2, 128><<<nblocks, 128, 0, st>>>(a);
-    } else if (a.R > 32) {
-        llr_prox_kernel<T, 2, 32><<<nblocks, 32, 0, st>>>(a);
+    if constexpr (T <= 2) {
+        if (a.R > 256) llr_small_kernel<T, 4, 128><<<nblocks, 128, 0, st>>>(a);
+        else if (a.R > 64) llr_small_kernel<T, 4, 64><<<nblocks, 64, 0, st>>>(a);
+        else if (a.R > 32) llr_small_kernel<T, 2, 32><<<nblocks, 32, 0, st>>>(a);
+        else llr_small_kernel<T, 1, 32><<<nblocks, 32, 0, st>>>(a);
+        return cudaGetLastError();
     } else {
-        llr_prox_kernel<T, 1, 32><<<nblocks, 32, 0, st>>>(a);
+        // R = 512, 256, 64 or 16 rows: few warps a block, so that few wait for the
+        // one that solves the eigenproblems; up to 20 matrix elements a thread
+        if (a.R > 256) {
+            if constexpr (T <= 5) llr_prox_kernel<T, 4, 128><<<nblocks, 128, 0, st>>>(a);
+            else llr_prox_kernel<T, 2, 256><<<nblocks, 256, 0, st>>>(a);
+        } else if (a.R > 64) {
+            if constexpr (T <= 5) llr_prox_kernel<T, 4, 64><<<nblocks, 64, 0, st>>>(a);
+            else llr_prox_kernel<T, 2, 128><<<nblocks, 128, 0, st>>>(a);
+        } else if (a.R > 32) {
+            llr_prox_kernel<T, 2, 32><<<nblocks, 32, 0, st>>>(a);
+        } else {
+            llr_prox_kernel<T, 1, 32><<<nblocks, 32, 0, st>>>(a);
+        }
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
 }
 
 }  // namespace

@@ -177,3 +177,34 @@ def test_llr_prox_below_the_range_is_finite(pp, T):
         pp.pp_prox_llr((8, 8), T, 8, lam, xin, out)
         got = host(out)
         assert np.all(np.isfinite(got)) and np.all(np.abs(got) <= 2e-24)
+
+
+@pytest.mark.parametrize("shape,block", [((8, 8, 8), 8), ((16, 16), 16), ((4, 4, 4), 4), ((4, 4), 4)],
+                         ids=["512rows", "256rows", "64rows", "16rows"])
+@pytest.mark.parametrize("T", [1, 2])
+def test_llr_prox_of_one_and_two_images(pp, shape, block, T):
+    """The kernel of one and two images: the ends of the range, blocks whose columns are
+    equal, orthogonal or zero, and a NaN that stays in its block.  Bound of the graded
+    spectra."""
+    import torch
+    for mag in (1e-20, 1.0, 1e18):
+        test_llr_prox_at_the_ends_of_the_range(pp, shape, block, T, mag)
+    R = int(np.prod(shape))
+    rng = np.random.default_rng(11 * T + R)
+    u = (rng.standard_normal((T,) + shape) + 1j * rng.standard_normal((T,) + shape)).astype(np.complex64)
+    if T > 1:
+        u.reshape(T, -1)[0, R // 2:] = 0     # orthogonal columns
+        u.reshape(T, -1)[1, :R // 2] = 0
+    for v in (np.repeat(u[:1], T, 0), u, u * np.float32(1e-3) + u[:1] * (1 + 1j)):
+        for lam in (0.0, 0.4 * float(np.linalg.norm(v[0]))):
+            xin = dev(v)
+            out = torch.empty_like(xin)
+            pp.pp_prox_llr(shape, T, block, lam, xin, out)
+            assert rel(host(out), O.prox_llr(v.astype(np.complex128), lam, block)) <= 6e-6, lam
+    wide = np.concatenate([u, u], -1)        # two blocks, the first with a NaN
+    wide.reshape(T, -1)[0, 0] = np.nan
+    xin = dev(wide)
+    out = torch.empty_like(xin)
+    pp.pp_prox_llr(shape[:-1] + (2 * shape[-1],), T, block, 0.1, xin, out)
+    got = host(out)
+    assert np.all(np.isnan(got[..., :shape[-1]].real)) and np.all(np.isfinite(got[..., shape[-1]:]))
