@@ -165,8 +165,8 @@ pp_status pp_plan_sizes(const pp_plan* plan, int64_t* image_elems, int64_t* kspa
 
 /* Launch shapes the plan chose by timing at creation:
  *  - row_ifft_variant: for non-Cartesian plans the row-IFFT stage of the
- *    normal operator (1, 2 or 4 = CTAs per image row, coil groups reduced
- *    through distributed shared memory; -1 = one IFFT per coil and row
+ *    normal operator (2 or 4 = CTAs per image row, coil groups reduced
+ *    through distributed shared memory; 1 = one CTA for a row or several; -1 = one IFFT per coil and row
  *    followed by a coil sum); for 3-D Cartesian plans 16 = the whole normal
  *    operator as one kernel on 16-CTA clusters, 4 x columns per cluster task
  *    (nz = 128, ny in {128, 192, 256}), -16 = the same with 2 columns per

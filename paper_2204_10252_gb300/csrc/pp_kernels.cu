@@ -1354,8 +1354,17 @@ pp_status launch_rows_fwd(const Plan& p, const DevFft& f, const RowArgs& a, cons
 pp_status launch_rows_adj(const Plan& p, const DevFft& f, const RowArgs& a, const float2* src,
                           const float2* sens, const float* wrow, const float* wcol, float2* out,
                           const float2* operand, float alpha, int ncoils, cudaStream_t st) {
-    (void)p;
     bool done = false;
+    // The compiled stage, whose lines hold several rows or coils, against one row a CTA
+    // of rows4_adj_kernel (164 registers at 320 points: two CTAs an SM): adjoint of
+    // 320 x 320, us: 14.4 / 16.6 at 4 coils, 26.8 / 38.2 at 20, 67.8 / 180 at 64; 256 x 256
+    // 12.4 / 12.4, 20.6 / 22.7, 43.4 / 84.8; 40 coils of a 256 x 256 spiral 98 / 119.  The other
+    // way round only for padded rows of one coil group: 8 coils of that spiral 42.5 / 40.9.
+    // Cluster variants are the tuner's choice or the caller's.
+    if (p.tune_rows_adj_cl <= 1 && !(a.n < a.G && ncoils <= 8) && RB * a.n <= KMAX * kThreads) {
+        PP_TRY(launch_lines_rows_adj(f, a, src, sens, wrow, wcol, out, operand, alpha, ncoils, st, &done));
+        if (done) return PP_OK;
+    }
     PP_TRY(launch_rows4_adj(f, a, src, sens, wrow, wcol, out, operand, alpha, ncoils, st, &done,
                             p.tune_rows_adj_cl));
     if (done) return PP_OK;

@@ -222,3 +222,26 @@ def test_coils_split_over_more_ctas_than_a_slice_has(pp):
             assert err(sol[lo:hi].view(s), ref) <= 1e-4
     finally:
         b.destroy()
+
+
+@pytest.mark.parametrize("coils", [4, 12, 33])
+def test_adjoint_rows_of_the_register_lengths(pp, coils):
+    """The adjoint's row stage at 16 x {8, 12, 16, 20, 24} points and four coils or more:
+    rows as long as the image, and padded ones of a grid (one coil group and several)."""
+    import torch
+    for nx in (128, 192, 256, 320, 384):
+        sens, mask, y = synth.coil_maps((20, nx), coils, 71), synth.line_mask((20, nx), 2, 4, 72), synth.crandn((coils, 20, nx), 73)
+        with pp.pp_plan_create((20, nx), coils, dev(sens), mask=mask, power_iters=0) as plan:
+            out = torch.empty((20, nx), dtype=torch.complex64, device="cuda")
+            pp.pp_adjoint_apply(plan, dev(y), out)
+            assert err(out, O.cart_adjoint(y, sens, mask)) <= TOL_APPLY, nx
+    for nx, s in ((128, 1.5), (160, 2.0), (256, 1.25)):
+        sens = synth.coil_maps((64, nx), coils, 74)
+        traj = (np.random.default_rng(75).uniform(-0.499, 0.499, (301, 2)) * [nx, 64]).astype(np.float32)
+        y = synth.crandn((coils, len(traj)), 76)
+        with pp.pp_plan_create((64, nx), coils, dev(sens), traj=traj, oversamp=s, power_iters=0) as plan:
+            out = torch.empty((64, nx), dtype=torch.complex64, device="cuda")
+            ref = O.nc_adjoint(y, sens, traj, 4, s)
+            pp.pp_plan_set_tuning(plan, 1, 0, 8)
+            pp.pp_adjoint_apply(plan, dev(y), out)
+            assert err(out, ref) <= TOL_APPLY, nx
