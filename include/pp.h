@@ -428,9 +428,10 @@ pp_status pp_batch_set_scales(pp_batch* batch, const double* L);
 /* autotuned form of the normal operator and its grid size (either may be NULL);
  * a positive number is the shared-memory Stockham kernel's columns per item;
  * -8, -16, -32 mean the compiled column chains: -8 the streaming form on 8
- * columns, -16 one column and -32 four columns per CTA (two where ny > 256),
- * their intermediates in shared memory through a chain of applications.  (The
- * numbers once stood for other kernels: one kept from such a version selects
+ * columns, -16 one column and -32 two or four columns per CTA (pp_batch_set_tile:
+ * four, two where ny > 256), their intermediates in shared memory through a chain of
+ * applications.  The number is the chains': a single application is timed by itself,
+ * and pp_batch_set_tile sets both.  (The numbers once stood for other kernels: one kept from such a version selects
  * another form, with the same results up to rounding.) */
 pp_status pp_batch_tile(const pp_batch* batch, int* cols_per_cta, int* persistent_ctas);
 /* override the autotuner: 4, 8 or 16 (Stockham) or -8, -16, -32 (the column

@@ -55,6 +55,7 @@ struct CartLaunch {
     int beside = 0;                  // items of the launches that run beside this one
     int max_coils = 1;               // largest coil count of the slices
     int resident = 1;                // maps of all coil groups in shared memory
+    bool lean = false;               // a streaming CTA takes no more slots than raise those on an SM
     bool pdl = false;
     bool follows = false;            // runs beside the launch before it (same input)
 };
@@ -62,6 +63,7 @@ struct CartLaunch {
 // The slices of one length ny in a batch: column groups of W columns.
 struct CartGroup {
     int n = 0, W = 1, max_coils = 1, nitems = 0;
+    bool lean = false;       // see CartLaunch
     int2* items = nullptr;   // (slice, first column), most expensive first
 };
 
@@ -82,9 +84,10 @@ struct BatchDev {
     SliceDesc* descs = nullptr;
     int2* items = nullptr;   // (slice, first column), most expensive first
     int nitems = 0, ny_max = 0, km = 0, lgt = 3, grid = 0;
-    int cols = 0;            // > 0: the column-resident kernels run, one launch per length,
-                             //   `cols` columns per CTA (fewer where a length has no such form)
-    std::vector<CartGroup> groups;
+    int cols = 0;            // > 0: the column-resident kernels run, one launch per length, a
+                             //   chain on `cols` columns per CTA (fewer where a length has no such
+                             //   form)
+    std::vector<CartGroup> groups, one;   // of chains, of a single application (or the same lists)
     Segments img, ksp, tiles;
 };
 

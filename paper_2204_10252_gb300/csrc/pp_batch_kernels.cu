@@ -484,14 +484,18 @@ pp_status launch_batch_chain(const BatchDev& b, const float2* x, const CartChain
     // one launch per length; each after the first may start while its
     // predecessor's last CTAs run (same input, other slices)
     bool first = true;
-    for (const CartGroup& g : b.groups) {
+    const std::vector<CartGroup>& groups = ch.J > 1 ? b.groups : b.one;
+    int all = 0;
+    for (const CartGroup& g : groups) all += g.nitems;
+    for (const CartGroup& g : groups) {
         CartLaunch L;
         L.descs = b.descs;
         L.items = g.items;
         L.nitems = g.nitems;
         L.W = g.W;
         L.max_coils = g.max_coils;
-        L.beside = b.grid - g.nitems;
+        L.lean = g.lean;
+        L.beside = all - g.nitems;
         L.pdl = L.follows = !first;
         PP_TRY(launch_cart_cols(g.n, L, x, ch, st));
         first = false;

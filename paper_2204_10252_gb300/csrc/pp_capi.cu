@@ -1298,7 +1298,7 @@ static void free_groups(Batch& b, std::vector<CartGroup>& groups) {
     }
     groups.clear();
 }
-static pp_status make_groups(Batch& b, int W, std::vector<CartGroup>* out) {
+static pp_status make_groups(Batch& b, int W, bool lean, std::vector<CartGroup>* out) {
     std::map<int, std::vector<std::pair<int, int2>>, std::greater<int>> by_len;
     std::map<int, CartGroup> info;
     for (int s = 0; s < b.n; ++s) {
@@ -1306,6 +1306,7 @@ static pp_status make_groups(Batch& b, int W, std::vector<CartGroup>* out) {
         CartGroup& g = info[d.ny];
         g.n = d.ny;
         g.W = W;
+        g.lean = lean;
         while (g.W > 1 && !cart_cols_width_ok(d.ny, g.W)) g.W >>= 1;
         g.max_coils = std::max(g.max_coils, d.C);
         for (int c0 = 0; c0 < d.nx; c0 += g.W) by_len[d.ny].push_back({d.C, make_int2(s, c0)});
@@ -1331,33 +1332,41 @@ static pp_status make_groups(Batch& b, int W, std::vector<CartGroup>* out) {
     *out = groups;
     return PP_OK;
 }
-static void use_groups(Batch& b, int W, const std::vector<CartGroup>& groups) {
+// `one` may be the same lists as `groups`.
+static void use_groups(Batch& b, int W, const std::vector<CartGroup>& groups, const std::vector<CartGroup>& one) {
     b.dev.groups = groups;
+    b.dev.one = one;
     b.dev.cols = groups.empty() ? 0 : W;
     b.dev.grid = 0;
     for (const CartGroup& g : groups) b.dev.grid += g.nitems;
 }
 static void drop_groups(Batch& b) {
+    if (!b.dev.one.empty() && b.dev.one[0].items != b.dev.groups[0].items) free_groups(b, b.dev.one);
     free_groups(b, b.dev.groups);
+    b.dev.one.clear();
     b.dev.cols = 0;
 }
 static pp_status set_cols(Batch& b, int W) {
     std::vector<CartGroup> groups;
-    PP_TRY(make_groups(b, W, &groups));
+    PP_TRY(make_groups(b, W, false, &groups));
     drop_groups(b);
-    use_groups(b, W, groups);
+    use_groups(b, W, groups, groups);
     return PP_OK;
 }
 
-// Batch autotuner: the columns per CTA of the column-resident kernels (one
-// application and a chain of three, as for a single plan) where every slice
-// length has one, else the tile width of the Stockham kernel.  One pass each, then
-// about 0.4 ms of passes for those within 20 % of the best.
+// Batch autotuner: the columns per CTA of the column-resident kernels where every
+// slice length has one, for an application and for a chain of three (the fastest of
+// each: one 256 x 256 x 16 slice takes 12.4 us on two columns and 16.5 on one, a solve
+// of d = 5 40.9 and 44.2 an iteration), else the tile width of the Stockham kernel.
+// The streaming form is tried with both counts of slots: us for as many as bring 16
+// warps to an SM / for no more than raise those on an SM (CartLaunch::lean), eight
+// slices of 384 x 384 x 8 53.3 / 45.2, of 256 x 256 x 16 43.9 / 40.9, 32 of 128 x 128 x 16
+// 39.1 / 32.9, but six of 320 x 320 x 20 59.8 / 80.2.  One pass each, then about 0.4 ms of
+// passes for those within 20 % of the best.
 static pp_status autotune(Batch& b, cudaStream_t st) {
     std::vector<int2> items;
-    cudaEvent_t e0, e1;
-    PP_TRY_CUDA(cudaEventCreate(&e0));
-    PP_TRY_CUDA(cudaEventCreate(&e1));
+    cudaEvent_t ev[3];
+    for (cudaEvent_t& e : ev) PP_TRY_CUDA(cudaEventCreate(&e));
     const bool cols = cols_supported(b);
     CartChain three;
     three.out = b.t;
@@ -1365,44 +1374,57 @@ static pp_status autotune(Batch& b, cudaStream_t st) {
     three.J = 3;
     for (int j = 0; j < 3; ++j) three.sc[j] = three.al[j] = 1.f;
     std::vector<int> cand;
-    for (int v : cols ? std::vector<int>{1, 4, 8} : std::vector<int>{2, 3, 4})
-        if (cols || km_for(b.dev.ny_max, v)) cand.push_back(v);
+    if (cols) {
+        // two columns only for batches that leave SMs idle on wider ones
+        int64_t wide = 0;
+        for (const SliceDesc& d : b.hdesc) wide += (d.nx + 7) / 8;
+        cand = wide <= 2 * 152 ? std::vector<int>{1, 2, 4, 8, 8} : std::vector<int>{1, 4, 8, 8};
+    } else {
+        for (int v : {2, 3, 4})
+            if (km_for(b.dev.ny_max, v)) cand.push_back(v);
+    }
     if (cand.empty()) {
         set_error("no batched kernel fits ny_max = %d", b.dev.ny_max);
         return PP_ERR_UNSUPPORTED;
     }
     std::vector<std::vector<CartGroup>> lists(cand.size());
     if (cols)
-        for (size_t i = 0; i < cand.size(); ++i) PP_TRY(make_groups(b, cand[i], &lists[i]));
-    auto pass = [&]() {
-        PP_TRY(launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st));
-        return cols ? launch_batch_chain(b.dev, b.v, three, st) : PP_OK;
-    };
-    std::vector<float> best(cand.size(), 1e30f);
+        for (size_t i = 0; i < cand.size(); ++i)
+            PP_TRY(make_groups(b, cand[i], i + 1 == cand.size(), &lists[i]));
+    auto single = [&]() { return launch_batch_normal(b.dev, b.v, b.t, 1.f, nullptr, 0.f, st); };
+    auto chain = [&]() { return cols ? launch_batch_chain(b.dev, b.v, three, st) : PP_OK; };
+    std::vector<float> one(cand.size(), 1e30f), chn(cand.size(), 1e30f);
     for (int round = 0; round < 2; ++round) {
-        const float lead = *std::min_element(best.begin(), best.end());
-        const int reps = round == 0 ? 1 : std::max(1, std::min(8, (int)(0.4f / lead)));
+        const float one0 = *std::min_element(one.begin(), one.end()), chn0 = *std::min_element(chn.begin(), chn.end());
+        const int reps = round == 0 ? 1 : std::max(2, std::min(8, (int)(0.4f / (one0 + chn0))));
         for (size_t i = 0; i < cand.size(); ++i) {
-            if (round > 0 && best[i] > 1.2f * lead) continue;
-            if (cols) use_groups(b, cand[i], lists[i]);
+            if (round > 0 && one[i] > 1.2f * one0 && (!cols || chn[i] > 1.2f * chn0)) continue;
+            if (cols) use_groups(b, cand[i], lists[i], lists[i]);
             else PP_TRY(set_items(b, cand[i], &items));
-            if (round == 0) PP_TRY(pass());
-            PP_TRY_CUDA(cudaEventRecord(e0, st));
-            for (int r = 0; r < reps; ++r) PP_TRY(pass());
-            PP_TRY_CUDA(cudaEventRecord(e1, st));
-            PP_TRY_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            PP_TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-            best[i] = std::min(best[i], ms / reps);
+            if (round == 0) {
+                PP_TRY(single());
+                PP_TRY(chain());
+            }
+            PP_TRY_CUDA(cudaEventRecord(ev[0], st));
+            for (int r = 0; r < reps; ++r) PP_TRY(single());
+            PP_TRY_CUDA(cudaEventRecord(ev[1], st));
+            for (int r = 0; r < reps; ++r) PP_TRY(chain());
+            PP_TRY_CUDA(cudaEventRecord(ev[2], st));
+            PP_TRY_CUDA(cudaEventSynchronize(ev[2]));
+            float t1 = 0.f, t3 = 0.f;
+            PP_TRY_CUDA(cudaEventElapsedTime(&t1, ev[0], ev[1]));
+            PP_TRY_CUDA(cudaEventElapsedTime(&t3, ev[1], ev[2]));
+            one[i] = t1 / reps;
+            chn[i] = t3 / reps;
         }
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    const size_t win = std::min_element(best.begin(), best.end()) - best.begin();
-    if (!cols) return set_items(b, cand[win], &items);
-    use_groups(b, cand[win], lists[win]);
+    for (cudaEvent_t& e : ev) cudaEventDestroy(e);
+    const size_t w1 = std::min_element(one.begin(), one.end()) - one.begin(),
+                 w3 = std::min_element(chn.begin(), chn.end()) - chn.begin();
+    if (!cols) return set_items(b, cand[w1], &items);
+    use_groups(b, cand[w3], lists[w3], lists[w1]);
     for (size_t i = 0; i < cand.size(); ++i)
-        if (i != win) free_groups(b, lists[i]);
+        if (i != w1 && i != w3) free_groups(b, lists[i]);
     return PP_OK;
 }
 

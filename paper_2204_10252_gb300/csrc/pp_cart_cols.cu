@@ -53,9 +53,14 @@ pp_status launch_cart_cols(int n, CartLaunch L, const float2* x, const CartChain
     // two coils are left to each, or one where the coils are split.
     if (l && L.W == 8) {
         const int items = L.items ? L.nitems : (L.one.nx + 7) / 8;
-        while (L.split < 4 && 2 * (items + L.beside) * L.split <= 152 && L.max_coils >= 4 * L.split) L.split *= 2;
+        while (L.split < 4 && 2 * items * L.split + L.beside <= 152 && L.max_coils >= 4 * L.split) L.split *= 2;
         const int ctas = items * L.split, coils = L.max_coils / L.split, left = L.split > 1 ? 2 : 4;
-        while (L.slots < 4 && ctas * L.slots * 8 * l->n2 < 152 * 512 && coils >= left * L.slots) L.slots *= 2;
+        auto in_flight = [&](int slots) {   // slots on the fullest SM
+            return std::min((ctas + 151) / 152, std::max(1, 512 / (8 * l->n2 * slots))) * slots;
+        };
+        while (L.slots < 4 && ctas * L.slots * 8 * l->n2 < 152 * 512 && coils >= left * L.slots &&
+               (!L.lean || in_flight(2 * L.slots) > in_flight(L.slots)))
+            L.slots *= 2;
     }
     cudaError_t e = l ? l->launch(L, x, ch, st) : cudaErrorInvalidValue;
     if (e != cudaSuccess) return cuda_status(e, "cart_cols_kernel launch");

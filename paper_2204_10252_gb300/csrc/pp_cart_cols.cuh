@@ -228,12 +228,14 @@ template <int Q, int TS> __device__ __forceinline__ void slot_sync(int q) {
     else asm volatile("barrier.cta.sync %0, %1;\n" ::"r"(q + 1), "n"(TS) : "memory");
 }
 
-// SPLIT: a cluster of R CTAs owns the columns and splits the coils.  After each
-// application every CTA adds the R partial sums in rank order, each slot a share of
-// the rows, so that all of them hold the same next image.  (A form of its own: the
-// exchange costs the unsplit one registers, 16 x 16 and longer spill.)
+// SPLIT: a cluster of R CTAs (2 or 4) owns the columns and splits the coils.  After
+// each application every CTA adds the R partial sums in rank order, each slot a share of
+// the rows, so that all of them hold the same next image; after the last one each rank
+// adds its own share.  (A form of its own: the
+// exchange costs the unsplit one registers, 16 x 16 and longer spill.  It runs at one
+// CTA an SM, so small CTAs may take more of them.)
 template <int N1, int N2, int Q, bool SPLIT>
-__global__ void __launch_bounds__(8 * N2 * Q, stream_min_ctas(8 * N2 * Q))
+__global__ void __launch_bounds__(8 * N2 * Q, SPLIT ? 1 : stream_min_ctas(8 * N2 * Q))
 cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
                    const int2* __restrict__ items, int follows, int R, const float2* x, const CartChain ch) {
     using K = CartStream<N1, N2>;
@@ -343,6 +345,30 @@ cart_stream_kernel(const SliceDesc one, const SliceDesc* __restrict__ descs,
             }
             cluster_arrive_release();
             cluster_wait_acquire();
+            if (j == ch.J - 1) {
+                // nothing follows: each rank adds and writes a share of the rows
+                const float sc = ch.sc[j] * D.invL, al = ch.al[j];
+                const float2* op = j == 0 && !ch.v_first ? ch.ext : (al != 0.f ? v : nullptr);
+                float2* out0 = j == 0 ? ch.first_out : nullptr;
+                float2* out1 = ch.all_out ? ch.all_out + j * ch.all_stride : nullptr;
+                for (int i = rank; i < RQ && q + Q * i < N1; i += R) {
+                    float2 t[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) t[k] = k < R ? cluster_load(Yr + N2 * Q * i * 8, k) : make_float2(0.f, 0.f);
+                    float2 s = cadd(t[0], t[1]);
+                    if (R > 2) s = cadd(cadd(s, t[2]), t[3]);
+                    if (!colok) continue;
+                    const int64_t o = o0 + N2 * (q + Q * i) * nx;
+                    s = cscale(s, sc);
+                    if (op) s = cadd(s, cscale(op[o], al));
+                    if (out0) out0[o] = s;
+                    if (out1) out1[o] = s;
+                    if (ch.out) ch.out[o] = s;
+                }
+                cluster_arrive_release();
+                cluster_wait_acquire();
+                break;
+            }
             float2 a[RQ];
             for (int k = 0; k < R; ++k) {
                 float2 t[RQ];

@@ -245,3 +245,59 @@ def test_adjoint_rows_of_the_register_lengths(pp, coils):
             pp.pp_plan_set_tuning(plan, 1, 0, 8)
             pp.pp_adjoint_apply(plan, dev(y), out)
             assert err(out, ref) <= TOL_APPLY, nx
+
+
+def test_batch_forms_of_applications_and_chains(pp):
+    """A batch keeps one form for a single application and one for chains; whichever the
+    timing takes, both agree with the oracle, also after another form was forced."""
+    import torch
+    for shapes, coils in (([(256, 24)], [9]), ([(128, 40)] * 3, [5, 17, 3]), ([(512, 12), (64, 60)], [6, 20])):
+        sens = [synth.coil_maps(s, n, 81 + i) for i, (s, n) in enumerate(zip(shapes, coils))]
+        masks = [synth.line_mask(s, 2, 6, 84 + i) for i, s in enumerate(shapes)]
+        xs = [synth.crandn(s, 87 + i) for i, s in enumerate(shapes)]
+        ys = [O.cart_forward(v, s, m).astype(np.complex64) for v, s, m in zip(xs, sens, masks)]
+        c = [1.5, -2.0, 1.25]
+        refs = [O.pfista(lambda v: O.cart_normal(v, s, m), lambda k: O.cart_adjoint(k, s, m),
+                         y.astype(np.complex128), 1e-3, c, 3, 1.25)
+                for s, m, y in zip(sens, masks, ys)]
+        b = pp.pp_batch_create(shapes, coils, [dev(s) for s in sens], masks, power_iters=0)
+        try:
+            pp.pp_batch_set_scales(b, np.full(b.n, 1.25))
+            x, y = (dev(np.concatenate([v.ravel() for v in vs])) for vs in (xs, ys))
+            for tile in (None, -16, -32, -8):
+                if tile:
+                    pp.pp_batch_set_tile(b, tile)
+                out, sol = torch.empty_like(x), torch.empty_like(x)
+                pp.pp_batch_normal_apply(b, x, out)
+                pp.pp_batch_fista_solve(b, y, 1e-3, 3, c, 2, sol)
+                for i, s in enumerate(shapes):
+                    lo, hi = b.image_off[i], b.image_off[i + 1]
+                    assert err(out[lo:hi].view(s), O.cart_normal(xs[i], sens[i], masks[i]) / 1.25) <= TOL_APPLY, (tile, i)
+                    assert err(sol[lo:hi].view(s), refs[i]) <= 1e-4, (tile, i)
+        finally:
+            b.destroy()
+
+
+@pytest.mark.parametrize("ny", [36, 60, 100, 180, 256, 480])
+def test_split_coils_of_one_application(pp, ny):
+    """One application whose coils are split over two and four CTAs: every rank adds and
+    writes its share of the rows, with and without an operand (a polynomial of degree 0
+    and 1 in the streamed form)."""
+    import torch
+    for coils in (6, 16, 40):
+        shape = (ny, 20)
+        sens, mask, x = synth.coil_maps(shape, coils, 91), synth.line_mask(shape, 2, 4, 92), synth.crandn(shape, 93)
+        with pp.pp_plan_create(shape, coils, dev(sens), mask=mask, power_iters=0) as plan:
+            pp.pp_plan_set_scale(plan, 1.25)
+            pp.pp_plan_set_tuning(plan, 8, 0, 8)
+            ref = O.cart_normal(x, sens, mask) / 1.25
+            out = torch.empty(shape, dtype=torch.complex64, device="cuda")
+            pp.pp_normal_apply(plan, dev(x), out)
+            assert err(out, ref) <= TOL_APPLY, coils
+            pp.pp_poly_apply(plan, [0.5, -2.0], 1, dev(x), out)
+            assert err(out, 0.5 * x.astype(np.complex128) - 2.0 * ref) <= TOL_APPLY, coils
+            y = (synth.crandn((coils,) + shape, 94) * mask[None]).astype(np.complex64)
+            pp.pp_fista_solve(plan, dev(y), 1e-3, 4, None, 0, out)
+            sol = O.pfista(lambda v: O.cart_normal(v, sens, mask), lambda k: O.cart_adjoint(k, sens, mask),
+                           y.astype(np.complex128), 1e-3, None, 4, 1.25)
+            assert err(out, sol) <= 1e-4, coils
