@@ -119,7 +119,7 @@ typedef struct pp_plan pp_plan;
  * Set-up times the plan's candidate launch shapes on its own buffers and
  * keeps the fastest (see pp_plan_tuning); the choice is remembered for the
  * life of the process per device, shape, coil count and sampling (the
- * trajectory's or the mask's bytes), so a later plan of the same geometry
+ * trajectory's bytes; any mask), so a later plan of the same geometry
  * takes it without timing again.  Non-Cartesian set-up computes the
  * per-sample gridding taps and tile lists on up to 16 host threads.
  * Device memory beside `sens`: 8 images, and

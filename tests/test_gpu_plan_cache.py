@@ -94,3 +94,22 @@ def test_second_3d_plan_reuses_the_tuning(pp):
     finally:
         for p in plans:
             p.destroy()
+
+
+@pytest.mark.parametrize("shape", [(96, 40), (16, 32, 24)])
+def test_a_plan_with_another_mask_reuses_the_tuning(pp, shape):
+    import torch
+    sens, x = synth.coil_maps(shape, 5, 721), synth.crandn(shape, 722)
+    masks = [synth.line_mask(shape, R, 4, 723 + R) for R in (2, 4)]
+    assert not np.array_equal(*masks)
+    plans = [pp.pp_plan_create(shape, 5, dev(sens), mask=m, power_iters=0) for m in masks]
+    try:
+        assert pp.pp_plan_tuning(plans[0]) == pp.pp_plan_tuning(plans[1])
+        for plan, m in zip(plans, masks):
+            out = torch.empty(shape, dtype=torch.complex64, device="cuda")
+            pp.pp_plan_set_scale(plan, 1.0)
+            pp.pp_normal_apply(plan, dev(x), out)
+            assert rel(host(out), O.cart_normal(x, sens, m)) <= 1e-5
+    finally:
+        for plan in plans:
+            plan.destroy()
