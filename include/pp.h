@@ -121,7 +121,8 @@ typedef struct pp_plan pp_plan;
  * life of the process per device, shape, coil count and sampling (the
  * trajectory's bytes; any mask), so a later plan of the same geometry
  * takes it without timing again.  Non-Cartesian set-up computes the
- * per-sample gridding taps and tile lists on up to 16 host threads.
+ * per-sample gridding taps on up to 16 host threads and sorts the samples by
+ * grid cell on one.
  * Device memory beside `sens`: 8 images, and
  *   2-D Cartesian    the k-space, 8*C*ny*nx bytes;
  *   3-D              the planes of as many coils as fit 512 MB (one at least), fewer

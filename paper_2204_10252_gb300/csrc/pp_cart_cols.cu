@@ -46,11 +46,13 @@ pp_status launch_cart_cols(int n, CartLaunch L, const float2* x, const CartChain
     L.resident = groups <= 2 || (ch.J > 1 && l && per_sm * (smem_of(*l, L.W, groups) + 1024) <= (size_t)kCartSmem);
     // Streaming: the coils of an item over a cluster of up to four CTAs, while those of
     // all launches side by side still get an SM each and two coils are left to each
-    // (256 x 256, us for 1 / 2 / 4 / 8 CTAs: 18.4 / 12.7 / 10.7 / 38.6 at 16 coils, 63 / 36 /
-    // 22.4 / 52 at 64; more CTAs than SMs, 320 x 320 x 12: 17.9 / 11.9 / 21.9; eight
-    // CTAs also where they fit, 128 x 128 x 32: 18.1 / 11.6 / 8.0 / 15.0).  Then as many
-    // slots as bring 16 warps to every SM (what 128 registers a thread allow), while
-    // two coils are left to each, or one where the coils are split.
+    // (256 x 256, us for 1 / 2 / 4 / 8 CTAs, when one rank still added up the last sum:
+    // 18.4 / 12.7 / 10.7 / 38.6 at 16 coils, 63 / 36 / 22.4 / 52 at 64; more CTAs than SMs,
+    // 320 x 320 x 12: 17.9 / 11.9 / 21.9; eight CTAs also where they fit, 128 x 128 x 32:
+    // 18.1 / 11.6 / 8.0 / 15.0).  Then as many slots as bring 16 warps to every SM (what
+    // 128 registers a thread allow), while two coils are left to each, or one where the
+    // coils are split.  A lean launch stops where more slots only take the place of
+    // CTAs (see the batch's timing).
     if (l && L.W == 8) {
         const int items = L.items ? L.nitems : (L.one.nx + 7) / 8;
         while (L.split < 4 && 2 * items * L.split + L.beside <= 152 && L.max_coils >= 4 * L.split) L.split *= 2;
